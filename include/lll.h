@@ -235,6 +235,21 @@ int lll_simulate_noalloc(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t
  *   nodes, weights: [Q] outputs, Q in [1, 128]. */
 int lll_build_nig_quadrature(lll_nig nig, double xmax, int Q, double *nodes, double *weights);
 
+/* lll_sweep_rule -- the rule that the full and Picard sweeps use in place of
+ * (nodes, weights), the arguments of lll_init: the shortest Gauss rule of the
+ * discrete measure sum_j weights[j] delta_nodes[j] (at most 32 nodes) whose
+ * moment generating function agrees with the given rule's to 2^-28 relative
+ * on [lo, hi].  With lo (hi) the most negative (positive) sum of the live
+ * volatilities over the steps, every compensator of Eq. (LIBOR-drift-PT) then
+ * agrees to 2^-28 of its terms, whatever the rates.  lo <= 0 <= hi.
+ *   count : nodes of the shorter rule; 0 where the given rule is swept (a
+ *           weight <= 0, or no shorter rule agrees);
+ *   padded: nodes the kernels process (the given rule padded where count = 0);
+ *   x, w  : [32] outputs, the first `count` used.
+ * Host computation. */
+int lll_sweep_rule(int Q, const double *nodes, const double *weights, double lo, double hi, int *count,
+                   int *padded, double *x, double *w);
+
 /* ---- Batches of independent term structures -------------------------------
  * Many models (uneven tenor counts, curves, volatilities, NIG parameters,
  * strike grids and path budgets) simulated by one persistent launch: the

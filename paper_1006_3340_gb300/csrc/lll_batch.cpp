@@ -46,7 +46,7 @@ struct Sched {
     int *d_item_inst = nullptr, *d_next = nullptr, *d_inst_seg_ptr = nullptr, *d_inst_segs = nullptr;
     uint2 *d_item_tiles = nullptr;
     size_t *d_seg_off = nullptr;
-    double *d_partials = nullptr;
+    double *d_partials = nullptr, *d_comps = nullptr;
     float *d_state = nullptr;
     int grid = 0, n_items = 0, CH = 0, R = 1, threads = 128;
     size_t smem = 0;
@@ -60,7 +60,8 @@ struct lll_batch {
     std::vector<lll_ctx *> inst;
     std::vector<uint64_t> paths;
     cudaStream_t stream = nullptr;
-    int sm_count = 0, QP = 0, n_max = 0, ns_max = 0;
+    int sm_count = 0, QP = 0, n_max = 0, ns_max = 0; // QP: padded nodes of the rules as given
+    int QK = 0; // > 0: the time-blocked kernel, each instance at its own rule's length up to QK = 8 or 32
     Shape shape[2]; // by scheme: LLL_FULL, LLL_PICARD
     Sched sched[2];
     PathArgs *d_desc = nullptr;
@@ -88,7 +89,7 @@ int berr(lll_batch *b, int code, const std::string &m)
 void free_sched(Sched &c)
 {
     cudaFree(c.d_item_inst); cudaFree(c.d_next); cudaFree(c.d_inst_seg_ptr); cudaFree(c.d_inst_segs);
-    cudaFree(c.d_item_tiles); cudaFree(c.d_seg_off); cudaFree(c.d_partials); cudaFree(c.d_state);
+    cudaFree(c.d_item_tiles); cudaFree(c.d_seg_off); cudaFree(c.d_partials); cudaFree(c.d_comps); cudaFree(c.d_state);
     if (c.graph) cudaGraphExecDestroy(c.graph);
     c = Sched();
 }
@@ -144,27 +145,37 @@ int build_schedule(lll_batch *b, int scheme)
     free_sched(c);
     const Shape &sh = b->shape[scheme];
     const int T = sh.threads, R = sh.R;
-    if (!batch_kernel_supported(scheme, b->QP, R))
+    if (R == 2 && b->QP > 64) // compiled for rules of up to 64 nodes as given
         return berr(b, LLL_EUNSUPPORTED, "no batch kernel for this Q and paths per thread");
-    const int CH = sh.chunk_rows > 0 ? std::min(sh.chunk_rows, b->n_max)
-                                     : std::min(b->n_max, std::max(1, (48 * 1024) / (2 * (b->QP / 4) * 16)));
+    int CH = sh.chunk_rows > 0 ? std::min(sh.chunk_rows, b->n_max)
+                               : std::min(b->n_max, std::max(1, (48 * 1024) / (2 * (b->QP / 4) * 16)));
     const int nst = scheme == LLL_PICARD ? 2 : 1;
     // smem as for the path kernel, sized for the largest instance
     size_t smem = path_kernel_smem(b->QP, b->n_max, b->ns_max, T, CH);
     if (smem > 227 * 1024) return berr(b, LLL_EUNSUPPORTED, "batch shared memory exceeds 227 KB");
+    if (b->QK > 0) { // the longest of the instances' rules decides
+        CH = b->n_max;
+        for (const lll_ctx *ic : b->inst) CH = std::min(CH, block_chunk_rates(ic->QR, R, b->n_max, sh.chunk_rows));
+        smem = 0;
+        for (const lll_ctx *ic : b->inst)
+            smem = std::max(smem, block_kernel_smem(ic->QR, R, b->n_max, b->ns_max, T, CH));
+    }
     int occ = 0;
-    cudaError_t e = (cudaError_t)batch_kernel_prepare(scheme, b->QP, R, smem, T, &occ);
+    cudaError_t e = (cudaError_t)(b->QK > 0 ? batch_block_prepare(scheme, b->QK, R, smem, T, &occ)
+                                            : batch_kernel_prepare(scheme, b->QP, R, smem, T, &occ));
     if (e != cudaSuccess) return berr(b, LLL_ECUDA, std::string("batch kernel attributes: ") + cudaGetErrorString(e));
     if (occ < 1) return berr(b, LLL_EUNSUPPORTED, "batch kernel does not fit on an SM");
     const int bps = sh.blocks_per_sm > 0 ? std::min(sh.blocks_per_sm, occ) : occ;
     // Work items: runs of consecutive tiles (T R paths each) of one instance,
     // each of at most 1/16 of a block's share of the total cost (one tile at
     // least).  A tile costs the same whether or not it is full (its idle lanes
-    // run along): s n (n+1)/2 path-rate-steps per path, plus kStepCost of them
+    // run along): s n (n+1)/2 path-rate-steps per path, plus `step` of them
     // for each of the s n steps, for what a step does once whatever the number
     // of live rates (the increment, chunk staging and synchronisation, the
-    // maturity payoffs).
-    constexpr double kStepCost = 3.0;
+    // maturity payoffs).  The time-blocked kernel: in FP32 instructions, about
+    // 8 + 3 nodes a path-rate-step and 300 a step.
+    auto unit_cost = [&](const lll_ctx *ic) { return b->QK > 0 ? 8.0 + 3.0 * ic->QR : 1.0; };
+    const double step_cost = b->QK > 0 ? 300.0 : 3.0;
     const int ni = (int)b->inst.size();
     const uint64_t TP = (uint64_t)T * R;
     std::vector<double> tile_cost(ni);
@@ -175,7 +186,7 @@ int build_schedule(lll_batch *b, int scheme)
         const lll_ctx *ic = b->inst[q];
         ntile[q] = (b->paths[q] + TP - 1) / TP;
         if (ntile[q] > 0xffffffffull) return berr(b, LLL_EINVAL, "instance has more than 2^32 tiles");
-        tile_cost[q] = (double)TP * ic->s * ic->n * ((ic->n + 1) / 2.0 + kStepCost);
+        tile_cost[q] = (double)TP * ic->s * ic->n * ((ic->n + 1) / 2.0 * unit_cost(ic) + step_cost);
         total += tile_cost[q] * (double)ntile[q];
         ntiles += ntile[q];
     }
@@ -226,6 +237,7 @@ int build_schedule(lll_batch *b, int scheme)
               upload(&c.d_inst_segs, inst_segs, st) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c.d_next, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c.d_partials, sizeof(double) * std::max<size_t>(off, 1)) == cudaSuccess;
+    ok = ok && (b->QK == 0 || cudaMalloc((void **)&c.d_comps, sizeof(double) * std::max<size_t>(off, 1)) == cudaSuccess);
     ok = ok && cudaMalloc((void **)&c.d_state, sizeof(float) * (size_t)grid * R * nst * b->n_max * T) == cudaSuccess;
     ok = ok && cudaStreamSynchronize(st) == cudaSuccess;
     if (!ok) {
@@ -247,7 +259,7 @@ int launch_all(lll_batch *b, int scheme)
     const Sched &c = b->sched[scheme];
     BatchArgs a{};
     a.desc = b->d_desc; a.item_inst = c.d_item_inst; a.item_tiles = c.d_item_tiles; a.seg_off = c.d_seg_off;
-    a.partials = c.d_partials; a.state = c.d_state; a.next = c.d_next;
+    a.partials = c.d_partials; a.comps = c.d_comps; a.state = c.d_state; a.next = c.d_next;
     a.n_items = c.n_items; a.n_max = b->n_max; a.ns_max = b->ns_max;
     a.chunk_rows = c.CH;
     cudaStream_t st = b->stream;
@@ -255,7 +267,8 @@ int launch_all(lll_batch *b, int scheme)
     if (e != cudaSuccess) return (int)e;
     e = cudaMemsetAsync(c.d_next, 0, sizeof(int), st);
     if (e != cudaSuccess) return (int)e;
-    e = (cudaError_t)launch_batch_kernel(scheme, b->QP, c.R, c.grid, c.threads, c.smem, st, a);
+    e = (cudaError_t)(b->QK > 0 ? launch_batch_block_kernel(scheme, b->QK, c.R, c.grid, c.threads, c.smem, st, a)
+                                : launch_batch_kernel(scheme, b->QP, c.R, c.grid, c.threads, c.smem, st, a));
     if (e != cudaSuccess) return (int)e;
     return batch_finalize(c.d_partials, c.d_seg_off, c.d_inst_seg_ptr, c.d_inst_segs, b->d_out_off,
                           (int)b->inst.size(), b->d_out_count, b->d_sums, st);
@@ -299,6 +312,22 @@ int lll_batch_init(lll_batch **out, int n_inst, const lll_instance *inst, void *
         b->ns_max = std::max(b->ns_max, c->ns);
     }
     b->sm_count = b->inst[0]->sm_count;
+    int longest = 0;
+    bool all_shorter = true;
+    for (const lll_ctx *c : b->inst) {
+        longest = std::max(longest, c->QR);
+        all_shorter = all_shorter && c->QR < c->QP;
+    }
+    b->QK = !all_shorter ? 0 : longest <= 8 ? 8 : 32;
+    if (!all_shorter) // some instance sweeps its rule as given: all do
+        for (lll_ctx *c : b->inst) {
+            const int rc = use_full_tables(c);
+            if (rc != LLL_OK) {
+                std::string m = lll_last_error(c);
+                lll_batch_destroy(b);
+                return berr(nullptr, rc, m);
+            }
+        }
     if (cudaMallocHost((void **)&b->h_desc, sizeof(PathArgs) * n_inst) != cudaSuccess ||
         cudaEventCreate(&b->ev[0]) != cudaSuccess || cudaEventCreate(&b->ev[1]) != cudaSuccess) {
         lll_batch_destroy(b);

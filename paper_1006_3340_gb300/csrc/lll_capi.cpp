@@ -63,9 +63,10 @@ cudaError_t dalloc(T **p, size_t count)
 void free_all(lll_ctx *c)
 {
     cudaFree(c->d_lam); cudaFree(c->d_x); cudaFree(c->d_W); cudaFree(c->d_w0); cudaFree(c->d_b0);
-    cudaFree(c->d_tab); cudaFree(c->d_row); cudaFree(c->d_Z0); cudaFree(c->d_c0);
+    cudaFree(c->d_tab); cudaFree(c->d_row); cudaFree(c->d_Z0); cudaFree(c->d_L0); cudaFree(c->d_c0);
     cudaFree(c->d_strikes); cudaFree(c->d_partials); cudaFree(c->d_sums); cudaFree(c->d_state);
     cudaFree(c->d_snap); cudaFree(c->d_C); cudaFree(c->d_cn); cudaFree(c->d_err);
+    cudaFree(c->d_tab_full); cudaFree(c->d_row_full); cudaFree(c->d_cn_full);
     cudaFree(c->d_K1); cudaFree(c->d_K2); cudaFree(c->d_K3);
     mlp_free(c->mlp);
     c->mlp = nullptr;
@@ -87,18 +88,72 @@ namespace lll {
 
 int record_error(lll_ctx *ctx, int code, const char *msg) { return fail(ctx, code, msg); }
 
+int ensure_full_tables(lll_ctx *ctx)
+{
+    if (ctx->QR == ctx->QP || ctx->d_tab_full) return LLL_OK;
+    const size_t rows = (size_t)ctx->S * ctx->n;
+    float4 *tab = nullptr, *row = nullptr;
+    float *cn = nullptr;
+    cudaError_t e = dalloc(&tab, rows * (ctx->QP / 4));
+    if (e == cudaSuccess) e = dalloc(&row, rows);
+    if (e == cudaSuccess) e = dalloc(&cn, ctx->QP);
+    const bool room = e == cudaSuccess;
+    // D0 and b0 h as in the sweeps' rows; lambda, K and C are written by the tables
+    if (room) e = cudaMemcpyAsync(row, ctx->d_row, sizeof(float4) * rows, cudaMemcpyDeviceToDevice, ctx->stream);
+    if (e == cudaSuccess)
+        e = (cudaError_t)launch_tables(ctx->d_lam, ctx->d_x, ctx->d_W, ctx->Q, ctx->d_x, ctx->d_W, ctx->Q, ctx->n,
+                                       ctx->S, ctx->QP, tab, cn, row, ctx->d_C, ctx->stream);
+    if (e != cudaSuccess) {
+        cudaFree(tab);
+        cudaFree(row);
+        cudaFree(cn);
+        return room ? cuda_fail(ctx, e, "tables of the given rule") : fail(ctx, LLL_ENOMEM, "tables of the given rule");
+    }
+    ctx->d_tab_full = tab;
+    ctx->d_row_full = row;
+    ctx->d_cn_full = cn;
+    return LLL_OK;
+}
+
+int use_full_tables(lll_ctx *ctx)
+{
+    const int rc = ensure_full_tables(ctx);
+    if (rc != LLL_OK || !ctx->d_tab_full) return rc;
+    std::swap(ctx->d_tab, ctx->d_tab_full);
+    std::swap(ctx->d_row, ctx->d_row_full);
+    std::swap(ctx->d_cn, ctx->d_cn_full);
+    cudaFree(ctx->d_tab_full);
+    cudaFree(ctx->d_row_full);
+    cudaFree(ctx->d_cn_full);
+    ctx->d_tab_full = ctx->d_row_full = nullptr;
+    ctx->d_cn_full = nullptr;
+    ctx->QR = ctx->QP;
+    return LLL_OK;
+}
+
 int launch_plan(const LaunchPlan &plan, const PathArgs &a)
 {
     if (plan.tenor > 0) return launch_tenor_kernel(plan.scheme, plan.qp, plan.tenor, plan.grid, plan.smem, plan.stream, a);
     if (plan.lpp > 1)
         return launch_group_kernel(plan.scheme, plan.qp, plan.lpp, plan.grid, plan.threads, plan.smem, plan.stream, a);
+    if (plan.block)
+        return launch_block_kernel(plan.scheme, plan.qp, plan.ppt, plan.grid, plan.threads, plan.smem, plan.stream, a);
     return launch_path_kernel(plan.scheme, plan.qp, plan.ppt, plan.grid, plan.threads, plan.smem, plan.stream, a);
+}
+
+// Paths per thread and threads per block of the time-blocked kernel where the
+// caller has not set them.
+static void block_shape(const lll_ctx *ctx, uint64_t paths, int *R, int *T)
+{
+    const uint64_t sms = ctx->sm_count;
+    if (ctx->ppt == 0) *R = paths >= 512 * sms ? 2 : 1;
+    if (ctx->threads == 0) *T = paths >= 256 * sms * *R ? 128 : paths >= 128 * sms ? 64 : 32;
 }
 
 // Same launch shape and arguments as lll_simulate, with no allocation: the
 // per-block scratch sizes are returned for the caller to place.
 int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, uint64_t seed,
-                LaunchPlan *plan, bool allow_tenor)
+                LaunchPlan *plan, bool allow_tenor, bool given_rule)
 {
     if (!ctx) return fail(nullptr, LLL_EINVAL, "ctx is NULL");
     if (!plan) return fail(ctx, LLL_EINVAL, "plan is NULL");
@@ -109,6 +164,8 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     if (ctx->ns == 0) return fail(ctx, LLL_ESTATE, "lll_set_strikes must come before simulating");
     if (paths == 0) return fail(ctx, LLL_EINVAL, "paths must be > 0");
     if (first_path + paths < first_path) return fail(ctx, LLL_EINVAL, "path range overflows");
+    // What a launch supports follows the rule as given (QPk nodes); the one-lane
+    // kernels sweep its shorter equivalent, where there is one, in time blocks.
     const int QPk = (scheme == LLL_FROZEN) ? 0 : ctx->QP;
     // Tenor-parallel mapping (lll_set_mapping): G lanes per path, full and
     // Picard with a node table and caplet payoffs; other schemes keep the
@@ -122,16 +179,23 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     // Lanes per group of paths: 1 (one lane sweeps all nodes of its path) or
     // 2 / 4 (lane groups share the node sweep); the default is 1.
     const int lpp = G > 0 ? 1 : (ctx->lpp > 0 ? ctx->lpp : 1);
-    const int R = (lpp > 1 || G > 0) ? 1 : (ctx->ppt > 0 ? ctx->ppt : 1);
+    int R = (lpp > 1 || G > 0) ? 1 : (ctx->ppt > 0 ? ctx->ppt : 1);
     if (lpp > 1 && !group_kernel_supported(scheme, QPk, lpp))
         return fail(ctx, LLL_EUNSUPPORTED, "lane groups need a node table (NIG, full or Picard)");
     if (G == 0 && lpp == 1 && !path_kernel_supported(scheme, QPk, R))
         return fail(ctx, LLL_EUNSUPPORTED, "no kernel for this Q and paths per thread");
-    const int T = G > 0 ? tenor_kernel_threads() : ctx->threads, CH = ctx->chunk_rows;
-    const size_t smem = G > 0 ? tenor_kernel_smem(QPk, ctx->n, ctx->ns, G)
-                      : lpp > 1 ? group_kernel_smem(QPk, ctx->n, ctx->ns, T, CH)
-                                : path_kernel_smem(QPk, ctx->n, ctx->ns, T, CH);
+    int T = G > 0 ? tenor_kernel_threads() : ctx->threads > 0 ? ctx->threads : 128;
+    int CH = ctx->chunk_rows > 0 ? ctx->chunk_rows : default_chunk_rows(ctx->n, QPk);
+    size_t smem = G > 0 ? tenor_kernel_smem(QPk, ctx->n, ctx->ns, G)
+                : lpp > 1 ? group_kernel_smem(QPk, ctx->n, ctx->ns, T, CH)
+                          : path_kernel_smem(QPk, ctx->n, ctx->ns, T, CH);
     if (smem > 227 * 1024) return fail(ctx, LLL_EUNSUPPORTED, "shared memory need exceeds 227 KB");
+    const bool block = !given_rule && G == 0 && lpp == 1 && QPk > 0 && ctx->QR < ctx->QP;
+    if (block) {
+        block_shape(ctx, paths, &R, &T);
+        CH = block_chunk_rates(ctx->QR, R, ctx->n, ctx->chunk_rows);
+        smem = block_kernel_smem(ctx->QR, R, ctx->n, ctx->ns, T, CH);
+    }
     int occ = 0;
     cudaError_t e;
     if (G > 0) {
@@ -140,6 +204,9 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     } else if (lpp > 1) {
         e = (cudaError_t)group_kernel_prepare(scheme, QPk, lpp, smem, T, &occ);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "group kernel attributes");
+    } else if (block) {
+        e = (cudaError_t)block_kernel_prepare(scheme, ctx->QR, R, smem, T, &occ);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "block kernel attributes");
     } else {
         e = (cudaError_t)path_kernel_prepare(scheme, QPk, R, T, smem);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
@@ -153,13 +220,17 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)bps * ctx->sm_count);
     const int nst = (scheme == LLL_PICARD) ? 2 : 1;
     PathArgs a{};
-    a.tab = ctx->d_tab; a.cn = ctx->d_cn; a.row = ctx->d_row; a.Z0 = ctx->d_Z0; a.c0 = ctx->d_c0;
+    const bool other = !block && ctx->d_tab_full;
+    a.tab = other ? ctx->d_tab_full : ctx->d_tab;
+    a.cn = other ? ctx->d_cn_full : ctx->d_cn;
+    a.row = other ? ctx->d_row_full : ctx->d_row;
+    a.Z0 = ctx->d_Z0; a.L0 = ctx->d_L0; a.c0 = ctx->d_c0;
     a.strikes = ctx->d_strikes; a.partials = nullptr; a.state = nullptr;
     a.snap = nullptr; a.n_snap = 0; a.snap_stride = 1; a.snap_pitch = 0;
     a.first_path = first_path; a.paths = paths;
     a.n = ctx->n; a.s = ctx->s; a.S = ctx->S; a.ns = ctx->ns; a.chunk_rows = CH;
     a.key0 = (uint32_t)seed; a.key1 = (uint32_t)(seed >> 32); a.inst = 0;
-    a.driver = ctx->driver;
+    a.driver = ctx->driver; a.qr = block ? ctx->QR : QPk;
     a.h = (float)ctx->h; a.sqrt_h = (float)std::sqrt(ctx->h); a.delta = (float)ctx->delta;
     a.dBN = (float)(ctx->delta * ctx->BN);
     a.product = ctx->product;
@@ -171,12 +242,12 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
         a.nig_beta = (float)ctx->nig.beta; a.nig_muh = (float)(ctx->mu * ctx->h);
     }
     plan->args = a;
-    plan->scheme = scheme; plan->qp = QPk; plan->ppt = R; plan->lpp = lpp; plan->threads = T; plan->grid = grid;
+    plan->scheme = scheme; plan->qp = block ? ctx->QR : QPk; plan->block = block; plan->ppt = R; plan->lpp = lpp; plan->threads = T; plan->grid = grid;
     plan->tenor = G;
     plan->smem = smem;
     // the tenor-parallel kernel keeps its path state in shared memory
     plan->state_floats_per_block = G > 0 ? 0 : (size_t)R * nst * ctx->n * T;
-    plan->partial_doubles_per_block = (size_t)ctx->n * ctx->ns * 2;
+    plan->partial_doubles_per_block = (size_t)ctx->n * ctx->ns * 2 * (block ? 2 : 1);
     plan->n_out = ctx->n * ctx->ns * 2;
     plan->stream = ctx->stream;
     plan->device = ctx->device;
@@ -200,6 +271,21 @@ int lll_build_nig_quadrature(lll_nig nig, double xmax, int Q, double *nodes, dou
     return LLL_OK;
 }
 
+int lll_sweep_rule(int Q, const double *nodes, const double *weights, double lo, double hi, int *count,
+                   int *padded, double *x, double *w)
+{
+    if (!nodes || !weights || !count || !padded || !x || !w || Q < 1 || !(lo <= 0.0) || !(hi >= 0.0))
+        return fail(nullptr, LLL_EINVAL, "null argument, Q < 1, or not lo <= 0 <= hi");
+    const int QP = padded_q(Q);
+    if (QP < 0) return fail(nullptr, LLL_EUNSUPPORTED, "Q > 128");
+    for (int j = 0; j < Q; ++j)
+        if (!isfin(nodes[j]) || nodes[j] == 0.0 || !isfin(weights[j]))
+            return fail(nullptr, LLL_EINVAL, "nodes must be finite and non-zero");
+    *padded = QP;
+    *count = shorter_rule(nodes, weights, Q, QP, lo, hi, x, w, padded);
+    return LLL_OK;
+}
+
 int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int steps_per_period,
              const double *lambda, int driver, lll_nig nig, int Q, const double *nodes,
              const double *weights, void *cuda_stream)
@@ -214,6 +300,7 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     if (driver != LLL_DRIVER_NIG && driver != LLL_DRIVER_BROWNIAN)
         return fail(nullptr, LLL_EINVAL, "unknown driver");
     const int n = N - 1, S = n * steps_per_period;
+    double up = 0, down = 0; // largest sums of the live positive and negative volatilities over the steps
     for (int m = 0; m < N; ++m)
         if (!(L0[m] > 0) || !isfin(L0[m])) return fail(nullptr, LLL_EINVAL, "L0 must be finite and > 0");
     for (long long e = 0; e < (long long)S * n; ++e)
@@ -235,15 +322,27 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
         mu = std::isnan(nig.mu) ? -nig.delta * nig.beta / gam : nig.mu;
         if (!isfin(mu)) return fail(nullptr, LLL_EINVAL, "mu is Inf");
         for (int k = 0; k < S; ++k) {
-            double sum = 0;
-            for (int l = 0; l < n; ++l) sum += std::fabs(lambda[(size_t)k * n + l]);
+            double sum = 0, pos = 0, neg = 0;
+            for (int l = 0; l < n; ++l) {
+                const double v = lambda[(size_t)k * n + l];
+                sum += std::fabs(v);
+                if (l >= k / steps_per_period) (v > 0 ? pos : neg) += v;
+            }
+            up = std::max(up, pos);
+            down = std::min(down, neg);
             if (sum >= nig.alpha - std::fabs(nig.beta)) domain_warn = true;
         }
     } else {
         Q = 0;
     }
 
+    std::vector<double> xs(std::max(Q, 1), 0.0), ws(std::max(Q, 1), 0.0);
+    for (int j = 0; j < Q; ++j) { xs[j] = nodes[j]; ws[j] = weights[j]; }
+    int QR = QP, Qr = 0;
+    std::vector<double> xw(2 * kMaxQP, 0.0); // the shorter rule: nodes, then weights
+    if (QP > 0) Qr = shorter_rule(xs.data(), ws.data(), Q, QP, down, up, xw.data(), xw.data() + kMaxQP, &QR);
     lll_ctx *c = new lll_ctx();
+    c->QR = QR;
     c->N = N; c->n = n; c->s = steps_per_period; c->S = S; c->Q = Q; c->QP = QP;
     c->driver = driver; c->delta = tenor_delta; c->h = tenor_delta / steps_per_period;
     c->c = (driver == LLL_DRIVER_BROWNIAN) ? 1.0 : 0.0;
@@ -254,10 +353,11 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     double BN = 1.0;
     for (int m = 0; m < N; ++m) BN /= 1.0 + tenor_delta * L0[m]; // Eq. (i-val) inverted
     c->BN = BN;
-    c->chunk_rows = default_chunk_rows(n, QP);
+    double *d_short = nullptr; // the shorter rule's nodes and weights, for the tables
 
     auto bail = [&](int code) {
         std::string m = c->err;
+        cudaFree(d_short);
         free_all(c);
         delete c;
         g_err = m;
@@ -268,10 +368,11 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     if ((e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device)) != cudaSuccess) {
         cuda_fail(c, e, "cudaDeviceGetAttribute"); return bail(LLL_ECUDA);
     }
-    std::vector<float> Z0(n), c0(n);
+    std::vector<float> Z0(n), c0(n), Lf(n);
     std::vector<double> w0(n);
     for (int l = 1; l <= n; ++l) {
         Z0[l - 1] = (float)std::log(L0[l]);
+        Lf[l - 1] = (float)L0[l];
         c0[l - 1] = (float)(std::log(L0[l]) + std::log(tenor_delta));
         w0[l - 1] = tenor_delta * L0[l] / (1.0 + tenor_delta * L0[l]);
     }
@@ -279,17 +380,16 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     bool ok = dalloc(&c->d_lam, rows) == cudaSuccess && dalloc(&c->d_x, std::max(Q, 1)) == cudaSuccess &&
               dalloc(&c->d_W, std::max(Q, 1)) == cudaSuccess && dalloc(&c->d_w0, n) == cudaSuccess &&
               dalloc(&c->d_b0, rows) == cudaSuccess &&
-              dalloc(&c->d_tab, rows * std::max(QP / 4, 1)) == cudaSuccess &&
-              dalloc(&c->d_cn, std::max(QP, 4)) == cudaSuccess &&
+              dalloc(&c->d_tab, rows * std::max(QR / 4, 1)) == cudaSuccess &&
+              dalloc(&c->d_cn, std::max(QR, 4)) == cudaSuccess &&
+              (Qr == 0 || dalloc(&d_short, xw.size()) == cudaSuccess) &&
               dalloc(&c->d_row, rows) == cudaSuccess && dalloc(&c->d_C, rows) == cudaSuccess &&
-              dalloc(&c->d_Z0, n) == cudaSuccess &&
+              dalloc(&c->d_Z0, n) == cudaSuccess && dalloc(&c->d_L0, n) == cudaSuccess &&
               dalloc(&c->d_c0, n) == cudaSuccess;
     if (!ok) { fail(c, LLL_ENOMEM, "cudaMalloc of model tables failed"); return bail(LLL_ENOMEM); }
     for (auto &ev : c->ev)
         if ((e = cudaEventCreate(&ev)) != cudaSuccess) { cuda_fail(c, e, "cudaEventCreate"); return bail(LLL_ECUDA); }
     cudaStream_t st = c->stream;
-    std::vector<double> xs(std::max(Q, 1), 0.0), ws(std::max(Q, 1), 0.0);
-    for (int j = 0; j < Q; ++j) { xs[j] = nodes[j]; ws[j] = weights[j]; }
 #define INIT_TRY(expr)                                                                             \
     do {                                                                                           \
         cudaError_t e2 = (expr);                                                                   \
@@ -300,14 +400,20 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     INIT_TRY(cudaMemcpyAsync(c->d_W, ws.data(), sizeof(double) * ws.size(), cudaMemcpyHostToDevice, st));
     INIT_TRY(cudaMemcpyAsync(c->d_w0, w0.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
     INIT_TRY(cudaMemcpyAsync(c->d_Z0, Z0.data(), sizeof(float) * n, cudaMemcpyHostToDevice, st));
+    INIT_TRY(cudaMemcpyAsync(c->d_L0, Lf.data(), sizeof(float) * n, cudaMemcpyHostToDevice, st));
     INIT_TRY(cudaMemcpyAsync(c->d_c0, c0.data(), sizeof(float) * n, cudaMemcpyHostToDevice, st));
     INIT_TRY(cudaMemsetAsync(c->d_row, 0, sizeof(float4) * rows, st));
-    INIT_TRY((cudaError_t)launch_tables(c->d_lam, c->d_x, c->d_W, n, S, Q, QP, c->d_tab, c->d_cn, c->d_row, c->d_C, st));
+    if (Qr > 0)
+        INIT_TRY(cudaMemcpyAsync(d_short, xw.data(), sizeof(double) * xw.size(), cudaMemcpyHostToDevice, st));
+    const double *xr = Qr > 0 ? d_short : c->d_x, *wr = Qr > 0 ? d_short + kMaxQP : c->d_W;
+    INIT_TRY((cudaError_t)launch_tables(c->d_lam, c->d_x, c->d_W, Q, xr, wr, Qr > 0 ? Qr : Q, n, S, QR, c->d_tab,
+                                        c->d_cn, c->d_row, c->d_C, st));
     INIT_TRY((cudaError_t)launch_frozen_drift(c->d_lam, c->d_x, c->d_W, c->d_w0, n, S, Q, c->c, c->h,
                                               c->d_b0, c->d_row, st));
     // The host vectors above go out of scope: wait for the copies.
     INIT_TRY(cudaStreamSynchronize(st));
 #undef INIT_TRY
+    cudaFree(d_short);
     *out = c;
     if (domain_warn)
         return fail(c, LLL_EDOMAIN,
@@ -373,11 +479,15 @@ int lll_set_launch(lll_ctx *ctx, int threads_per_block, int blocks_per_sm, int c
         return fail(ctx, LLL_EINVAL, "paths_per_thread must be 0 (automatic), 1 or 2");
     if (lanes_per_path != 0 && lanes_per_path != 1 && lanes_per_path != 2 && lanes_per_path != 4)
         return fail(ctx, LLL_EINVAL, "lanes_per_path must be 0 (default), 1, 2 or 4");
+    if (lanes_per_path > 1) {
+        const int rc = ensure_full_tables(ctx);
+        if (rc != LLL_OK) return rc;
+    }
     ctx->ppt = paths_per_thread;
     ctx->lpp = lanes_per_path;
     if (threads_per_block) ctx->threads = threads_per_block;
     ctx->blocks_per_sm = blocks_per_sm;
-    ctx->chunk_rows = chunk_rows ? std::min(chunk_rows, ctx->n) : default_chunk_rows(ctx->n, ctx->QP);
+    ctx->chunk_rows = std::min(chunk_rows, ctx->n);
     return LLL_OK;
 }
 
@@ -397,6 +507,8 @@ int lll_set_mapping(lll_ctx *ctx, int mapping, int lanes)
     if (mapping != LLL_MAP_TENOR) return fail(ctx, LLL_EINVAL, "unknown mapping");
     if (lanes != 4 && lanes != 8 && lanes != 16 && lanes != 32)
         return fail(ctx, LLL_EINVAL, "lanes must be 4, 8, 16 or 32");
+    const int rc = ensure_full_tables(ctx);
+    if (rc != LLL_OK) return rc;
     ctx->tenor_lanes = lanes;
     ctx->step_map = false;
     return LLL_OK;
@@ -413,7 +525,7 @@ int simulate_step(lll_ctx *ctx, uint64_t first_path, uint64_t paths, uint64_t se
     LaunchPlan plan;
     int rc = plan_launch(ctx, LLL_PICARD, first_path, paths, seed, &plan, false);
     if (rc != LLL_OK) return rc;
-    if (plan.qp == 0 || !step_kernels_supported(plan.qp, ctx->ns))
+    if (plan.qp == 0 || !step_kernels_supported(plan.qp, plan.block, ctx->ns))
         return fail(ctx, LLL_EUNSUPPORTED, "the step-parallel mapping needs a node table and at most 64 strikes");
     const int n = ctx->n, S = ctx->S;
     // intermediate arrays of about 4 (S + 2 S n + n^2) bytes per path: chunks within 2 GiB
@@ -453,7 +565,7 @@ int simulate_step(lll_ctx *ctx, uint64_t first_path, uint64_t paths, uint64_t se
     int block0 = 0;
     for (uint64_t c0 = 0; c0 < paths; c0 += Pc) {
         const int pc = (int)std::min<uint64_t>(Pc, paths - c0);
-        const cudaError_t e = (cudaError_t)launch_step_chunk(plan.qp, a, c0, pc, dH, Y, Bh, Zm, block0,
+        const cudaError_t e = (cudaError_t)launch_step_chunk(plan.qp, plan.block, a, c0, pc, dH, Y, Bh, Zm, block0,
                                                              ctx->d_partials, ctx->stream);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "step-parallel kernels");
         block0 += step_blocks_per_chunk(pc);
@@ -505,14 +617,13 @@ int lll_simulate(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, 
         if (dalloc(&ctx->d_state, state_need) != cudaSuccess) return fail(ctx, LLL_ENOMEM, "state scratch");
         ctx->state_cap = state_need;
     }
-    const size_t nout = (size_t)plan.n_out;
-    if ((size_t)grid * nout > ctx->partials_cap) {
+    const size_t nout = (size_t)plan.n_out, part_need = plan.partial_doubles_per_block * grid;
+    if (part_need > ctx->partials_cap) {
         cudaFree(ctx->d_partials);
         ctx->d_partials = nullptr;
         ctx->partials_cap = 0;
-        if (dalloc(&ctx->d_partials, (size_t)grid * nout) != cudaSuccess)
-            return fail(ctx, LLL_ENOMEM, "partials");
-        ctx->partials_cap = (size_t)grid * nout;
+        if (dalloc(&ctx->d_partials, part_need) != cudaSuccess) return fail(ctx, LLL_ENOMEM, "partials");
+        ctx->partials_cap = part_need;
     }
     if (nout > ctx->sums_cap) {
         cudaFree(ctx->d_sums);

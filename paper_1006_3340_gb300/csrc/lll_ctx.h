@@ -16,6 +16,7 @@ void mlp_free(MlpState *m);
 
 struct lll_ctx {
     int N = 0, n = 0, s = 0, S = 0, Q = 0, QP = 0, driver = 0;
+    int QR = 0; // padded nodes of the rule the sweeps use (shorter_rule), <= QP
     double delta = 0, h = 0, c = 0, mu = 0, gam = 0, BN = 0;
     lll_nig nig{};
     cudaStream_t stream = nullptr;
@@ -23,10 +24,15 @@ struct lll_ctx {
     std::vector<double> L0;
     // device
     double *d_lam = nullptr, *d_x = nullptr, *d_W = nullptr, *d_w0 = nullptr, *d_b0 = nullptr;
-    float4 *d_tab = nullptr, *d_row = nullptr;
-    float *d_cn = nullptr; // [QP]: c_j = W_j / x_j^2
+    float4 *d_tab = nullptr, *d_row = nullptr; // of the sweeps' rule
+    float *d_cn = nullptr; // [QR]: c_j = W_j / x_j^2
+    // The same for the rule as given (lane groups, the tenor-parallel mapping and
+    // training data), built when one of them is first selected; null where the
+    // sweeps' rule is the given one.
+    float4 *d_tab_full = nullptr, *d_row_full = nullptr;
+    float *d_cn_full = nullptr;
     float *d_C = nullptr; // [S][n]: C_l(t_k), the compensator at zero weights (FP64-built)
-    float *d_Z0 = nullptr, *d_c0 = nullptr, *d_strikes = nullptr;
+    float *d_Z0 = nullptr, *d_L0 = nullptr, *d_c0 = nullptr, *d_strikes = nullptr;
     double *d_partials = nullptr, *d_sums = nullptr;
     size_t partials_cap = 0, sums_cap = 0;
     float *d_state = nullptr;
@@ -38,7 +44,7 @@ struct lll_ctx {
     bool simulated = false;
     uint64_t last_paths = 0;
     uint64_t last_snap_paths = 0;
-    int threads = 128, blocks_per_sm = 0, chunk_rows = 0, ppt = 0, lpp = 0; // 0: automatic
+    int threads = 0, blocks_per_sm = 0, chunk_rows = 0, ppt = 0, lpp = 0; // 0: automatic
     int tenor_lanes = 0; // > 0: full and Picard on the tenor-parallel kernel (lll_set_mapping)
     bool step_map = false; // Picard with its Euler steps in parallel (lll_set_mapping)
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};

@@ -21,6 +21,7 @@ struct PathArgs {
     const float *cn;      // [QP]: c_j = W_j / x_j^2 (0 on padding nodes)
     const float4 *row;    // [S][n]: (lambda_l(t_k), K_l(k), D0_l(t_k), b0_l(t_k) * h)
     const float *Z0;      // [n]: log L(0, T_l)
+    const float *L0;      // [n]: L(0, T_l)
     const float *c0;      // [n]: log L(0, T_l) + log delta
     const float *strikes; // [n][ns]
     double *partials;     // [grid][n][ns][2]: per-block payoff sum and sum of squares
@@ -30,6 +31,7 @@ struct PathArgs {
     uint64_t first_path, paths;
     int n, s, S, ns, chunk_rows;
     uint32_t key0, key1, inst;
+    int qr;               // padded nodes per table row (0: no table)
     int driver;           // 0 NIG, 1 Brownian
     float h, sqrt_h, delta, dBN; // dBN = delta * B(0, T_N)
     int product;          // 0: caplets, 1: co-terminal payer swaptions (see lll_device.cuh)
@@ -46,6 +48,7 @@ struct BatchArgs {
     const uint2 *item_tiles; // [items] tile range [x, y) of the item within its instance
     const size_t *seg_off;   // [items] offset (doubles) of each item's output in partials
     double *partials;        // item outputs: [n][ns][2] per item
+    double *comps;           // their Kahan compensations (block kernels)
     float *state;            // [grid][NST][n_max][threads]
     int *next;               // claim counter, 0 at launch
     int n_items, n_max, ns_max, chunk_rows;
@@ -56,8 +59,11 @@ struct BatchArgs {
 struct LaunchPlan {
     PathArgs args;
     int scheme, qp, ppt, lpp, threads, grid; // lpp: lanes per group of paths (1, 2 or 4)
+    bool block;                              // time-blocked kernel (lll_paths_block.cu)
     int tenor;                               // > 0: tenor-parallel kernel with this many lanes per path
     size_t smem;
+    // scratch per block: path state; payoff sums (block kernel: and their compensations,
+    // behind the sums of all blocks)
     size_t state_floats_per_block, partial_doubles_per_block;
     int n_out; // doubles written by the final reduction: n * n_strikes * 2
     cudaStream_t stream;
@@ -73,6 +79,18 @@ int path_kernel_prepare(int scheme, int QP, int R, int threads, size_t smem);
 bool path_kernel_supported(int scheme, int QP, int R);
 size_t path_kernel_smem(int QP, int n, int ns, int threads, int chunk_rows);
 
+// Launchers implemented in lll_paths_block.cu (rules with a shorter equivalent,
+// QP = 4, 8, 12, 16, 24 or 32; a batch at each instance's own length up to
+// QMAX = 8 or 32).
+int block_chunk_rates(int QP, int R, int n, int rows);
+size_t block_kernel_smem(int QP, int R, int n, int ns, int threads, int chunk_rates);
+int block_kernel_prepare(int scheme, int QP, int R, size_t smem, int threads, int *blocks_per_sm);
+int launch_block_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st,
+                        const PathArgs &a);
+int batch_block_prepare(int scheme, int QMAX, int R, size_t smem, int threads, int *blocks_per_sm);
+int launch_batch_block_kernel(int scheme, int QMAX, int R, int grid, int threads, size_t smem, cudaStream_t st,
+                              const struct BatchArgs &b);
+
 // Launchers implemented in lll_paths_group.cu (four lanes per group of four paths).
 bool group_kernel_supported(int scheme, int QP, int G);
 size_t group_kernel_smem(int QP, int n, int ns, int threads, int chunk_rows);
@@ -87,10 +105,10 @@ int tenor_kernel_threads();
 int tenor_kernel_prepare(int scheme, int QP, int G, size_t smem, int *blocks_per_sm);
 int launch_tenor_kernel(int scheme, int QP, int G, int grid, size_t smem, cudaStream_t st, const PathArgs &a);
 // Launchers implemented in lll_paths_step.cu (Picard with its Euler steps in parallel).
-bool step_kernels_supported(int QP, int ns);
+bool step_kernels_supported(int QP, bool shorter, int ns);
 size_t step_bytes_per_path(int n, int S);
 int step_blocks_per_chunk(int Pc);
-int launch_step_chunk(int QP, const PathArgs &a, uint64_t chunk_first, int Pc, float *dH, float *Y, float *Bh,
+int launch_step_chunk(int QP, bool shorter, const PathArgs &a, uint64_t chunk_first, int Pc, float *dH, float *Y, float *Bh,
                       float *Zm, int block0, double *partials, cudaStream_t st);
 struct LaunchPlan;
 int launch_plan(const LaunchPlan &plan, const PathArgs &a);
@@ -100,8 +118,9 @@ int launch_batch_kernel(int scheme, int QP, int R, int grid, int threads, size_t
                         const BatchArgs &b);
 
 // Launchers implemented in lll_tables.cu.
-int launch_tables(const double *lam, const double *x, const double *W, int n, int S, int Q, int QP,
-                  float4 *tab, float *cn, float4 *row, float *Ctab, cudaStream_t st);
+// xr, Wr, Qr: the rule of the table (padded to QP nodes); x, W, Q: the rule as given, for C.
+int launch_tables(const double *lam, const double *x, const double *W, int Q, const double *xr, const double *Wr,
+                  int Qr, int n, int S, int QP, float4 *tab, float *cn, float4 *row, float *Ctab, cudaStream_t st);
 int launch_frozen_drift(const double *lam, const double *x, const double *W, const double *w0,
                         int n, int S, int Q, double c, double h, double *b0, float4 *row,
                         cudaStream_t st);
@@ -119,7 +138,13 @@ namespace lll {
 // Implemented in lll_capi.cpp.
 // allow_tenor: honour the context's tenor-parallel mapping (lll_set_mapping);
 // callers that only need the path arguments of the full scheme pass false.
+// given_rule: plan for the rule as given, not for its shorter equivalent.
 int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, uint64_t seed,
-                LaunchPlan *plan, bool allow_tenor = true);
+                LaunchPlan *plan, bool allow_tenor = true, bool given_rule = false);
 int record_error(lll_ctx *ctx, int code, const char *msg);
+int ensure_full_tables(lll_ctx *ctx); // the tables of the rule as given
+int use_full_tables(lll_ctx *ctx);    // every sweep of this context takes them from now on
+// Implemented in lll_quadrature.cpp.
+int shorter_rule(const double *x, const double *W, int Q, int Qpad, double lo, double hi, double *xr, double *Wr,
+                 int *pad);
 }  // namespace lll

@@ -493,7 +493,13 @@ int lll_mlp_train(lll_ctx *ctx, const lll_mlp_cfg *cfg, double *final_loss)
     // 1. training data from the quadrature full scheme
     LaunchPlan plan;
     rc = plan_launch(ctx, LLL_FULL, 0, P, cfg->seed ^ 0x5EED5EEDull, &plan, false);
+    if (rc == LLL_OK) rc = ensure_full_tables(ctx); // the targets are integrals of the rule as given
     if (rc != LLL_OK) return rc;
+    if (ctx->d_tab_full) {
+        plan.args.tab = ctx->d_tab_full;
+        plan.args.cn = ctx->d_cn_full;
+        plan.args.row = ctx->d_row_full;
+    }
     float *state = nullptr, *rec_u = nullptr, *rec_y = nullptr;
     int *rec_k = nullptr;
     double *part = nullptr;

@@ -16,6 +16,7 @@
 // cudaDeviceReset the module, and with it the array, may be reloaded at
 // another address); a call made during a capture, when the lookup is not
 // allowed, uses the address the last uncaptured call found on that device.
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 #include <string>
@@ -64,11 +65,15 @@ extern "C" int lll_simulate_noalloc(lll_ctx *ctx, int scheme, uint64_t first_pat
     using namespace lll;
     if (!ctx) return record_error(nullptr, LLL_EINVAL, "ctx is NULL");
     if (!d_sums) return record_error(ctx, LLL_EINVAL, "d_sums is NULL");
+    // The maximum is held against the launch of the rule as given, whatever
+    // kernel sweeps its shorter equivalent.
     LaunchPlan plan;
-    int rc = plan_launch(ctx, scheme, first_path, paths, seed, &plan);
+    int rc = plan_launch(ctx, scheme, first_path, paths, seed, &plan, true, true);
     if (rc != LLL_OK) return rc;
-    const size_t state_bytes = round256(sizeof(float) * plan.state_floats_per_block * plan.grid);
-    const size_t need = state_bytes + sizeof(double) * plan.partial_doubles_per_block * plan.grid;
+    auto state_of = [](const LaunchPlan &p, int grid) {
+        return round256(sizeof(float) * p.state_floats_per_block * grid);
+    };
+    const size_t need = state_of(plan, plan.grid) + sizeof(double) * plan.partial_doubles_per_block * plan.grid;
     if (need > kScratchBytes) {
         char msg[256];
         std::snprintf(msg, sizeof msg,
@@ -77,6 +82,13 @@ extern "C" int lll_simulate_noalloc(lll_ctx *ctx, int scheme, uint64_t first_pat
                       need, plan.grid, kScratchBytes);
         return record_error(ctx, LLL_EUNSUPPORTED, msg);
     }
+    rc = plan_launch(ctx, scheme, first_path, paths, seed, &plan);
+    if (rc != LLL_OK) return rc;
+    // as many of the launch's blocks as the scratch holds: the blocks loop over
+    // the path tiles, and the sums differ only in how FP64 partials are grouped
+    while (plan.grid > 1 && state_of(plan, plan.grid) + sizeof(double) * plan.partial_doubles_per_block * plan.grid > kScratchBytes)
+        plan.grid = plan.grid - std::max(1, plan.grid / 16);
+    const size_t state_bytes = state_of(plan, plan.grid);
     int current = -1;
     cudaError_t e = cudaGetDevice(&current);
     if (e != cudaSuccess || current != plan.device)

@@ -40,43 +40,10 @@
 
 #include "lll_device.cuh"
 #include "lll_internal.h"
+#include "lll_sweep.cuh"
 
 namespace lll {
 namespace {
-
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
-{
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_wait_0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// delta L / (1 + delta L) for x = log(delta L) (approximate ex2 and rcp: w only
-// scales the state-dependent part of the compensator).
-__device__ __forceinline__ float weight_of(float x)
-{
-    float e, r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-1.4426950408889634f * x));
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
-    return r;
-}
-
-__device__ __forceinline__ void kahan_add(double *s, double *c, double x)
-{
-    const double y = x - *c;
-    const double t = *s + y;
-    *c = (t - *s) - y;
-    *s = t;
-}
-
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
 
 struct Smem {
     float4 *tab;  // [2][CH * QP/4]
@@ -389,7 +356,8 @@ __global__ void __launch_bounds__(Bounds<LB>::threads, Bounds<LB>::blocks) path_
 // item writes its payoff sums to its own segment, and a second kernel adds the
 // segments of each instance in tile order, so the results do not depend on
 // which block ran which item.  R paths per thread, as in path_kernel (a tile
-// is T R paths).
+// is T R paths).  Instances whose rules have shorter equivalents run in
+// lll_paths_block.cu.
 template <int SCHEME, int QP, int R>
 __global__ void __launch_bounds__(kMaxThreads) batch_kernel(const BatchArgs b)
 {

@@ -28,26 +28,12 @@
 
 #include "lll_device.cuh"
 #include "lll_internal.h"
+#include "lll_sweep.cuh"
 
 namespace lll {
 namespace {
 
 constexpr int kSpT = 128; // threads per block of every kernel here
-
-__device__ __forceinline__ float weight_of(float x)
-{
-    float e, r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-1.4426950408889634f * x));
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
-    return r;
-}
-
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
 
 __global__ void __launch_bounds__(kSpT) sp_draw(const PathArgs a, uint64_t chunk_first, int Pc, float *dH)
 {
@@ -94,7 +80,8 @@ __global__ void __launch_bounds__(kSpT) sp_scan_y(const PathArgs a, int Pc, cons
 
 // block (path block, step k): the live E rows of step k in shared memory, one
 // thread per path sweeping the live rates n .. imin as the one-lane kernel does.
-template <int QP>
+// SHORT: the shorter equivalent rule, with the arithmetic of lll_sweep.cuh.
+template <int QP, bool SHORT>
 __global__ void __launch_bounds__(kSpT) sp_sweep(const PathArgs a, int Pc, const float *Y, float *Bh)
 {
     constexpr int Q2 = QP / 2, Q4 = QP / 4;
@@ -125,30 +112,42 @@ __global__ void __launch_bounds__(kSpT) sp_sweep(const PathArgs a, int Pc, const
         const float4 rc = row[r]; // lambda, K, D0, b0 h
         const float w = weight_of(c0[r] + rc.z + yn);
         if (i > imin) yn = Yk[(size_t)(i - 2) * Pc];
-        const float2 w2 = make_float2(w, w);
         const float4 *tr = tab + (size_t)r * Q4;
-        float2 acc[4];
+        float A;
+        if constexpr (SHORT) {
+            float4 E[Q4];
 #pragma unroll
-        for (int j4 = 0; j4 < Q4; ++j4) {
-            const float4 v = tr[j4];
+            for (int j = 0; j < Q4; ++j) E[j] = tr[j];
+            A = sweep_dot<QP>(E, P, rc.y);
+            sweep_grow<QP>(E, P, w);
+        } else {
+            const float2 w2 = make_float2(w, w);
+            float2 acc[4];
 #pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                const int j = 2 * j4 + hf;
-                const float2 e2 = hf ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
-                const float2 u = __fmul2_rn(e2, P[j]);
-                acc[j & 3] = (j < 4) ? u : __fadd2_rn(acc[j & 3], u);
-                P[j] = __ffma2_rn(w2, u, P[j]);
+            for (int j4 = 0; j4 < Q4; ++j4) {
+                const float4 v = tr[j4];
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    const int j = 2 * j4 + hf;
+                    const float2 e2 = hf ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+                    const float2 u = __fmul2_rn(e2, P[j]);
+                    acc[j & 3] = (j < 4) ? u : __fadd2_rn(acc[j & 3], u);
+                    P[j] = __ffma2_rn(w2, u, P[j]);
+                }
             }
+            const float2 s2 = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
+            A = rc.y + (s2.x + s2.y);
         }
-        const float2 s2 = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
-        Bh[((size_t)k * n + (i - 1)) * Pc + lp] = -(rc.y + (s2.x + s2.y)) * h;
+        Bh[((size_t)k * n + (i - 1)) * Pc + lp] = -A * h;
     }
 }
 
 // thread (i, path): running sums of the drift and of lambda dH; at every
-// maturity T_m (m <= i) the log-rate log L_i(T_m) into Zm[m-1][i-1][p].  The
+// maturity T_m (m <= i) log L_i(T_m) (shorter rule: its offset from log L_i(0),
+// which the time-blocked kernels' payoffs take) into Zm[m-1][i-1][p].  The
 // drift terms of sixteen steps are loaded ahead of their additions (same
 // operations in the same order), as in sp_scan_y.
+template <bool SHORT>
 __global__ void __launch_bounds__(kSpT) sp_scan_d(const PathArgs a, int Pc, uint64_t chunk_first,
                                                   const float *__restrict__ dH, const float *__restrict__ Y,
                                                   const float *__restrict__ Bh, float *__restrict__ Zm)
@@ -182,7 +181,7 @@ __global__ void __launch_bounds__(kSpT) sp_scan_d(const PathArgs a, int Pc, uint
                                       : fmaf(a.row[(size_t)k * n + (i - 1)].x, __ldg(dH + (size_t)k * Pc + lp),
                                              __ldg(Y + ki));
                 const float z = y + d + a.Z0[i - 1];
-                Zm[((size_t)(m - 1) * n + (i - 1)) * Pc + lp] = z;
+                Zm[((size_t)(m - 1) * n + (i - 1)) * Pc + lp] = SHORT ? y + d : z;
                 if (sidx != ~0ull) a.snap[((size_t)(m - 1) * n + (i - 1)) * a.snap_pitch + sidx] = z;
             }
         }
@@ -191,6 +190,7 @@ __global__ void __launch_bounds__(kSpT) sp_scan_d(const PathArgs a, int Pc, uint
 
 // block (path block, maturity m): caplet payoffs of the block's paths at T_m,
 // reduced in fixed order into partials[block][m-1][q][2].
+template <bool SHORT>
 __global__ void __launch_bounds__(kSpT) sp_payoff(const PathArgs a, int Pc, uint64_t chunk_first, const float *Zm,
                                                   int block0, double *partials)
 {
@@ -201,8 +201,11 @@ __global__ void __launch_bounds__(kSpT) sp_payoff(const PathArgs a, int Pc, uint
     const bool active = lp < Pc && chunk_first + lp < a.paths;
     double Pp = 1.0, Sp = 1.0;
     float Lm = 0.0f;
-    if (lp < Pc)
-        maturity_products(a, m, [&](int i) { return Zm[((size_t)(m - 1) * n + (i - 1)) * Pc + lp]; }, Pp, Sp, Lm);
+    if (lp < Pc) {
+        auto z = [&](int i) { return Zm[((size_t)(m - 1) * n + (i - 1)) * Pc + lp]; };
+        if constexpr (SHORT) maturity_factors(a, m, z, Pp, Sp, Lm);
+        else maturity_products(a, m, z, Pp, Sp, Lm);
+    }
     for (int q = 0; q < ns; ++q) {
         const float K = a.strikes[(size_t)(m - 1) * ns + q];
         const size_t slot = (size_t)warp * ns + q;
@@ -231,14 +234,18 @@ __global__ void __launch_bounds__(kSpT) sp_payoff(const PathArgs a, int Pc, uint
 
 typedef void (*SweepFn)(const PathArgs, int, const float *, float *);
 
-SweepFn pick_sweep(int QP)
+SweepFn pick_sweep(int QP, bool shorter)
 {
     switch (QP) {
-    case 16: return sp_sweep<16>;
-    case 32: return sp_sweep<32>;
-    case 64: return sp_sweep<64>;
-    case 96: return sp_sweep<96>;
-    case 128: return sp_sweep<128>;
+    case 4: return shorter ? sp_sweep<4, true> : nullptr;
+    case 8: return shorter ? sp_sweep<8, true> : nullptr;
+    case 12: return shorter ? sp_sweep<12, true> : nullptr;
+    case 16: return shorter ? sp_sweep<16, true> : sp_sweep<16, false>;
+    case 24: return shorter ? sp_sweep<24, true> : nullptr;
+    case 32: return shorter ? sp_sweep<32, true> : sp_sweep<32, false>;
+    case 64: return shorter ? nullptr : sp_sweep<64, false>;
+    case 96: return shorter ? nullptr : sp_sweep<96, false>;
+    case 128: return shorter ? nullptr : sp_sweep<128, false>;
     default: return nullptr;
     }
 }
@@ -247,7 +254,7 @@ unsigned blocks_of(size_t count) { return (unsigned)((count + kSpT - 1) / kSpT);
 
 }  // namespace
 
-bool step_kernels_supported(int QP, int ns) { return pick_sweep(QP) != nullptr && ns <= 64; }
+bool step_kernels_supported(int QP, bool shorter, int ns) { return pick_sweep(QP, shorter) != nullptr && ns <= 64; }
 
 size_t step_bytes_per_path(int n, int S) { return 4 * ((size_t)S + 2 * (size_t)S * n + (size_t)n * n); }
 
@@ -262,10 +269,10 @@ size_t step_sweep_smem(int QP, int n)
 // One chunk of Pc paths starting at chunk_first (relative to a.first_path).
 // scratch: dH [S][Pc], Y and Bh [S][n][Pc], Zm [n][n][Pc] (floats).
 // Payoff partials go to blocks block0 .. block0 + step_blocks_per_chunk(Pc) - 1.
-int launch_step_chunk(int QP, const PathArgs &a, uint64_t chunk_first, int Pc, float *dH, float *Y, float *Bh,
+int launch_step_chunk(int QP, bool shorter, const PathArgs &a, uint64_t chunk_first, int Pc, float *dH, float *Y, float *Bh,
                       float *Zm, int block0, double *partials, cudaStream_t st)
 {
-    SweepFn sw = pick_sweep(QP);
+    SweepFn sw = pick_sweep(QP, shorter);
     if (!sw || a.ns > 64) return (int)cudaErrorInvalidValue;
     const int n = a.n, S = a.S;
     sp_draw<<<blocks_of((size_t)S * Pc), kSpT, 0, st>>>(a, chunk_first, Pc, dH);
@@ -274,8 +281,10 @@ int launch_step_chunk(int QP, const PathArgs &a, uint64_t chunk_first, int Pc, f
     cudaError_t e = cudaFuncSetAttribute(sw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     sw<<<dim3(blocks_of((size_t)Pc), S), kSpT, smem, st>>>(a, Pc, Y, Bh);
-    sp_scan_d<<<blocks_of((size_t)n * Pc), kSpT, 0, st>>>(a, Pc, chunk_first, dH, Y, Bh, Zm);
-    sp_payoff<<<dim3(blocks_of((size_t)Pc), n), kSpT, 0, st>>>(a, Pc, chunk_first, Zm, block0, partials);
+    const auto scan_d = shorter ? sp_scan_d<true> : sp_scan_d<false>;
+    scan_d<<<blocks_of((size_t)n * Pc), kSpT, 0, st>>>(a, Pc, chunk_first, dH, Y, Bh, Zm);
+    const auto pay = shorter ? sp_payoff<true> : sp_payoff<false>;
+    pay<<<dim3(blocks_of((size_t)Pc), n), kSpT, 0, st>>>(a, Pc, chunk_first, Zm, block0, partials);
     return (int)cudaGetLastError();
 }
 

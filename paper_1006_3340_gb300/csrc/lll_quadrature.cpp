@@ -51,35 +51,16 @@ double x2nu(double x, double alpha, double beta, double dbar)
     return dbar * alpha / M_PI * ax * std::exp(beta * x) * std::cyl_bessel_k(1.0, alpha * ax);
 }
 
-}  // namespace
-
-// Returns 0 on success.
-int build_nig_rule(double alpha, double beta, double dbar, double a, int Q, double *nodes,
-                   double *weights)
+// Recurrence coefficients al[0..Q), bt[1..Q) of the polynomials orthonormal for
+// the measure sum_i v_i delta_{y_i} (Stieltjes procedure with orthonormal
+// vectors q_k(y_i) sqrt(v_i) and full re-orthogonalisation).  0 on success.
+int jacobi_of_measure(const std::vector<double> &y, const std::vector<double> &v, int Q, std::vector<double> &al,
+                      std::vector<double> &bt, double &mu0)
 {
-    const int G = 32;
-    std::vector<double> gt, gw;
-    gauss_legendre(G, gt, gw);
-    std::vector<double> edges;
-    edges.push_back(0.0);
-    const int outer = 24;
-    for (double e = 1e-14 * a; e < a / outer; e /= 0.35) edges.push_back(e);
-    for (int i = 1; i <= outer; ++i) edges.push_back(a * i / outer);
-    std::vector<double> y, v;
-    for (int side = -1; side <= 1; side += 2)
-        for (size_t p = 0; p + 1 < edges.size(); ++p) {
-            const double lo = edges[p], hi = edges[p + 1];
-            const double mid = 0.5 * (lo + hi), half = 0.5 * (hi - lo);
-            for (int g = 0; g < G; ++g) {
-                const double xx = side * (mid + half * gt[g]);
-                y.push_back(xx);
-                v.push_back(half * gw[g] * x2nu(xx, alpha, beta, dbar));
-            }
-        }
     const size_t M = y.size();
-    // Stieltjes with orthonormal vectors q_k(y_i) sqrt(v_i).
-    std::vector<double> al(Q, 0.0), bt(Q + 1, 0.0);
-    double mu0 = 0.0;
+    al.assign(Q, 0.0);
+    bt.assign(Q + 1, 0.0);
+    mu0 = 0.0;
     for (size_t i = 0; i < M; ++i) mu0 += v[i];
     if (!(mu0 > 0.0)) return -1;
     std::vector<std::vector<double>> qs;
@@ -108,6 +89,13 @@ int build_nig_rule(double alpha, double beta, double dbar, double a, int Q, doub
         for (size_t i = 0; i < M; ++i) r[i] /= nr;
         qs.push_back(r);
     }
+    return 0;
+}
+
+// The Q-point Gauss rule of those coefficients (Q at most their number).
+void gauss_of_jacobi(const std::vector<double> &al, const std::vector<double> &bt, double mu0, int Q, double *nodes,
+                     double *weights)
+{
     // Eigenvalues of the Jacobi matrix by bisection on Sturm counts.
     double lo = al[0], hi = al[0];
     for (int k = 0; k < Q; ++k) {
@@ -147,6 +135,117 @@ int build_nig_rule(double alpha, double beta, double dbar, double a, int Q, doub
             s += pc * pc;
         }
         weights[j] = 1.0 / s;
+    }
+}
+
+}  // namespace
+
+// Returns 0 on success.
+int build_nig_rule(double alpha, double beta, double dbar, double a, int Q, double *nodes,
+                   double *weights)
+{
+    const int G = 32;
+    std::vector<double> gt, gw;
+    gauss_legendre(G, gt, gw);
+    std::vector<double> edges;
+    edges.push_back(0.0);
+    const int outer = 24;
+    for (double e = 1e-14 * a; e < a / outer; e /= 0.35) edges.push_back(e);
+    for (int i = 1; i <= outer; ++i) edges.push_back(a * i / outer);
+    std::vector<double> y, v;
+    for (int side = -1; side <= 1; side += 2)
+        for (size_t p = 0; p + 1 < edges.size(); ++p) {
+            const double lo = edges[p], hi = edges[p + 1];
+            const double mid = 0.5 * (lo + hi), half = 0.5 * (hi - lo);
+            for (int g = 0; g < G; ++g) {
+                const double xx = side * (mid + half * gt[g]);
+                y.push_back(xx);
+                v.push_back(half * gw[g] * x2nu(xx, alpha, beta, dbar));
+            }
+        }
+    std::vector<double> al, bt;
+    double mu0 = 0.0;
+    const int rc = jacobi_of_measure(y, v, Q, al, bt, mu0);
+    if (rc != 0) return rc;
+    gauss_of_jacobi(al, bt, mu0, Q, nodes, weights);
+    return 0;
+}
+
+// ---- A shorter rule for the same measure -----------------------------------
+// The path kernels integrate, for every path, step and rate,
+//     A_i - C_i = sum_j W_j / x_j^2 (e^{lambda_i x_j} - 1) (P(x_j) - 1),
+//     P(x) = prod_{l > i} (1 - w_l + w_l e^{lambda_l x}),  w_l in (0, 1).
+// Expanded, P is a convex combination of exponentials e^{theta x}, theta a sum
+// of some of the lambda_l, and
+//     (e^{lambda x} - 1) (e^{theta x} - 1) / x^2 = int_0^lambda int_0^theta e^{(u+v) x} dv du,
+// so every such integral is an integral over tau = u + v of the rule's moment
+// generating function G(tau) = sum_j W_j e^{tau x_j}, tau between minus the sum
+// of the negative and the sum of the positive lambda's.  A rule of q nodes
+// whose generating function agrees with G to a relative eps over that interval
+// therefore gives A_i - C_i to the relative error eps (against the absolute
+// value of its terms, where the lambda's differ in sign), whatever the path's
+// rates are.  The q-point Gauss rule of the discrete measure sum_j W_j
+// delta_{x_j} is the natural one (Gautschi 2004, "Orthogonal Polynomials:
+// Computation and Approximation", 2.2): exact to degree 2q - 1.
+//
+// eps = 2^-28, a sixteenth of FP32's unit roundoff, in which the integral is
+// summed.  A second condition keeps the sum's rounding no larger than the
+// given rule's: the terms c_j E_ij sum in absolute value to about
+// |lambda| sum_j W_j / |x_j|, which a node next to 0 inflates.
+constexpr double kRuleTol = 1.0 / 268435456.0;
+
+static bool same_generating_function(const double *x, const double *W, int Q, const double *xr, const double *Wr,
+                                     int q, double lo, double hi)
+{
+    constexpr int kGrid = 32; // the relative error grows smoothly away from tau = 0
+    for (int g = 0; g <= 2 * kGrid; ++g) {
+        const double tau = g <= kGrid ? lo * g / kGrid : hi * (g - kGrid) / kGrid;
+        if (tau == 0.0 && g > 0) continue;
+        double top = 0.0; // largest exponent, taken out against overflow
+        for (int j = 0; j < Q; ++j) top = std::max(top, tau * x[j]);
+        double G = 0.0, Gr = 0.0;
+        for (int j = 0; j < Q; ++j) G += W[j] * std::exp(tau * x[j] - top);
+        for (int j = 0; j < q; ++j) Gr += Wr[j] * std::exp(tau * xr[j] - top);
+        if (!(std::fabs(Gr - G) <= kRuleTol * G)) return false;
+    }
+    return true;
+}
+
+// Shortest rule (4, 8, 12, 16, 24 or 32 nodes at most, less than Qpad) that
+// stands for (x, W) by the two conditions above; lo <= 0 <= hi bound tau.
+// Returns its node count, 0 if there is none (the given rule is then swept).
+// *pad: the node count it is padded to.
+int shorter_rule(const double *x, const double *W, int Q, int Qpad, double lo, double hi, double *xr, double *Wr,
+                 int *pad)
+{
+    double spread = 0.0;
+    for (int j = 0; j < Q; ++j) {
+        if (!(W[j] > 0.0)) return 0; // a Gauss rule of the measure needs positive weights
+        spread += W[j] / std::fabs(x[j]);
+    }
+    if (!std::isfinite(lo) || !std::isfinite(hi) || !std::isfinite(spread)) return 0;
+    std::vector<double> y(x, x + Q), v(W, W + Q), al, bt;
+    double mu0 = 0.0;
+    const int most = std::min(Q, 32);
+    if (jacobi_of_measure(y, v, most, al, bt, mu0) != 0) return 0;
+    const int pads[] = {4, 8, 12, 16, 24, 32};
+    int below = 0;
+    for (int p : pads) {
+        if (p >= Qpad) break;
+        for (int q = std::min(p, most); q > below; --q) {
+            gauss_of_jacobi(al, bt, mu0, q, xr, Wr);
+            if (!same_generating_function(x, W, Q, xr, Wr, q, lo, hi)) break; // fewer nodes are no nearer
+            double s = 0.0;
+            bool fine = true;
+            for (int j = 0; j < q; ++j) {
+                s += Wr[j] / std::fabs(xr[j]);
+                fine = fine && Wr[j] > 0.0 && std::isfinite((float)(Wr[j] / (xr[j] * xr[j])));
+            }
+            if (!fine || !(s <= spread)) continue;
+            *pad = p;
+            return q;
+        }
+        below = p;
     }
     return 0;
 }

@@ -82,6 +82,8 @@ def load():
         "lll_set_mapping": (I, [V, I, I]),
         "lll_kernel_ms": (I, [V, _fp, _fp]),
         "lll_build_nig_quadrature": (I, [lll_nig, ctypes.c_double, I, _dp, _dp]),
+        "lll_sweep_rule": (I, [I, _dp, _dp, ctypes.c_double, ctypes.c_double, ctypes.POINTER(I),
+                               ctypes.POINTER(I), _dp, _dp]),
         "lll_mlp_init": (I, [V, I, I, U64]),
         "lll_mlp_init_head": (I, [V, I, I, I, U64]),
         "lll_mlp_shape": (I, [V, ctypes.POINTER(I), ctypes.POINTER(I)]),
@@ -140,6 +142,17 @@ def lll_build_nig_quadrature(alpha, beta, delta, xmax, Q, mu=float("nan")):
     w = np.zeros(Q)
     _check(lib.lll_build_nig_quadrature(lll_nig(alpha, beta, delta, mu), float(xmax), int(Q), _d(x), _d(w)))
     return x, w
+
+
+def lll_sweep_rule(nodes, weights, lo, hi):
+    """The rule the full and Picard sweeps use: (x, w, padded nodes); x is empty where
+    they use the given one (see include/lll.h)."""
+    nodes, weights = _f64(nodes), _f64(weights)
+    x, w = np.zeros(32), np.zeros(32)
+    count, padded = ctypes.c_int(), ctypes.c_int()
+    _check(load().lll_sweep_rule(len(nodes), _d(nodes), _d(weights), float(lo), float(hi), ctypes.byref(count),
+                                 ctypes.byref(padded), _d(x), _d(w)))
+    return x[:count.value].copy(), w[:count.value].copy(), padded.value
 
 
 def lll_init(N, delta, L0, s, lam, driver, nig=(0.0, 0.0, 0.0, float("nan")), nodes=None,
