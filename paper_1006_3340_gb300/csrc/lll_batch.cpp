@@ -158,7 +158,7 @@ int build_schedule(lll_batch *b, int scheme)
         for (const lll_ctx *ic : b->inst) CH = std::min(CH, block_chunk_rates(ic->QR, R, b->n_max, sh.chunk_rows));
         smem = 0;
         for (const lll_ctx *ic : b->inst)
-            smem = std::max(smem, block_kernel_smem(ic->QR, R, b->n_max, b->ns_max, T, CH));
+            smem = std::max(smem, block_kernel_smem(ic->QR, R, b->n_max, T, CH));
     }
     int occ = 0;
     cudaError_t e = (cudaError_t)(b->QK > 0 ? batch_block_prepare(scheme, b->QK, R, smem, T, &occ)

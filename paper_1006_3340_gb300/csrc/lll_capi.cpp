@@ -63,7 +63,7 @@ cudaError_t dalloc(T **p, size_t count)
 void free_all(lll_ctx *c)
 {
     cudaFree(c->d_lam); cudaFree(c->d_x); cudaFree(c->d_W); cudaFree(c->d_w0); cudaFree(c->d_b0);
-    cudaFree(c->d_tab); cudaFree(c->d_row); cudaFree(c->d_Z0); cudaFree(c->d_L0); cudaFree(c->d_c0);
+    cudaFree(c->d_tab); cudaFree(c->d_row); cudaFree(c->d_brow); cudaFree(c->d_Z0); cudaFree(c->d_L0); cudaFree(c->d_c0);
     cudaFree(c->d_strikes); cudaFree(c->d_partials); cudaFree(c->d_sums); cudaFree(c->d_state);
     cudaFree(c->d_snap); cudaFree(c->d_C); cudaFree(c->d_cn); cudaFree(c->d_err);
     cudaFree(c->d_tab_full); cudaFree(c->d_row_full); cudaFree(c->d_cn_full);
@@ -102,7 +102,7 @@ int ensure_full_tables(lll_ctx *ctx)
     if (room) e = cudaMemcpyAsync(row, ctx->d_row, sizeof(float4) * rows, cudaMemcpyDeviceToDevice, ctx->stream);
     if (e == cudaSuccess)
         e = (cudaError_t)launch_tables(ctx->d_lam, ctx->d_x, ctx->d_W, ctx->Q, ctx->d_x, ctx->d_W, ctx->Q, ctx->n,
-                                       ctx->S, ctx->QP, tab, cn, row, ctx->d_C, ctx->stream);
+                                       ctx->S, ctx->QP, ctx->h, tab, cn, row, nullptr, nullptr, ctx->d_C, ctx->stream);
     if (e != cudaSuccess) {
         cudaFree(tab);
         cudaFree(row);
@@ -127,6 +127,8 @@ int use_full_tables(lll_ctx *ctx)
     cudaFree(ctx->d_cn_full);
     ctx->d_tab_full = ctx->d_row_full = nullptr;
     ctx->d_cn_full = nullptr;
+    cudaFree(ctx->d_brow);
+    ctx->d_brow = nullptr;
     ctx->QR = ctx->QP;
     return LLL_OK;
 }
@@ -136,6 +138,7 @@ int launch_plan(const LaunchPlan &plan, const PathArgs &a)
     if (plan.tenor > 0) return launch_tenor_kernel(plan.scheme, plan.qp, plan.tenor, plan.grid, plan.smem, plan.stream, a);
     if (plan.lpp > 1)
         return launch_group_kernel(plan.scheme, plan.qp, plan.lpp, plan.grid, plan.threads, plan.smem, plan.stream, a);
+    if (plan.pipe) return launch_pipe_kernel(plan.scheme, plan.qp, plan.pipe, plan.smem, a.paths, plan.stream, a);
     if (plan.block)
         return launch_block_kernel(plan.scheme, plan.qp, plan.ppt, plan.grid, plan.threads, plan.smem, plan.stream, a);
     return launch_path_kernel(plan.scheme, plan.qp, plan.ppt, plan.grid, plan.threads, plan.smem, plan.stream, a);
@@ -153,7 +156,7 @@ static void block_shape(const lll_ctx *ctx, uint64_t paths, int *R, int *T)
 // Same launch shape and arguments as lll_simulate, with no allocation: the
 // per-block scratch sizes are returned for the caller to place.
 int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, uint64_t seed,
-                LaunchPlan *plan, bool allow_tenor, bool given_rule)
+                LaunchPlan *plan, bool allow_tenor, bool given_rule, bool allow_pipe)
 {
     if (!ctx) return fail(nullptr, LLL_EINVAL, "ctx is NULL");
     if (!plan) return fail(ctx, LLL_EINVAL, "plan is NULL");
@@ -194,11 +197,22 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     if (block) {
         block_shape(ctx, paths, &R, &T);
         CH = block_chunk_rates(ctx->QR, R, ctx->n, ctx->chunk_rows);
-        smem = block_kernel_smem(ctx->QR, R, ctx->n, ctx->ns, T, CH);
+        smem = block_kernel_smem(ctx->QR, R, ctx->n, T, CH);
     }
+    // The pipeline serves a default launch of caplets on few paths.
+    size_t pipe_smem = 0;
+    const int pipe = allow_pipe && block && ctx->threads == 0 && ctx->blocks_per_sm == 0 && ctx->ppt == 0 &&
+                             ctx->chunk_rows == 0 && ctx->product == LLL_PRODUCT_CAPLET
+                         ? pipe_steps(scheme, ctx->QR, ctx->n, ctx->s, ctx->S, (paths + 31) / 32, ctx->sm_count, &pipe_smem)
+                         : 0;
     int occ = 0;
     cudaError_t e;
-    if (G > 0) {
+    if (pipe) {
+        R = 1;
+        T = 32; // paths a block
+        smem = pipe_smem;
+        occ = 1;
+    } else if (G > 0) {
         e = (cudaError_t)tenor_kernel_prepare(scheme, QPk, G, smem, &occ);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "tenor kernel attributes");
     } else if (lpp > 1) {
@@ -217,12 +231,13 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     const int bps = ctx->blocks_per_sm > 0 ? std::min(ctx->blocks_per_sm, occ) : occ;
     const uint64_t per_tile = G > 0 ? (uint64_t)(T / G) : (uint64_t)T * R; // paths per block tile
     const uint64_t tiles = (paths + per_tile - 1) / per_tile;
-    const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)bps * ctx->sm_count);
+    const int grid = (int)(pipe ? tiles : std::min<uint64_t>(tiles, (uint64_t)bps * ctx->sm_count));
     const int nst = (scheme == LLL_PICARD) ? 2 : 1;
     PathArgs a{};
     const bool other = !block && ctx->d_tab_full;
     a.tab = other ? ctx->d_tab_full : ctx->d_tab;
     a.cn = other ? ctx->d_cn_full : ctx->d_cn;
+    a.brow = ctx->d_brow;
     a.row = other ? ctx->d_row_full : ctx->d_row;
     a.Z0 = ctx->d_Z0; a.L0 = ctx->d_L0; a.c0 = ctx->d_c0;
     a.strikes = ctx->d_strikes; a.partials = nullptr; a.state = nullptr;
@@ -242,12 +257,12 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
         a.nig_beta = (float)ctx->nig.beta; a.nig_muh = (float)(ctx->mu * ctx->h);
     }
     plan->args = a;
-    plan->scheme = scheme; plan->qp = block ? ctx->QR : QPk; plan->block = block; plan->ppt = R; plan->lpp = lpp; plan->threads = T; plan->grid = grid;
+    plan->scheme = scheme; plan->qp = block ? ctx->QR : QPk; plan->block = block; plan->pipe = pipe; plan->ppt = R; plan->lpp = lpp; plan->threads = T; plan->grid = grid;
     plan->tenor = G;
     plan->smem = smem;
     // the tenor-parallel kernel keeps its path state in shared memory
-    plan->state_floats_per_block = G > 0 ? 0 : (size_t)R * nst * ctx->n * T;
-    plan->partial_doubles_per_block = (size_t)ctx->n * ctx->ns * 2 * (block ? 2 : 1);
+    plan->state_floats_per_block = G > 0 || pipe ? 0 : (size_t)R * nst * ctx->n * T;
+    plan->partial_doubles_per_block = (size_t)ctx->n * ctx->ns * 2 * (block && !pipe ? 2 : 1);
     plan->n_out = ctx->n * ctx->ns * 2;
     plan->stream = ctx->stream;
     plan->device = ctx->device;
@@ -339,8 +354,9 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     std::vector<double> xs(std::max(Q, 1), 0.0), ws(std::max(Q, 1), 0.0);
     for (int j = 0; j < Q; ++j) { xs[j] = nodes[j]; ws[j] = weights[j]; }
     int QR = QP, Qr = 0;
-    std::vector<double> xw(2 * kMaxQP, 0.0); // the shorter rule: nodes, then weights
+    std::vector<double> xw(2 * kMaxQP + N, 0.0); // the shorter rule: nodes, then weights; then L0
     if (QP > 0) Qr = shorter_rule(xs.data(), ws.data(), Q, QP, down, up, xw.data(), xw.data() + kMaxQP, &QR);
+    std::copy(L0, L0 + N, xw.begin() + 2 * kMaxQP);
     lll_ctx *c = new lll_ctx();
     c->QR = QR;
     c->N = N; c->n = n; c->s = steps_per_period; c->S = S; c->Q = Q; c->QP = QP;
@@ -353,7 +369,7 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     double BN = 1.0;
     for (int m = 0; m < N; ++m) BN /= 1.0 + tenor_delta * L0[m]; // Eq. (i-val) inverted
     c->BN = BN;
-    double *d_short = nullptr; // the shorter rule's nodes and weights, for the tables
+    double *d_short = nullptr; // the shorter rule's nodes and weights and L0, for the tables
 
     auto bail = [&](int code) {
         std::string m = c->err;
@@ -382,7 +398,7 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
               dalloc(&c->d_b0, rows) == cudaSuccess &&
               dalloc(&c->d_tab, rows * std::max(QR / 4, 1)) == cudaSuccess &&
               dalloc(&c->d_cn, std::max(QR, 4)) == cudaSuccess &&
-              (Qr == 0 || dalloc(&d_short, xw.size()) == cudaSuccess) &&
+              (Qr == 0 || (dalloc(&d_short, xw.size()) == cudaSuccess && dalloc(&c->d_brow, rows) == cudaSuccess)) &&
               dalloc(&c->d_row, rows) == cudaSuccess && dalloc(&c->d_C, rows) == cudaSuccess &&
               dalloc(&c->d_Z0, n) == cudaSuccess && dalloc(&c->d_L0, n) == cudaSuccess &&
               dalloc(&c->d_c0, n) == cudaSuccess;
@@ -406,10 +422,10 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     if (Qr > 0)
         INIT_TRY(cudaMemcpyAsync(d_short, xw.data(), sizeof(double) * xw.size(), cudaMemcpyHostToDevice, st));
     const double *xr = Qr > 0 ? d_short : c->d_x, *wr = Qr > 0 ? d_short + kMaxQP : c->d_W;
-    INIT_TRY((cudaError_t)launch_tables(c->d_lam, c->d_x, c->d_W, Q, xr, wr, Qr > 0 ? Qr : Q, n, S, QR, c->d_tab,
-                                        c->d_cn, c->d_row, c->d_C, st));
+    INIT_TRY((cudaError_t)launch_tables(c->d_lam, c->d_x, c->d_W, Q, xr, wr, Qr > 0 ? Qr : Q, n, S, QR, c->h,
+                                        c->d_tab, c->d_cn, c->d_row, c->d_brow, c->d_b0, c->d_C, st));
     INIT_TRY((cudaError_t)launch_frozen_drift(c->d_lam, c->d_x, c->d_W, c->d_w0, n, S, Q, c->c, c->h,
-                                              c->d_b0, c->d_row, st));
+                                              d_short ? d_short + 2 * kMaxQP : nullptr, tenor_delta, c->d_b0, c->d_row, c->d_brow, st));
     // The host vectors above go out of scope: wait for the copies.
     INIT_TRY(cudaStreamSynchronize(st));
 #undef INIT_TRY

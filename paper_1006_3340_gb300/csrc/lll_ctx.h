@@ -25,7 +25,8 @@ struct lll_ctx {
     // device
     double *d_lam = nullptr, *d_x = nullptr, *d_W = nullptr, *d_w0 = nullptr, *d_b0 = nullptr;
     float4 *d_tab = nullptr, *d_row = nullptr; // of the sweeps' rule
-    float *d_cn = nullptr; // [QR]: c_j = W_j / x_j^2
+    float4 *d_brow = nullptr; // rows of the shorter rule (null where the given one is swept)
+    float *d_cn = nullptr; // [QR]: c_j = W_j / x_j^2 (shorter rule: -h c_j)
     // The same for the rule as given (lane groups, the tenor-parallel mapping and
     // training data), built when one of them is first selected; null where the
     // sweeps' rule is the given one.

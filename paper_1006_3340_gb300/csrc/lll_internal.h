@@ -18,7 +18,8 @@ constexpr int kMaxThreads = 256;
 // Arguments of the path kernels (one simulation of one scheme).
 struct PathArgs {
     const float4 *tab;    // [S][n][QP/4]: (E_j .. E_j+3), E_lj = e^{lambda_l(t_k) x_j} - 1
-    const float *cn;      // [QP]: c_j = W_j / x_j^2 (0 on padding nodes)
+    const float *cn;      // [QP]: c_j = W_j / x_j^2, shorter rule: -h c_j (0 on padding nodes)
+    const float4 *brow;   // [S][n]: rows of the shorter rule (lll_sweep.cuh)
     const float4 *row;    // [S][n]: (lambda_l(t_k), K_l(k), D0_l(t_k), b0_l(t_k) * h)
     const float *Z0;      // [n]: log L(0, T_l)
     const float *L0;      // [n]: L(0, T_l)
@@ -60,6 +61,7 @@ struct LaunchPlan {
     PathArgs args;
     int scheme, qp, ppt, lpp, threads, grid; // lpp: lanes per group of paths (1, 2 or 4)
     bool block;                              // time-blocked kernel (lll_paths_block.cu)
+    int pipe;                                // > 0: its pipeline for few paths (lll_paths_pipe.cu), steps per block
     int tenor;                               // > 0: tenor-parallel kernel with this many lanes per path
     size_t smem;
     // scratch per block: path state; payoff sums (block kernel: and their compensations,
@@ -80,16 +82,21 @@ bool path_kernel_supported(int scheme, int QP, int R);
 size_t path_kernel_smem(int QP, int n, int ns, int threads, int chunk_rows);
 
 // Launchers implemented in lll_paths_block.cu (rules with a shorter equivalent,
-// QP = 4, 8, 12, 16, 24 or 32; a batch at each instance's own length up to
+// QP = 4, 8, 12, 16, 20, 24 or 32; a batch at each instance's own length up to
 // QMAX = 8 or 32).
 int block_chunk_rates(int QP, int R, int n, int rows);
-size_t block_kernel_smem(int QP, int R, int n, int ns, int threads, int chunk_rates);
+size_t block_kernel_smem(int QP, int R, int n, int threads, int chunk_rates);
 int block_kernel_prepare(int scheme, int QP, int R, size_t smem, int threads, int *blocks_per_sm);
 int launch_block_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st,
                         const PathArgs &a);
 int batch_block_prepare(int scheme, int QMAX, int R, size_t smem, int threads, int *blocks_per_sm);
 int launch_batch_block_kernel(int scheme, int QMAX, int R, int grid, int threads, size_t smem, cudaStream_t st,
                               const struct BatchArgs &b);
+
+// Launchers implemented in lll_paths_pipe.cu (few paths: 32 paths a block, a
+// pipeline of warps over the rates).
+int pipe_steps(int scheme, int QP, int n, int s, int S, uint64_t tiles, int sms, size_t *smem);
+int launch_pipe_kernel(int scheme, int QP, int B, size_t smem, uint64_t paths, cudaStream_t st, const PathArgs &a);
 
 // Launchers implemented in lll_paths_group.cu (four lanes per group of four paths).
 bool group_kernel_supported(int scheme, int QP, int G);
@@ -118,12 +125,15 @@ int launch_batch_kernel(int scheme, int QP, int R, int grid, int threads, size_t
                         const BatchArgs &b);
 
 // Launchers implemented in lll_tables.cu.
-// xr, Wr, Qr: the rule of the table (padded to QP nodes); x, W, Q: the rule as given, for C.
+// xr, Wr, Qr: the rule of the table (padded to QP nodes); x, W, Q: the rule as
+// given, for C.  brow (null: none): rows of the shorter rule, whose factors cn
+// and constants are scaled by -h; Cs: scratch for them, [S][n].
 int launch_tables(const double *lam, const double *x, const double *W, int Q, const double *xr, const double *Wr,
-                  int Qr, int n, int S, int QP, float4 *tab, float *cn, float4 *row, float *Ctab, cudaStream_t st);
+                  int Qr, int n, int S, int QP, double h, float4 *tab, float *cn, float4 *row, float4 *brow,
+                  double *Cs, float *Ctab, cudaStream_t st);
 int launch_frozen_drift(const double *lam, const double *x, const double *W, const double *w0,
-                        int n, int S, int Q, double c, double h, double *b0, float4 *row,
-                        cudaStream_t st);
+                        int n, int S, int Q, double c, double h, const double *L0, double delta, double *b0,
+                        float4 *row, float4 *brow, cudaStream_t st);
 int launch_finalize(const double *partials, int grid, int n_out, double *sums, cudaStream_t st);
 
 // Implemented in lll_gemm_tc.cu: read and clear the error word of the tcgen05
@@ -139,8 +149,9 @@ namespace lll {
 // allow_tenor: honour the context's tenor-parallel mapping (lll_set_mapping);
 // callers that only need the path arguments of the full scheme pass false.
 // given_rule: plan for the rule as given, not for its shorter equivalent.
+// allow_pipe: the pipeline kernel may be chosen (its grid is the path tiles).
 int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, uint64_t seed,
-                LaunchPlan *plan, bool allow_tenor = true, bool given_rule = false);
+                LaunchPlan *plan, bool allow_tenor = true, bool given_rule = false, bool allow_pipe = true);
 int record_error(lll_ctx *ctx, int code, const char *msg);
 int ensure_full_tables(lll_ctx *ctx); // the tables of the rule as given
 int use_full_tables(lll_ctx *ctx);    // every sweep of this context takes them from now on

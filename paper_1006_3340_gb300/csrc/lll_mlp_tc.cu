@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_kernel(const PathArgs a, c
                         if (!warp_wait(&payb[0], php, abort, g.err)) { ok = false; break; }
                         for (int qs = lane; qs < ns; qs += 32) { // one strike per lane
                             double s1, s2;
-                            block_payoff_sums(a, red + (size_t)buf * 4 * ns * 2, 4, ns, qs, s1, s2);
+                            block_payoff_sums(a.product == 0, red + (size_t)buf * 4 * ns * 2, 4, ns, qs, s1, s2);
                             double *acc = bsum + 4 * ((size_t)(m - 1) * ns + qs);
                             kahan_add(acc + 0, acc + 1, s1);
                             kahan_add(acc + 2, acc + 3, s2);
@@ -864,7 +864,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_vec_kernel(const PathArgs 
                         if (!warp_wait(payb, php, abort, g.err)) { ok = false; break; }
                         for (int qs = lane; qs < ns; qs += 32) { // one strike per lane
                             double s1, s2;
-                            block_payoff_sums(a, red + (size_t)buf * 4 * ns * 2, 4, ns, qs, s1, s2);
+                            block_payoff_sums(a.product == 0, red + (size_t)buf * 4 * ns * 2, 4, ns, qs, s1, s2);
                             double *acc = bsum + 4 * ((size_t)(m - 1) * ns + qs);
                             kahan_add(acc + 0, acc + 1, s1);
                             kahan_add(acc + 2, acc + 3, s2);

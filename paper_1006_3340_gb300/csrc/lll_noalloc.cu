@@ -84,6 +84,9 @@ extern "C" int lll_simulate_noalloc(lll_ctx *ctx, int scheme, uint64_t first_pat
     }
     rc = plan_launch(ctx, scheme, first_path, paths, seed, &plan);
     if (rc != LLL_OK) return rc;
+    if (plan.pipe && sizeof(double) * plan.partial_doubles_per_block * plan.grid > kScratchBytes)
+        rc = plan_launch(ctx, scheme, first_path, paths, seed, &plan, true, false, false);
+    if (rc != LLL_OK) return rc;
     // as many of the launch's blocks as the scratch holds: the blocks loop over
     // the path tiles, and the sums differ only in how FP64 partials are grouped
     while (plan.grid > 1 && state_of(plan, plan.grid) + sizeof(double) * plan.partial_doubles_per_block * plan.grid > kScratchBytes)

@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kMaxThreads, blocks_of(QP, R)) block_kernel(co
     constexpr int B = steps_of(QP, R), NST = (SCHEME == PICARD) ? 2 : 1;
     const int T = blockDim.x, tid = threadIdx.x;
     const BlockSmem sm = block_carve(smem_raw, QP, B, R, a.n, T, a.chunk_rows);
-    for (int e = tid; e < a.n; e += T) sm.c0[e] = a.c0[e];
+    for (int e = tid; e < a.n; e += T) sm.c0[e] = -1.4426950408889634f * a.c0[e];
     for (int e = tid; e < QP; e += T) reinterpret_cast<float *>(sm.cn)[e] = a.cn[e];
     State<NST * R> *st = reinterpret_cast<State<NST * R> *>(a.state) + (size_t)blockIdx.x * a.n * T + tid;
     const size_t nout = (size_t)a.n * a.ns * 2;
@@ -56,7 +56,7 @@ __device__ __forceinline__ void batch_item(const PathArgs &a, unsigned char *sme
     constexpr int B = steps_of(QP, R), NST = (SCHEME == PICARD) ? 2 : 1;
     const int T = blockDim.x, tid = threadIdx.x;
     const BlockSmem sm = block_carve(smem, QP, B, R, a.n, T, a.chunk_rows);
-    for (int e = tid; e < a.n; e += T) sm.c0[e] = a.c0[e];
+    for (int e = tid; e < a.n; e += T) sm.c0[e] = -1.4426950408889634f * a.c0[e];
     for (int e = tid; e < QP; e += T) reinterpret_cast<float *>(sm.cn)[e] = a.cn[e];
     State<NST * R> *st = reinterpret_cast<State<NST * R> *>(state) + tid;
     for (uint32_t t = tiles.x; t < tiles.y; ++t)
@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(kMaxThreads, blocks_of(QMAX > 8 ? 24 : 8, R)) 
             if constexpr (QMAX > 8) {
                 if (sa.qr == 12) batch_item<SCHEME, 12, R>(sa, smem_raw, state, tr, acc, comp);
                 else if (sa.qr == 16) batch_item<SCHEME, 16, R>(sa, smem_raw, state, tr, acc, comp);
+                else if (sa.qr == 20) batch_item<SCHEME, 20, R>(sa, smem_raw, state, tr, acc, comp);
                 else if (sa.qr == 24) batch_item<SCHEME, 24, R>(sa, smem_raw, state, tr, acc, comp);
                 else batch_item<SCHEME, 32, R>(sa, smem_raw, state, tr, acc, comp);
             }
@@ -112,6 +113,7 @@ KernelFn pick_qp(int QP)
     case 8: return block_kernel<SCHEME, 8, R>;
     case 12: return block_kernel<SCHEME, 12, R>;
     case 16: return block_kernel<SCHEME, 16, R>;
+    case 20: return block_kernel<SCHEME, 20, R>;
     case 24: return block_kernel<SCHEME, 24, R>;
     case 32: return block_kernel<SCHEME, 32, R>;
     default: return nullptr;
@@ -154,9 +156,9 @@ int block_chunk_rates(int QP, int R, int n, int rows)
     return max(1, min(rows > 0 ? min(rows, n) : n, fit));
 }
 
-size_t block_kernel_smem(int QP, int R, int n, int ns, int threads, int chunk_rates)
+size_t block_kernel_smem(int QP, int R, int n, int threads, int chunk_rates)
 {
-    return block_smem_bytes(QP, steps_of(QP, R), R, n, ns, threads, chunk_rates);
+    return block_smem_bytes(QP, steps_of(QP, R), R, n, threads, chunk_rates);
 }
 
 int block_kernel_prepare(int scheme, int QP, int R, size_t smem, int threads, int *blocks_per_sm)

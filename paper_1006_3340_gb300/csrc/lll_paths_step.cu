@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kSpT) sp_sweep(const PathArgs a, int Pc, const
     const size_t r0 = (size_t)k * n + (imin - 1);
     for (int e = threadIdx.x; e < live * Q4; e += kSpT) tab[e] = a.tab[r0 * Q4 + e];
     for (int e = threadIdx.x; e < live; e += kSpT) {
-        row[e] = a.row[r0 + e];
+        row[e] = SHORT ? a.brow[r0 + e] : a.row[r0 + e];
         c0[e] = a.c0[imin - 1 + e];
     }
     for (int e = threadIdx.x; e < QP; e += kSpT) reinterpret_cast<float *>(cn)[e] = a.cn[e];
@@ -109,16 +109,16 @@ __global__ void __launch_bounds__(kSpT) sp_sweep(const PathArgs a, int Pc, const
     float yn = Yk[(size_t)(n - 1) * Pc];
     for (int i = n; i >= imin; --i) {
         const int r = i - imin;
-        const float4 rc = row[r]; // lambda, K, D0, b0 h
-        const float w = weight_of(c0[r] + rc.z + yn);
+        const float4 rc = row[r];
+        const float w = SHORT ? sweep_weight(rc.y, yn) : weight_of(c0[r] + rc.z + yn);
         if (i > imin) yn = Yk[(size_t)(i - 2) * Pc];
         const float4 *tr = tab + (size_t)r * Q4;
-        float A;
+        float bh;
         if constexpr (SHORT) {
             float4 E[Q4];
 #pragma unroll
             for (int j = 0; j < Q4; ++j) E[j] = tr[j];
-            A = sweep_dot<QP>(E, P, rc.y);
+            bh = sweep_dot<QP>(E, P) + rc.z;
             sweep_grow<QP>(E, P, w);
         } else {
             const float2 w2 = make_float2(w, w);
@@ -136,9 +136,9 @@ __global__ void __launch_bounds__(kSpT) sp_sweep(const PathArgs a, int Pc, const
                 }
             }
             const float2 s2 = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
-            A = rc.y + (s2.x + s2.y);
+            bh = -(rc.y + (s2.x + s2.y)) * h;
         }
-        Bh[((size_t)k * n + (i - 1)) * Pc + lp] = -A * h;
+        Bh[((size_t)k * n + (i - 1)) * Pc + lp] = bh;
     }
 }
 
@@ -199,19 +199,24 @@ __global__ void __launch_bounds__(kSpT) sp_payoff(const PathArgs a, int Pc, uint
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lp = blockIdx.x * kSpT + threadIdx.x;
     const bool active = lp < Pc && chunk_first + lp < a.paths;
+    auto z = [&](int i) { return Zm[((size_t)(m - 1) * n + (i - 1)) * Pc + lp]; };
     double Pp = 1.0, Sp = 1.0;
     float Lm = 0.0f;
+    float4 mv = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (lp < Pc) {
-        auto z = [&](int i) { return Zm[((size_t)(m - 1) * n + (i - 1)) * Pc + lp]; };
-        if constexpr (SHORT) maturity_factors(a, m, z, Pp, Sp, Lm);
+        if constexpr (SHORT) mv = maturity_values(a, m, z);
         else maturity_products(a, m, z, Pp, Sp, Lm);
     }
     for (int q = 0; q < ns; ++q) {
         const float K = a.strikes[(size_t)(m - 1) * ns + q];
         const size_t slot = (size_t)warp * ns + q;
-        if (a.product == 0) {
-            const float v[1] = {active ? caplet_payoff(a, (float)Pp, Lm, K) : 0.0f};
-            const float4 r = caplet_warp_sums(v);
+        if (SHORT || a.product == 0) {
+            DFloat v{0.0f, 0.0f};
+            if (active) {
+                if constexpr (SHORT) v = payoff_of(a.product, mv, K);
+                else v.hi = caplet_payoff(a, (float)Pp, Lm, K);
+            }
+            const float4 r = caplet_warp_sums_inline(v, SHORT ? df_square_pair(v) : df_square(v.hi));
             if (lane == 0) reinterpret_cast<float4 *>(red)[slot] = r;
         } else {
             const double v = active ? payoff(a, Pp, Sp, Lm, K) : 0.0;
@@ -225,7 +230,11 @@ __global__ void __launch_bounds__(kSpT) sp_payoff(const PathArgs a, int Pc, uint
     __syncthreads();
     if (threadIdx.x < ns) {
         double s1, s2;
-        block_payoff_sums(a, red, kSpT / 32, ns, threadIdx.x, s1, s2);
+        block_payoff_sums(a.product == 0 || SHORT, red, kSpT / 32, ns, threadIdx.x, s1, s2);
+        if (SHORT) {
+            s1 *= payoff_scale(a);
+            s2 *= payoff_scale(a) * payoff_scale(a);
+        }
         double *out = partials + ((size_t)(block0 + blockIdx.x) * n + (m - 1)) * ns * 2 + 2 * threadIdx.x;
         out[0] = s1;
         out[1] = s2;
@@ -241,6 +250,7 @@ SweepFn pick_sweep(int QP, bool shorter)
     case 8: return shorter ? sp_sweep<8, true> : nullptr;
     case 12: return shorter ? sp_sweep<12, true> : nullptr;
     case 16: return shorter ? sp_sweep<16, true> : sp_sweep<16, false>;
+    case 20: return shorter ? sp_sweep<20, true> : nullptr;
     case 24: return shorter ? sp_sweep<24, true> : nullptr;
     case 32: return shorter ? sp_sweep<32, true> : sp_sweep<32, false>;
     case 64: return shorter ? nullptr : sp_sweep<64, false>;

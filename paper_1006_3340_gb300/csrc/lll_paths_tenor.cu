@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(kTenorThreads) tenor_kernel(const PathArgs a, 
                 __syncthreads();
                 if (tid < ns) {
                     double s1, s2;
-                    block_payoff_sums(a, sm.red, T >> 5, ns, tid, s1, s2);
+                    block_payoff_sums(a.product == 0, sm.red, T >> 5, ns, tid, s1, s2);
                     double *acc = sm.bsum + 4 * ((size_t)(m - 1) * ns + tid);
                     kahan_add(acc + 0, acc + 1, s1);
                     kahan_add(acc + 2, acc + 3, s2);

@@ -211,7 +211,7 @@ static bool same_generating_function(const double *x, const double *W, int Q, co
     return true;
 }
 
-// Shortest rule (4, 8, 12, 16, 24 or 32 nodes at most, less than Qpad) that
+// Shortest rule (4, 8, 12, 16, 20, 24 or 32 nodes at most, less than Qpad) that
 // stands for (x, W) by the two conditions above; lo <= 0 <= hi bound tau.
 // Returns its node count, 0 if there is none (the given rule is then swept).
 // *pad: the node count it is padded to.
@@ -228,7 +228,7 @@ int shorter_rule(const double *x, const double *W, int Q, int Qpad, double lo, d
     double mu0 = 0.0;
     const int most = std::min(Q, 32);
     if (jacobi_of_measure(y, v, most, al, bt, mu0) != 0) return 0;
-    const int pads[] = {4, 8, 12, 16, 24, 32};
+    const int pads[] = {4, 8, 12, 16, 20, 24, 32};
     int below = 0;
     for (int p : pads) {
         if (p >= Qpad) break;

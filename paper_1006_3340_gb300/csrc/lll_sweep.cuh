@@ -56,19 +56,36 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// A_i = K_i + sum_j E_ij P~_j for one row E of QP nodes (P~ as pairs).
+// Rows of the sweeps' rule: (lambda, x, K', 0) with x = -log2(e) (log(delta
+// L(0,T_i)) + D0), the constant part of the weight's exponent under Picard.
+// The node factors are scaled, -h c_j, so that the dot product and K' together
+// are the drift's contribution b_i h to the step itself; K' closes the sum at
+// zero weights (P~_j = -h c_j) as FP32 forms it, -h C_i less that sum, so that
+// its rounding leaves no bias common to all paths (lll_tables.cu).
+//
+// sum_j E_ij P~_j for one row E of QP nodes (P~ as pairs).
 template <int QP>
-__device__ __forceinline__ float sweep_dot(const float4 (&E)[QP / 4], const float2 (&P)[QP / 2], float K)
+__device__ __forceinline__ float sweep_dot(const float4 (&E)[QP / 4], const float2 (&P)[QP / 2])
 {
-    float2 a = make_float2(K, 0.0f), b = make_float2(0.0f, 0.0f);
+    float2 a, b;
 #pragma unroll
     for (int j4 = 0; j4 < QP / 4; ++j4) {
-        a = __ffma2_rn(make_float2(E[j4].x, E[j4].y), P[2 * j4], a);
-        if (j4 == 0) b = __fmul2_rn(make_float2(E[j4].z, E[j4].w), P[2 * j4 + 1]);
-        else b = __ffma2_rn(make_float2(E[j4].z, E[j4].w), P[2 * j4 + 1], b);
+        const float2 e0 = make_float2(E[j4].x, E[j4].y), e1 = make_float2(E[j4].z, E[j4].w);
+        a = j4 == 0 ? __fmul2_rn(e0, P[0]) : __ffma2_rn(e0, P[2 * j4], a);
+        b = j4 == 0 ? __fmul2_rn(e1, P[1]) : __ffma2_rn(e1, P[2 * j4 + 1], b);
     }
     a = __fadd2_rn(a, b);
     return a.x + a.y;
+}
+
+// w = delta L / (1 + delta L) = 1 / (1 + 2^(x - log2(e) z)) for the offset z of
+// log L from x's constant (approximate ex2 and rcp, as weight_of).
+__device__ __forceinline__ float sweep_weight(float x, float z)
+{
+    float e, r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fmaf(-1.4426950408889634f, z, x)));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
+    return r;
 }
 
 // P~_j *= 1 + w E_ij.
@@ -87,21 +104,22 @@ __device__ __forceinline__ void sweep_grow(const float4 (&E)[QP / 4], float2 (&P
 
 // Shared memory of a block: table rows of CH rates for B steps, double-buffered.
 struct BlockSmem {
-    float4 *tab;  // [2][B][CH][QP/4]
-    float4 *row;  // [2][B][CH]: lambda, K, D0, b0 h
-    float2 *cn;   // [QP/2]: c_j
-    float *c0;    // [n]: log(delta L(0, T_l))
+    float4 *tab;  // [2][CH][B][QP/4]: the B steps of a rate side by side, at immediate offsets
+    float4 *row;  // [2][CH][B]
+    float2 *cn;   // [QP/2]: -h c_j
+    float *c0;    // [n]: -log2(e) log(delta L(0, T_l))
     float *dh;    // [B][R][T]: increments on their way to registers
-    double *red;  // [2][warps][ns] 16-byte slots (block_payoff_sums), by maturity parity
+    float4 *pay;  // [R][T]: maturity_values of the block's paths
+    float4 *part; // [T]: payoff sums of slices of them
 };
 
 __host__ __device__ inline size_t up16(size_t v) { return (v + 15) & ~size_t(15); }
 
 // Bytes of each part, in the order of BlockSmem.
-__host__ __device__ inline size_t block_smem_bytes(int QP, int B, int R, int n, int ns, int T, int CH)
+__host__ __device__ inline size_t block_smem_bytes(int QP, int B, int R, int n, int T, int CH)
 {
     return 2 * (size_t)B * CH * QP * 4 + 2 * (size_t)B * CH * 16 + up16((size_t)QP * 4) + up16((size_t)n * 4) +
-           up16((size_t)B * R * T * 4) + 2 * (size_t)(T / 32) * ns * 16;
+           up16((size_t)B * R * T * 4) + (size_t)(R + 1) * T * 16;
 }
 
 __device__ inline BlockSmem block_carve(unsigned char *p, int QP, int B, int R, int n, int T, int CH)
@@ -117,7 +135,8 @@ __device__ inline BlockSmem block_carve(unsigned char *p, int QP, int B, int R, 
     p += up16((size_t)n * 4);
     s.dh = reinterpret_cast<float *>(p);
     p += up16((size_t)B * R * T * 4);
-    s.red = reinterpret_cast<double *>(p);
+    s.pay = reinterpret_cast<float4 *>(p);
+    s.part = s.pay + (size_t)R * T;
     return s;
 }
 
@@ -137,12 +156,15 @@ __device__ __forceinline__ void stage_rows(const PathArgs &a, const BlockSmem &s
     const int ibot = max(at.m, itop - CH + 1);
     const int cnt = itop - ibot + 1;
     const int nb = min(B, a.s - at.kb);
-    size_t r0 = ((size_t)(at.m - 1) * a.s + at.kb) * n + (ibot - 1);
+    const size_t r0 = ((size_t)(at.m - 1) * a.s + at.kb) * n + (ibot - 1);
     float4 *dt = sm.tab + (size_t)b * B * CH * Q4, *dr = sm.row + (size_t)b * B * CH;
-    for (int s = 0; s < nb; ++s, r0 += n, dt += (size_t)CH * Q4, dr += CH) {
-        const float4 *src = a.tab + r0 * Q4;
-        for (int e = threadIdx.x; e < cnt * Q4; e += blockDim.x) cp_async16(dt + e, src + e);
-        for (int e = threadIdx.x; e < cnt; e += blockDim.x) cp_async16(dr + e, a.row + r0 + e);
+    for (int e = threadIdx.x; e < cnt * B * Q4; e += blockDim.x) {
+        const int j = e % Q4, s = e / Q4 % B, r = e / (Q4 * B);
+        if (s < nb) cp_async16(dt + e, a.tab + (r0 + (size_t)s * n + r) * Q4 + j);
+    }
+    for (int e = threadIdx.x; e < cnt * B; e += blockDim.x) {
+        const int s = e % B, r = e / B;
+        if (s < nb) cp_async16(dr + e, a.brow + r0 + (size_t)s * n + r);
     }
 }
 
@@ -154,65 +176,69 @@ struct alignas(4 * N) State {
 };
 
 // Payoffs of the block's paths at T_m into the block's FP64 Kahan sums
-// acc[(m-1) ns + q][2] with compensations comp[..][2].
+// acc[(m-1) ns + q][2] with compensations comp[..][2].  Every thread leaves its
+// paths' values in shared memory; then thread (strike q, slice g) adds up the
+// payoffs of every G-th path in double-float pairs, and thread q the G slices.
+// (Reducing each strike over the warp's lanes instead, by shuffles, took 0.25
+// of 2.08 ms on the N = 40 workload and three times the latency.)
 template <int NST, int R>
 __device__ __forceinline__ void block_maturity(const PathArgs &a, const BlockSmem &sm, const State<NST * R> *st, int T,
                                                int m, const uint64_t (&lp)[R], double *acc, double *comp, bool first)
 {
-    const int n = a.n, ns = a.ns, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = T >> 5;
-    double *red = sm.red + (size_t)(m & 1) * nw * ns * 2;
-    double Pp[R], Sp[R];
-    float Lm[R];
-    auto z_of = [&](int u, int i) {
-        const State<NST * R> v = st[(size_t)(i - 1) * T];
-        float z = v.v[NST * u];
-        if constexpr (NST == 2) z += v.v[2 * u + 1];
-        return z;
-    };
+    const int n = a.n, ns = a.ns, tid = threadIdx.x;
 #pragma unroll
     for (int u = 0; u < R; ++u) {
-        maturity_factors(a, m, [&](int i) { return z_of(u, i); }, Pp[u], Sp[u], Lm[u]);
+        auto z = [&](int i) {
+            const State<NST * R> v = st[(size_t)(i - 1) * T];
+            float x = v.v[NST * u];
+            if constexpr (NST == 2) x += v.v[2 * u + 1];
+            return x;
+        };
+        float4 v = maturity_values(a, m, z);
+        if (lp[u] >= a.paths) v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        sm.pay[u * T + tid] = v;
         if (a.snap != nullptr && lp[u] < a.paths && lp[u] % a.snap_stride == 0 && lp[u] / a.snap_stride < a.n_snap)
             for (int i = n; i >= m; --i)
-                a.snap[((size_t)(m - 1) * n + (i - 1)) * a.snap_pitch + lp[u] / a.snap_stride] = z_of(u, i) + a.Z0[i - 1];
-    }
-    for (int q = 0; q < ns; ++q) {
-        const float K = a.strikes[(size_t)(m - 1) * ns + q];
-        const size_t slot = (size_t)warp * ns + q;
-        if (a.product == 0) {
-            float v[R];
-#pragma unroll
-            for (int u = 0; u < R; ++u) v[u] = lp[u] < a.paths ? caplet_payoff(a, (float)Pp[u], Lm[u], K) : 0.0f;
-            const float4 r = caplet_warp_sums(v);
-            if (lane == 0) reinterpret_cast<float4 *>(red)[slot] = r;
-        } else {
-            double pay = 0.0, pay2 = 0.0;
-#pragma unroll
-            for (int u = 0; u < R; ++u) {
-                const double v = lp[u] < a.paths ? payoff(a, Pp[u], Sp[u], Lm[u], K) : 0.0;
-                pay += v;
-                pay2 += v * v;
-            }
-            const double s1 = warp_sum(pay), s2 = warp_sum(pay2);
-            if (lane == 0) {
-                red[2 * slot + 0] = s1;
-                red[2 * slot + 1] = s2;
-            }
-        }
+                a.snap[((size_t)(m - 1) * n + (i - 1)) * a.snap_pitch + lp[u] / a.snap_stride] = z(i) + a.Z0[i - 1];
     }
     __syncthreads();
-    for (int q = tid; q < ns; q += T) {
-        double s1, s2;
-        block_payoff_sums(a, red, nw, ns, q, s1, s2);
-        const size_t e = 2 * ((size_t)(m - 1) * ns + q);
-        if (first) {
-            acc[e] = s1;
-            acc[e + 1] = s2;
-            comp[e] = comp[e + 1] = 0.0;
-        } else {
-            kahan_add(acc + e, comp + e, s1);
-            kahan_add(acc + e + 1, comp + e + 1, s2);
+    for (int q0 = 0; q0 < ns; q0 += T) { // one pass unless there are more strikes than threads
+        const int nq = min(ns - q0, T);
+        // slices: about the square root of the paths, which balances the two sums
+        const int G = min(T / nq, R * T >= 256 ? 16 : R * T >= 64 ? 8 : 6);
+        const int q = tid % nq, g = tid / nq;
+        if (g < G) {
+            const float K = a.strikes[(size_t)(m - 1) * ns + q0 + q];
+            DFloat s1{0.0f, 0.0f}, s2{0.0f, 0.0f};
+            for (int p = g; p < R * T; p += G) {
+                const DFloat v = payoff_of(a.product, sm.pay[p], K);
+                s1 = df_add(s1, v);
+                s2 = df_add(s2, df_square_pair(v));
+            }
+            sm.part[g * nq + q] = make_float4(s1.hi, s1.lo, s2.hi, s2.lo);
         }
+        __syncthreads();
+        if (tid < nq) {
+            float4 r = sm.part[tid];
+            DFloat x{r.x, r.y}, y{r.z, r.w};
+            for (int k = 1; k < G; ++k) {
+                r = sm.part[k * nq + tid];
+                x = df_add(x, DFloat{r.x, r.y});
+                y = df_add(y, DFloat{r.z, r.w});
+            }
+            const double c = payoff_scale(a);
+            const double v1 = c * ((double)x.hi + (double)x.lo), v2 = c * c * ((double)y.hi + (double)y.lo);
+            const size_t e = 2 * ((size_t)(m - 1) * ns + q0 + tid);
+            if (first) {
+                acc[e] = v1;
+                acc[e + 1] = v2;
+                comp[e] = comp[e + 1] = 0.0;
+            } else {
+                kahan_add(acc + e, comp + e, v1);
+                kahan_add(acc + e + 1, comp + e + 1, v2);
+            }
+        }
+        if (q0 + T < ns) __syncthreads();
     }
 }
 
@@ -225,28 +251,24 @@ __device__ __forceinline__ void sweep_chunk(const PathArgs &a, const BlockSmem &
 {
     constexpr int Q4 = QP / 4, NST = (SCHEME == PICARD) ? 2 : 1;
     const int CH = a.chunk_rows;
-    const float4 *tb = sm.tab + (size_t)buf * B * CH * Q4;
-    const float4 *rb = sm.row + (size_t)buf * B * CH;
-    const float h = a.h;
+    const float4 *tr = sm.tab + ((size_t)buf * CH + (itop - ibot)) * (B * Q4);
+    const float4 *rr = sm.row + ((size_t)buf * CH + (itop - ibot)) * B;
     State<NST * R> next = st[(size_t)(itop - 1) * T];
-    for (int i = itop; i >= ibot; --i) {
-        const int r = i - ibot;
+    for (int i = itop; i >= ibot; --i, tr -= B * Q4, rr -= B) {
         State<NST * R> cur = next;
         if (i > ibot) next = st[(size_t)(i - 2) * T];
         const float c0 = sm.c0[i - 1];
 #pragma unroll
         for (int b = 0; b < B; ++b) {
             if (TAIL && b >= nb) break;
-            const float4 rc = rb[b * CH + r]; // lambda, K, D0, b0 h
-            const float4 *tr = tb + (size_t)(b * CH + r) * Q4;
+            const float4 rc = rr[b];
             float4 E[Q4];
 #pragma unroll
-            for (int j = 0; j < Q4; ++j) E[j] = tr[j];
-            const float cx = SCHEME == PICARD ? c0 + rc.z : c0;
+            for (int j = 0; j < Q4; ++j) E[j] = tr[b * Q4 + j];
 #pragma unroll
             for (int q = 0; q < R; ++q) {
-                const float w = weight_of(cx + cur.v[NST * q]);
-                const float bh = -sweep_dot<QP>(E, P[q][b], rc.y) * h;
+                const float w = sweep_weight(SCHEME == PICARD ? rc.y : c0, cur.v[NST * q]);
+                const float bh = sweep_dot<QP>(E, P[q][b]) + rc.z;
                 if constexpr (SCHEME == PICARD) {
                     cur.v[2 * q] = fmaf(rc.x, dH[q][b], cur.v[2 * q]); // int lambda dH
                     cur.v[2 * q + 1] += bh;                            // Picard drift integral
@@ -287,8 +309,9 @@ __device__ __forceinline__ void block_tile(const PathArgs &a, const BlockSmem &s
         const int nch = (n - m + CH) / CH; // ceil((n - m + 1) / CH)
         for (int kb = 0; kb < s; kb += B) {
             const int k0 = (m - 1) * s + kb, nb = min(B, s - kb);
-            // the draws stay one loop body (their code is long); registers take them afterwards
-#pragma unroll 1
+            // the draws stay a loop (their code is long), two at a time to overlap their
+            // latencies; registers take them afterwards
+#pragma unroll 2
             for (int e = 0; e < nb * R; ++e) {
                 const int b = e / R, q = e % R;
                 sm.dh[(size_t)e * T + tid] =

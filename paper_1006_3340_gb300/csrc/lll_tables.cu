@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "lll_internal.h"
+#include "lll_sweep.cuh"
 
 namespace lll {
 namespace {
@@ -25,14 +26,14 @@ namespace {
 // rates already fixed hold lambda alone, nothing reads the rest), and the
 // warps of a block and the blocks are independent.
 __global__ void tables_kernel(const double *lam, const double *x, const double *W, int Q, const double *xr,
-                              const double *Wr, int Qr, int n, int s, int QP, float4 *tab, float *cn, float4 *row,
-                              float *Ctab)
+                              const double *Wr, int Qr, int n, int s, int QP, double scale, float4 *tab, float *cn,
+                              float4 *row, float4 *brow, double *Cs, float *Ctab)
 {
     const int k = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int imin = k / s + 1;
     if (k == 0)
         for (int j = threadIdx.x; j < QP; j += blockDim.x)
-            cn[j] = (j < Qr) ? (float)(Wr[j] / (xr[j] * xr[j])) : 0.0f;
+            cn[j] = (j < Qr) ? (float)(scale * (Wr[j] / (xr[j] * xr[j]))) : 0.0f;
     for (int i = warp + 1; i <= n; i += nw) {
         const size_t idx = (size_t)k * n + (i - 1);
         const double li = lam[idx];
@@ -47,7 +48,7 @@ __global__ void tables_kernel(const double *lam, const double *x, const double *
             float e = 0.0f;
             if (i >= imin && j < Qr) {
                 e = (float)expm1(li * xr[j]);
-                sa += (double)__fmul_rn(e, (float)(Wr[j] / (xr[j] * xr[j])));
+                sa += (double)__fmul_rn(e, (float)(scale * (Wr[j] / (xr[j] * xr[j]))));
             }
             out[j] = e;
         }
@@ -57,10 +58,31 @@ __global__ void tables_kernel(const double *lam, const double *x, const double *
             sa += __shfl_xor_sync(0xffffffffu, sa, o);
         }
         if (lane == 0) {
-            *reinterpret_cast<float2 *>(&row[idx]) = make_float2((float)li, (float)(C - sa));
+            *reinterpret_cast<float2 *>(&row[idx]) = make_float2((float)li, (float)(C - sa / scale));
+            if (brow) {
+                brow[idx].x = (float)li;
+                brow[idx].w = 0.0f;
+                Cs[idx] = scale * C;
+            }
             Ctab[idx] = (float)C;
         }
     }
+}
+
+// K' = -h C less the dot product at zero weights, formed by the sweeps' own FP32
+// operations.  One thread a row.
+template <int QP>
+__global__ void close_kernel(const float4 *tab, const float *cn, const double *Cs, int rows, float4 *brow)
+{
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= rows) return;
+    float4 E[QP / 4];
+    float2 P[QP / 2];
+#pragma unroll
+    for (int j = 0; j < QP / 4; ++j) E[j] = tab[(size_t)r * (QP / 4) + j];
+#pragma unroll
+    for (int j = 0; j < QP / 2; ++j) P[j] = reinterpret_cast<const float2 *>(cn)[j];
+    brow[r].z = (float)(Cs[r] - (double)sweep_dot<QP>(E, P));
 }
 
 // One block per step, one thread per node carrying its product P_j down the
@@ -107,12 +129,14 @@ __global__ void frozen_drift_kernel(const double *lam, const double *x, const do
 
 // Thread per rate: the running integral over the steps it lives, eight steps'
 // loads ahead of their additions.
-__global__ void prefix_kernel(const double *b0, int n, int s, double h, float4 *row)
+__global__ void prefix_kernel(const double *b0, int n, int s, double h, const double *L0, double delta, float4 *row,
+                              float4 *brow)
 {
     constexpr int U = 8;
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n) return;
     const int K = (l + 1) * s;
+    const double c0 = brow ? log(delta * L0[l + 1]) : 0.0;
     double D = 0.0;
     for (int k0 = 0; k0 < K; k0 += U) {
         double b[U];
@@ -124,6 +148,7 @@ __global__ void prefix_kernel(const double *b0, int n, int s, double h, float4 *
             const double bh = b[u] * h;
             float2 *out = reinterpret_cast<float2 *>(&row[(size_t)(k0 + u) * n + l].z);
             *out = make_float2((float)D, (float)bh);
+            if (brow) brow[(size_t)(k0 + u) * n + l].y = (float)(-1.4426950408889634 * (c0 + D));
             D += bh;
         }
     }
@@ -193,22 +218,37 @@ int batch_finalize(const double *partials, const size_t *seg_off, const int *ins
 }
 
 int launch_tables(const double *lam, const double *x, const double *W, int Q, const double *xr, const double *Wr,
-                  int Qr, int n, int S, int QP, float4 *tab, float *cn, float4 *row, float *Ctab, cudaStream_t st)
+                  int Qr, int n, int S, int QP, double h, float4 *tab, float *cn, float4 *row, float4 *brow,
+                  double *Cs, float *Ctab, cudaStream_t st)
 {
     const int warps = n < 8 ? n : 8;
-    tables_kernel<<<S, 32 * warps, 0, st>>>(lam, x, W, Q, xr, Wr, Qr, n, S / n, QP, tab, cn, row, Ctab);
+    tables_kernel<<<S, 32 * warps, 0, st>>>(lam, x, W, Q, xr, Wr, Qr, n, S / n, QP, brow ? -h : 1.0, tab, cn, row,
+                                            brow, Cs, Ctab);
+    if (brow) {
+        const int rows = S * n, blocks = (rows + 127) / 128;
+        switch (QP) {
+        case 4: close_kernel<4><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
+        case 8: close_kernel<8><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
+        case 12: close_kernel<12><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
+        case 16: close_kernel<16><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
+        case 20: close_kernel<20><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
+        case 24: close_kernel<24><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
+        case 32: close_kernel<32><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
+        default: return (int)cudaErrorInvalidValue;
+        }
+    }
     return (int)cudaGetLastError();
 }
 
 int launch_frozen_drift(const double *lam, const double *x, const double *W, const double *w0,
-                        int n, int S, int Q, double c, double h, double *b0, float4 *row,
-                        cudaStream_t st)
+                        int n, int S, int Q, double c, double h, const double *L0, double delta, double *b0,
+                        float4 *row, float4 *brow, cudaStream_t st)
 {
     const int threads = Q <= 0 ? 32 : (Q + 31) / 32 * 32;
     frozen_drift_kernel<<<S, threads, 0, st>>>(lam, x, W, w0, n, S / n, Q, c, b0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return (int)e;
-    prefix_kernel<<<(n + 31) / 32, 32, 0, st>>>(b0, n, S / n, h, row);
+    prefix_kernel<<<(n + 31) / 32, 32, 0, st>>>(b0, n, S / n, h, L0, delta, row, brow);
     return (int)cudaGetLastError();
 }
 

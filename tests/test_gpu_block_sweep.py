@@ -48,7 +48,7 @@ def _check(lll, wl, x, W, scheme, paths, launch):
 
 # (N, s, volatility level, padded nodes expected): steeper volatilities need longer rules
 SHAPES = [(2, 1, 0.12, 4), (3, 7, 0.12, 4), (5, 9, 0.12, 4), (41, 3, 0.05, 8), (34, 5, 0.15, 12), (40, 2, 0.24, 16),
-          (60, 3, 0.27, 24)]
+          (60, 3, 0.27, 20), (70, 2, 0.28, 24)]
 
 
 @pytest.mark.parametrize("N,s,level,padded", SHAPES)
@@ -101,3 +101,29 @@ def test_batch_of_rule_lengths(lll, levels, scheme, ppt):
     for q, (wl, x, W) in enumerate(inst):
         ref = ora.simulate(ora.OracleModel(wl, x, W), SCHEMES[scheme], seed=11, inst=q)
         assert np.abs(got[q] - ref["price"]).max() <= 1e-7, q
+
+
+# The pipeline for few paths (lll_paths_pipe.cu): the same arithmetic, so its
+# recorded log-rates equal the block kernel's bit for bit, and its sums differ
+# only by their double-float order.
+@pytest.mark.parametrize("N,s,level", [(2, 1, 0.12), (4, 8, 0.12), (9, 5, 0.1), (10, 10, 0.12), (18, 3, 0.12),
+                                       (41, 8, 0.05), (34, 5, 0.15), (40, 3, 0.24), (120, 4, 0.02), (60, 4, 0.27),
+                                       (70, 2, 0.28)])
+@pytest.mark.parametrize("scheme", ["full", "picard"])
+@pytest.mark.parametrize("paths", [1, 70, 5000])
+def test_pipeline_equals_block_kernel(lll, N, s, level, scheme, paths):
+    wl = workloads.tiny(N=N, s=s, Q=64)
+    wl = dataclasses.replace(wl, lam=np.full_like(wl.lam, level), L0=np.full(N, 0.03))
+    x, W = quadrature.rule_for(wl)
+    got = []
+    for launch in ((0, 0, 0, 0, 0), (64, 0, 0, 1, 1)):
+        sim = lll.LevyLibor(wl, x, W)
+        try:
+            sim.set_launch(*launch)
+            sim.simulate(scheme, paths=paths, snapshots=min(paths, 200), snapshot_stride=7 if paths > 1400 else 1)
+            got.append((sim.paths(0, min(paths, 200)), *sim.sums()))
+        finally:
+            sim.close()
+    assert np.array_equal(got[0][0], got[1][0], equal_nan=True)
+    for u, v in ((got[0][1], got[1][1]), (got[0][2], got[1][2])):
+        assert np.all(np.abs(u - v) <= 1e-12 * np.abs(v))
