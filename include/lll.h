@@ -282,7 +282,7 @@ typedef struct lll_batch lll_batch;
 int lll_batch_init(lll_batch **out, int n_inst, const lll_instance *inst, void *cuda_stream);
 
 /* lll_batch_set_launch -- the launch shape of scheme LLL_FULL or LLL_PICARD
- * (-1: both): threads per block (0: 128), blocks per SM (0: occupancy
+ * (-1: both): threads per block (0: default), blocks per SM (0: occupancy
  * maximum), table rows per staged chunk (0: default) and paths per thread
  * (0 or 1: one; 2: two paths share every staged table load, for padded
  * Q <= 64).  Each scheme keeps its own shape, schedule and graph: alternating

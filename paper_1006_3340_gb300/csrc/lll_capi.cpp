@@ -145,12 +145,16 @@ int launch_plan(const LaunchPlan &plan, const PathArgs &a)
 }
 
 // Paths per thread and threads per block of the time-blocked kernel where the
-// caller has not set them.
+// caller has not set them.  128 threads share a block's staged rows (32-thread
+// blocks fill shared memory with copies of them: N = 120 Picard, 16,384 paths
+// 5.8 against 3.05 ms).  Two paths a thread pay up to 8 nodes once they leave no
+// scheduler short of warps: N = 40, 90,000 paths 1.42 ms (one: 1.38), 130,000
+// paths 1.81 (1.85), 2^20 paths 12.3 (12.6); with 20 nodes (N = 120, 2^17 paths)
+// 16.4 against 14.7.
 static void block_shape(const lll_ctx *ctx, uint64_t paths, int *R, int *T)
 {
-    const uint64_t sms = ctx->sm_count;
-    if (ctx->ppt == 0) *R = paths >= 512 * sms ? 2 : 1;
-    if (ctx->threads == 0) *T = paths >= 256 * sms * *R ? 128 : paths >= 128 * sms ? 64 : 32;
+    if (ctx->ppt == 0) *R = ctx->QR <= 8 && paths >= 640ull * ctx->sm_count ? 2 : 1;
+    if (ctx->threads == 0) *T = 128;
 }
 
 // Same launch shape and arguments as lll_simulate, with no allocation: the
@@ -534,6 +538,24 @@ int lll_set_mapping(lll_ctx *ctx, int mapping, int lanes)
 
 namespace {
 
+// Whether the step mapping of a default launch runs the path mapping's kernels
+// instead (the same log-rates bit for bit).  Up to 8 nodes the pipeline and the
+// time-blocked kernel are faster at every path count: N = 40, 2000 paths 0.127
+// against 0.153 ms, 4096 paths 0.127 against 0.229, 50,000 paths 0.83 against
+// 1.93; N = 10, 2000 paths 0.040 against 0.052.  Longer rules keep the step
+// kernels, whose threads do not carry products across steps, while their
+// intermediate arrays are small: N = 120 (20 nodes), 2000 paths 0.53 against 0.75
+// ms, 4096 paths (1.2e8 units) 0.89 against 0.75; the 9-rate heavy-tailed example
+// (32 nodes), 8192 paths (1.8e6 units) 0.058 against 0.090.
+bool step_as_path(const lll_ctx *ctx, uint64_t paths)
+{
+    if (ctx->QR >= ctx->QP || ctx->lpp > 1 || ctx->ppt > 0 || ctx->threads > 0 || ctx->blocks_per_sm > 0 ||
+        ctx->chunk_rows > 0)
+        return false;
+    const double units = (double)paths * ctx->s * ctx->n * (ctx->n + 1) / 2;
+    return ctx->QR <= 8 || units > (ctx->n >= 24 ? 1e8 : 4e6);
+}
+
 // The Picard scheme with its Euler steps in parallel (lll_paths_step.cu):
 // chunks of paths through the five kernels, then the fixed-order block sum.
 int simulate_step(lll_ctx *ctx, uint64_t first_path, uint64_t paths, uint64_t seed)
@@ -619,7 +641,7 @@ int lll_simulate(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, 
                         "the step-parallel mapping is Picard's: the full scheme's drift reads the simulated rates");
         if (ctx->ns == 0) return fail(ctx, LLL_ESTATE, "lll_set_strikes must come before lll_simulate");
         if (paths == 0) return fail(ctx, LLL_EINVAL, "paths must be > 0");
-        return simulate_step(ctx, first_path, paths, seed);
+        if (!step_as_path(ctx, paths)) return simulate_step(ctx, first_path, paths, seed);
     }
     LaunchPlan plan;
     int rc = plan_launch(ctx, scheme, first_path, paths, seed, &plan);

@@ -21,17 +21,23 @@
 namespace lll {
 namespace {
 
-// Steps per block for QP nodes and R paths per thread.
+// Steps per block for QP nodes and R paths per thread.  N = 120 (20 nodes, four
+// steps a period), 2^17 paths: 14.7 ms with two steps, 13.4 with four.
 __host__ __device__ constexpr int steps_of(int QP, int R)
 {
-    return R == 2 ? (QP <= 4 ? 8 : QP <= 8 ? 4 : QP <= 24 ? 2 : 1) : (QP <= 8 ? 8 : QP <= 16 ? 4 : 2);
+    return R == 2 ? (QP <= 4 ? 8 : QP <= 8 ? 4 : QP <= 24 ? 2 : 1) : (QP <= 8 ? 8 : QP <= 20 ? 4 : 2);
 }
 
-// Blocks of 256 threads per SM the registers are budgeted for.
-__host__ __device__ constexpr int blocks_of(int QP, int R) { return R * steps_of(QP, R) * QP <= 64 ? 2 : 1; }
+// Blocks of 256 threads per SM the registers are budgeted for.  (With 20 nodes
+// and four steps the Picard kernel gains by 128 registers, 15.6 -> 14.0 ms, and
+// the full one loses, 13.4 -> 14.8.)
+__host__ __device__ constexpr int blocks_of(int scheme, int QP, int R)
+{
+    return R * steps_of(QP, R) * QP <= 64 || (scheme == PICARD && R == 1 && QP == 20) ? 2 : 1;
+}
 
 template <int SCHEME, int QP, int R>
-__global__ void __launch_bounds__(kMaxThreads, blocks_of(QP, R)) block_kernel(const PathArgs a)
+__global__ void __launch_bounds__(kMaxThreads, blocks_of(SCHEME, QP, R)) block_kernel(const PathArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int B = steps_of(QP, R), NST = (SCHEME == PICARD) ? 2 : 1;
@@ -64,7 +70,7 @@ __device__ __forceinline__ void batch_item(const PathArgs &a, unsigned char *sme
 }
 
 template <int SCHEME, int QMAX, int R>
-__global__ void __launch_bounds__(kMaxThreads, blocks_of(QMAX > 8 ? 24 : 8, R)) batch_block_kernel(const BatchArgs b)
+__global__ void __launch_bounds__(kMaxThreads, blocks_of(FULL, QMAX > 8 ? 24 : 8, R)) batch_block_kernel(const BatchArgs b)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int NST = (SCHEME == PICARD) ? 2 : 1;
