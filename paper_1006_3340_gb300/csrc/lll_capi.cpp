@@ -19,6 +19,14 @@ int simulate_mlp(lll_ctx *ctx, uint64_t first_path, uint64_t paths, uint64_t see
 int simulate_expand(lll_ctx *ctx, int order, uint64_t first_path, uint64_t paths, uint64_t seed);
 }
 
+namespace lll {
+void dev_free(lll_ctx *ctx, void *p)
+{
+    const char *q = static_cast<const char *>(p);
+    if (q && !(ctx->arena && q >= ctx->arena && q < ctx->arena + ctx->arena_bytes)) cudaFree(p);
+}
+}
+
 using namespace lll;
 
 namespace {
@@ -62,17 +70,19 @@ cudaError_t dalloc(T **p, size_t count)
 
 void free_all(lll_ctx *c)
 {
-    cudaFree(c->d_lam); cudaFree(c->d_x); cudaFree(c->d_W); cudaFree(c->d_w0); cudaFree(c->d_b0);
-    cudaFree(c->d_tab); cudaFree(c->d_row); cudaFree(c->d_brow); cudaFree(c->d_Z0); cudaFree(c->d_L0); cudaFree(c->d_c0);
-    cudaFree(c->d_strikes); cudaFree(c->d_partials); cudaFree(c->d_sums); cudaFree(c->d_state);
-    cudaFree(c->d_snap); cudaFree(c->d_C); cudaFree(c->d_cn); cudaFree(c->d_err);
-    cudaFree(c->d_tab_full); cudaFree(c->d_row_full); cudaFree(c->d_cn_full);
-    cudaFree(c->d_K1); cudaFree(c->d_K2); cudaFree(c->d_K3);
+    for (void *p : {(void *)c->d_tab, (void *)c->d_row, (void *)c->d_brow, (void *)c->d_cn, (void *)c->d_tab_full,
+                    (void *)c->d_row_full, (void *)c->d_cn_full, (void *)c->d_partials, (void *)c->d_sums,
+                    (void *)c->d_state, (void *)c->d_snap, (void *)c->d_err, (void *)c->d_K1, (void *)c->d_K2,
+                    (void *)c->d_K3})
+        dev_free(c, p);
+    cudaFree(c->arena);
     mlp_free(c->mlp);
     c->mlp = nullptr;
     for (auto &e : c->ev)
         if (e) cudaEventDestroy(e);
 }
+
+constexpr size_t kArenaPartials = size_t(1) << 15; // doubles: 608 blocks of 9 rates and 3 strikes
 
 int default_chunk_rows(int n, int QP)
 {
@@ -98,11 +108,11 @@ int ensure_full_tables(lll_ctx *ctx)
     if (e == cudaSuccess) e = dalloc(&row, rows);
     if (e == cudaSuccess) e = dalloc(&cn, ctx->QP);
     const bool room = e == cudaSuccess;
-    // D0 and b0 h as in the sweeps' rows; lambda, K and C are written by the tables
-    if (room) e = cudaMemcpyAsync(row, ctx->d_row, sizeof(float4) * rows, cudaMemcpyDeviceToDevice, ctx->stream);
+    if (room)
+        e = (cudaError_t)launch_tables(ctx->d_lam, ctx->d_x, ctx->d_W, ctx->Q, ctx->n, ctx->S, ctx->QP, ctx->h, ctx->c,
+                                       nullptr, tab, cn, row, nullptr, ctx->d_C, nullptr, ctx->stream);
     if (e == cudaSuccess)
-        e = (cudaError_t)launch_tables(ctx->d_lam, ctx->d_x, ctx->d_W, ctx->Q, ctx->d_x, ctx->d_W, ctx->Q, ctx->n,
-                                       ctx->S, ctx->QP, ctx->h, tab, cn, row, nullptr, nullptr, ctx->d_C, ctx->stream);
+        e = (cudaError_t)launch_prefix(ctx->d_b0, ctx->n, ctx->S, ctx->h, nullptr, ctx->delta, row, nullptr, ctx->stream);
     if (e != cudaSuccess) {
         cudaFree(tab);
         cudaFree(row);
@@ -119,15 +129,11 @@ int use_full_tables(lll_ctx *ctx)
 {
     const int rc = ensure_full_tables(ctx);
     if (rc != LLL_OK || !ctx->d_tab_full) return rc;
-    std::swap(ctx->d_tab, ctx->d_tab_full);
-    std::swap(ctx->d_row, ctx->d_row_full);
-    std::swap(ctx->d_cn, ctx->d_cn_full);
-    cudaFree(ctx->d_tab_full);
-    cudaFree(ctx->d_row_full);
-    cudaFree(ctx->d_cn_full);
+    ctx->d_tab = ctx->d_tab_full; // the shorter rule's stay in the arena, unused
+    ctx->d_row = ctx->d_row_full;
+    ctx->d_cn = ctx->d_cn_full;
     ctx->d_tab_full = ctx->d_row_full = nullptr;
     ctx->d_cn_full = nullptr;
-    cudaFree(ctx->d_brow);
     ctx->d_brow = nullptr;
     ctx->QR = ctx->QP;
     return LLL_OK;
@@ -355,12 +361,9 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
         Q = 0;
     }
 
-    std::vector<double> xs(std::max(Q, 1), 0.0), ws(std::max(Q, 1), 0.0);
-    for (int j = 0; j < Q; ++j) { xs[j] = nodes[j]; ws[j] = weights[j]; }
     int QR = QP, Qr = 0;
-    std::vector<double> xw(2 * kMaxQP + N, 0.0); // the shorter rule: nodes, then weights; then L0
-    if (QP > 0) Qr = shorter_rule(xs.data(), ws.data(), Q, QP, down, up, xw.data(), xw.data() + kMaxQP, &QR);
-    std::copy(L0, L0 + N, xw.begin() + 2 * kMaxQP);
+    double xr[32], wr[32];
+    if (QP > 0) Qr = shorter_rule(nodes, weights, Q, QP, down, up, xr, wr, &QR);
     lll_ctx *c = new lll_ctx();
     c->QR = QR;
     c->N = N; c->n = n; c->s = steps_per_period; c->S = S; c->Q = Q; c->QP = QP;
@@ -373,11 +376,9 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     double BN = 1.0;
     for (int m = 0; m < N; ++m) BN /= 1.0 + tenor_delta * L0[m]; // Eq. (i-val) inverted
     c->BN = BN;
-    double *d_short = nullptr; // the shorter rule's nodes and weights and L0, for the tables
 
     auto bail = [&](int code) {
         std::string m = c->err;
-        cudaFree(d_short);
         free_all(c);
         delete c;
         g_err = m;
@@ -388,25 +389,57 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     if ((e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device)) != cudaSuccess) {
         cuda_fail(c, e, "cudaDeviceGetAttribute"); return bail(LLL_ECUDA);
     }
-    std::vector<float> Z0(n), c0(n), Lf(n);
-    std::vector<double> w0(n);
-    for (int l = 1; l <= n; ++l) {
-        Z0[l - 1] = (float)std::log(L0[l]);
-        Lf[l - 1] = (float)L0[l];
-        c0[l - 1] = (float)(std::log(L0[l]) + std::log(tenor_delta));
-        w0[l - 1] = tenor_delta * L0[l] / (1.0 + tenor_delta * L0[l]);
-    }
+    // One arena: the inputs (one host image, one copy), then the tables, then
+    // strikes, sums and payoff scratch for the usual sizes.
     const size_t rows = (size_t)S * n;
-    bool ok = dalloc(&c->d_lam, rows) == cudaSuccess && dalloc(&c->d_x, std::max(Q, 1)) == cudaSuccess &&
-              dalloc(&c->d_W, std::max(Q, 1)) == cudaSuccess && dalloc(&c->d_w0, n) == cudaSuccess &&
-              dalloc(&c->d_b0, rows) == cudaSuccess &&
-              dalloc(&c->d_tab, rows * std::max(QR / 4, 1)) == cudaSuccess &&
-              dalloc(&c->d_cn, std::max(QR, 4)) == cudaSuccess &&
-              (Qr == 0 || (dalloc(&d_short, xw.size()) == cudaSuccess && dalloc(&c->d_brow, rows) == cudaSuccess)) &&
-              dalloc(&c->d_row, rows) == cudaSuccess && dalloc(&c->d_C, rows) == cudaSuccess &&
-              dalloc(&c->d_Z0, n) == cudaSuccess && dalloc(&c->d_L0, n) == cudaSuccess &&
-              dalloc(&c->d_c0, n) == cudaSuccess;
-    if (!ok) { fail(c, LLL_ENOMEM, "cudaMalloc of model tables failed"); return bail(LLL_ENOMEM); }
+    size_t bytes = 0;
+    auto place = [&](size_t size) {
+        const size_t at = bytes;
+        bytes += (size + 255) & ~size_t(255);
+        return at;
+    };
+    const size_t at_lam = place(8 * rows), at_x = place(8 * (size_t)Q), at_W = place(8 * (size_t)Q),
+                 at_xr = place(8 * (size_t)Qr), at_wr = place(8 * (size_t)Qr), at_w0 = place(8 * (size_t)n),
+                 at_Ld = place(8 * (size_t)N), at_Z0 = place(4 * (size_t)n), at_L0 = place(4 * (size_t)n),
+                 at_c0 = place(4 * (size_t)n);
+    const size_t in_bytes = bytes;
+    const size_t at_b0 = place(8 * rows), at_tab = place(4 * rows * std::max(QR, 4)), at_cn = place(4 * std::max(QR, 4)),
+                 at_row = place(16 * rows), at_brow = place(Qr > 0 ? 16 * rows : 0), at_C = place(4 * rows),
+                 at_strikes = place(4 * (size_t)n * 64), at_sums = place(16 * (size_t)n * 64),
+                 at_part = place(kArenaPartials * 8);
+    std::vector<char> in(in_bytes);
+    auto host = [&](size_t at) { return reinterpret_cast<double *>(in.data() + at); };
+    std::memcpy(host(at_lam), lambda, 8 * rows);
+    std::memcpy(host(at_Ld), L0, 8 * (size_t)N);
+    if (Q > 0) {
+        std::memcpy(host(at_x), nodes, 8 * (size_t)Q);
+        std::memcpy(host(at_W), weights, 8 * (size_t)Q);
+    }
+    if (Qr > 0) {
+        std::memcpy(host(at_xr), xr, 8 * (size_t)Qr);
+        std::memcpy(host(at_wr), wr, 8 * (size_t)Qr);
+    }
+    for (int l = 1; l <= n; ++l) {
+        host(at_w0)[l - 1] = tenor_delta * L0[l] / (1.0 + tenor_delta * L0[l]);
+        reinterpret_cast<float *>(in.data() + at_Z0)[l - 1] = (float)std::log(L0[l]);
+        reinterpret_cast<float *>(in.data() + at_L0)[l - 1] = (float)L0[l];
+        reinterpret_cast<float *>(in.data() + at_c0)[l - 1] = (float)(std::log(L0[l]) + std::log(tenor_delta));
+    }
+    if (cudaMalloc((void **)&c->arena, bytes) != cudaSuccess) {
+        c->arena = nullptr;
+        fail(c, LLL_ENOMEM, "cudaMalloc of model tables failed");
+        return bail(LLL_ENOMEM);
+    }
+    c->arena_bytes = bytes;
+    auto dev = [&](size_t at) { return c->arena + at; };
+    c->d_lam = (double *)dev(at_lam); c->d_x = (double *)dev(at_x); c->d_W = (double *)dev(at_W);
+    c->d_w0 = (double *)dev(at_w0); c->d_b0 = (double *)dev(at_b0); c->d_tab = (float4 *)dev(at_tab);
+    c->d_cn = (float *)dev(at_cn); c->d_row = (float4 *)dev(at_row); c->d_brow = Qr > 0 ? (float4 *)dev(at_brow) : nullptr;
+    c->d_C = (float *)dev(at_C); c->d_Z0 = (float *)dev(at_Z0); c->d_L0 = (float *)dev(at_L0);
+    c->d_c0 = (float *)dev(at_c0); c->d_strikes = (float *)dev(at_strikes); c->d_sums = (double *)dev(at_sums);
+    c->sums_cap = 2 * (size_t)n * 64;
+    c->d_partials = (double *)dev(at_part);
+    c->partials_cap = kArenaPartials;
     for (auto &ev : c->ev)
         if ((e = cudaEventCreate(&ev)) != cudaSuccess) { cuda_fail(c, e, "cudaEventCreate"); return bail(LLL_ECUDA); }
     cudaStream_t st = c->stream;
@@ -415,25 +448,14 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
         cudaError_t e2 = (expr);                                                                   \
         if (e2 != cudaSuccess) { cuda_fail(c, e2, #expr); return bail(LLL_ECUDA); }               \
     } while (0)
-    INIT_TRY(cudaMemcpyAsync(c->d_lam, lambda, sizeof(double) * rows, cudaMemcpyHostToDevice, st));
-    INIT_TRY(cudaMemcpyAsync(c->d_x, xs.data(), sizeof(double) * xs.size(), cudaMemcpyHostToDevice, st));
-    INIT_TRY(cudaMemcpyAsync(c->d_W, ws.data(), sizeof(double) * ws.size(), cudaMemcpyHostToDevice, st));
-    INIT_TRY(cudaMemcpyAsync(c->d_w0, w0.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
-    INIT_TRY(cudaMemcpyAsync(c->d_Z0, Z0.data(), sizeof(float) * n, cudaMemcpyHostToDevice, st));
-    INIT_TRY(cudaMemcpyAsync(c->d_L0, Lf.data(), sizeof(float) * n, cudaMemcpyHostToDevice, st));
-    INIT_TRY(cudaMemcpyAsync(c->d_c0, c0.data(), sizeof(float) * n, cudaMemcpyHostToDevice, st));
-    INIT_TRY(cudaMemsetAsync(c->d_row, 0, sizeof(float4) * rows, st));
-    if (Qr > 0)
-        INIT_TRY(cudaMemcpyAsync(d_short, xw.data(), sizeof(double) * xw.size(), cudaMemcpyHostToDevice, st));
-    const double *xr = Qr > 0 ? d_short : c->d_x, *wr = Qr > 0 ? d_short + kMaxQP : c->d_W;
-    INIT_TRY((cudaError_t)launch_tables(c->d_lam, c->d_x, c->d_W, Q, xr, wr, Qr > 0 ? Qr : Q, n, S, QR, c->h,
-                                        c->d_tab, c->d_cn, c->d_row, c->d_brow, c->d_b0, c->d_C, st));
-    INIT_TRY((cudaError_t)launch_frozen_drift(c->d_lam, c->d_x, c->d_W, c->d_w0, n, S, Q, c->c, c->h,
-                                              d_short ? d_short + 2 * kMaxQP : nullptr, tenor_delta, c->d_b0, c->d_row, c->d_brow, st));
-    // The host vectors above go out of scope: wait for the copies.
+    INIT_TRY(cudaMemcpyAsync(c->arena, in.data(), in_bytes, cudaMemcpyHostToDevice, st));
+    INIT_TRY((cudaError_t)launch_tables(c->d_lam, Qr > 0 ? (double *)dev(at_xr) : c->d_x,
+                                        Qr > 0 ? (double *)dev(at_wr) : c->d_W, Qr > 0 ? Qr : Q, n, S, QR, c->h, c->c,
+                                        c->d_w0, c->d_tab, c->d_cn, c->d_row, c->d_brow, c->d_C, c->d_b0, st));
+    INIT_TRY((cudaError_t)launch_prefix(c->d_b0, n, S, c->h, (double *)dev(at_Ld), tenor_delta, c->d_row, c->d_brow, st));
+    // The host image goes out of scope: wait for the copy.
     INIT_TRY(cudaStreamSynchronize(st));
 #undef INIT_TRY
-    cudaFree(d_short);
     *out = c;
     if (domain_warn)
         return fail(c, LLL_EDOMAIN,
@@ -460,9 +482,6 @@ int lll_set_strikes(lll_ctx *ctx, int n_strikes, const double *strikes)
         if (!isfin(strikes[e])) return fail(ctx, LLL_EINVAL, "strike is NaN/Inf");
         f[e] = (float)strikes[e];
     }
-    cudaFree(ctx->d_strikes);
-    ctx->d_strikes = nullptr;
-    CUDA_TRY(ctx, dalloc(&ctx->d_strikes, cnt));
     CUDA_TRY(ctx, cudaMemcpyAsync(ctx->d_strikes, f.data(), sizeof(float) * cnt, cudaMemcpyHostToDevice,
                                   ctx->stream));
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
@@ -572,7 +591,7 @@ int simulate_step(lll_ctx *ctx, uint64_t first_path, uint64_t paths, uint64_t se
     Pc = std::min<uint64_t>(Pc, paths);
     const size_t floats = per_path / 4 * Pc;
     if (floats > ctx->state_cap) {
-        cudaFree(ctx->d_state);
+        dev_free(ctx, ctx->d_state);
         ctx->d_state = nullptr;
         ctx->state_cap = 0;
         if (dalloc(&ctx->d_state, floats) != cudaSuccess) return fail(ctx, LLL_ENOMEM, "step-parallel scratch");
@@ -582,14 +601,14 @@ int simulate_step(lll_ctx *ctx, uint64_t first_path, uint64_t paths, uint64_t se
     for (uint64_t c0 = 0; c0 < paths; c0 += Pc) blocks += step_blocks_per_chunk((int)std::min<uint64_t>(Pc, paths - c0));
     const size_t nout = (size_t)plan.n_out;
     if ((size_t)blocks * nout > ctx->partials_cap) {
-        cudaFree(ctx->d_partials);
+        dev_free(ctx, ctx->d_partials);
         ctx->d_partials = nullptr;
         ctx->partials_cap = 0;
         if (dalloc(&ctx->d_partials, (size_t)blocks * nout) != cudaSuccess) return fail(ctx, LLL_ENOMEM, "partials");
         ctx->partials_cap = (size_t)blocks * nout;
     }
     if (nout > ctx->sums_cap) {
-        cudaFree(ctx->d_sums);
+        dev_free(ctx, ctx->d_sums);
         ctx->d_sums = nullptr;
         ctx->sums_cap = 0;
         if (dalloc(&ctx->d_sums, nout) != cudaSuccess) return fail(ctx, LLL_ENOMEM, "sums");
@@ -649,7 +668,7 @@ int lll_simulate(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, 
     const int grid = plan.grid;
     const size_t state_need = plan.state_floats_per_block * grid;
     if (state_need > ctx->state_cap) {
-        cudaFree(ctx->d_state);
+        dev_free(ctx, ctx->d_state);
         ctx->d_state = nullptr;
         ctx->state_cap = 0;
         if (dalloc(&ctx->d_state, state_need) != cudaSuccess) return fail(ctx, LLL_ENOMEM, "state scratch");
@@ -657,14 +676,14 @@ int lll_simulate(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, 
     }
     const size_t nout = (size_t)plan.n_out, part_need = plan.partial_doubles_per_block * grid;
     if (part_need > ctx->partials_cap) {
-        cudaFree(ctx->d_partials);
+        dev_free(ctx, ctx->d_partials);
         ctx->d_partials = nullptr;
         ctx->partials_cap = 0;
         if (dalloc(&ctx->d_partials, part_need) != cudaSuccess) return fail(ctx, LLL_ENOMEM, "partials");
         ctx->partials_cap = part_need;
     }
     if (nout > ctx->sums_cap) {
-        cudaFree(ctx->d_sums);
+        dev_free(ctx, ctx->d_sums);
         ctx->d_sums = nullptr;
         ctx->sums_cap = 0;
         if (dalloc(&ctx->d_sums, nout) != cudaSuccess) return fail(ctx, LLL_ENOMEM, "sums");

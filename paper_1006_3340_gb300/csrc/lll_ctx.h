@@ -22,7 +22,10 @@ struct lll_ctx {
     cudaStream_t stream = nullptr;
     int device = 0, sm_count = 0;
     std::vector<double> L0;
-    // device
+    // device: model tables, strikes, sums and a first payoff scratch lie in one
+    // allocation (an init of a 9-rate model spent 105 of 290 us in 17 cudaMallocs)
+    char *arena = nullptr;
+    size_t arena_bytes = 0;
     double *d_lam = nullptr, *d_x = nullptr, *d_W = nullptr, *d_w0 = nullptr, *d_b0 = nullptr;
     float4 *d_tab = nullptr, *d_row = nullptr; // of the sweeps' rule
     float4 *d_brow = nullptr; // rows of the shorter rule (null where the given one is swept)

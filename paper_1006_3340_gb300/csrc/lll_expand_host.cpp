@@ -107,7 +107,7 @@ int simulate_expand(lll_ctx *ctx, int order, uint64_t first_path, uint64_t paths
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)occ * ctx->sm_count);
     const size_t state_need = (size_t)grid * ctx->n * T;
     if (state_need > ctx->state_cap) {
-        cudaFree(ctx->d_state);
+        dev_free(ctx, ctx->d_state);
         ctx->d_state = nullptr;
         ctx->state_cap = 0;
         if (cudaMalloc((void **)&ctx->d_state, 4 * state_need) != cudaSuccess)
@@ -116,7 +116,7 @@ int simulate_expand(lll_ctx *ctx, int order, uint64_t first_path, uint64_t paths
     }
     const size_t nout = (size_t)plan.n_out;
     if ((size_t)grid * nout > ctx->partials_cap) {
-        cudaFree(ctx->d_partials);
+        dev_free(ctx, ctx->d_partials);
         ctx->d_partials = nullptr;
         ctx->partials_cap = 0;
         if (cudaMalloc((void **)&ctx->d_partials, 8 * grid * nout) != cudaSuccess)
@@ -124,7 +124,7 @@ int simulate_expand(lll_ctx *ctx, int order, uint64_t first_path, uint64_t paths
         ctx->partials_cap = (size_t)grid * nout;
     }
     if (nout > ctx->sums_cap) {
-        cudaFree(ctx->d_sums);
+        dev_free(ctx, ctx->d_sums);
         ctx->d_sums = nullptr;
         ctx->sums_cap = 0;
         if (cudaMalloc((void **)&ctx->d_sums, 8 * nout) != cudaSuccess) return record_error(ctx, LLL_ENOMEM, "sums");

@@ -125,15 +125,13 @@ int launch_batch_kernel(int scheme, int QP, int R, int grid, int threads, size_t
                         const BatchArgs &b);
 
 // Launchers implemented in lll_tables.cu.
-// xr, Wr, Qr: the rule of the table (padded to QP nodes); x, W, Q: the rule as
-// given, for C.  brow (null: none): rows of the shorter rule, whose factors cn
-// and constants are scaled by -h; Cs: scratch for them, [S][n].
-int launch_tables(const double *lam, const double *x, const double *W, int Q, const double *xr, const double *Wr,
-                  int Qr, int n, int S, int QP, double h, float4 *tab, float *cn, float4 *row, float4 *brow,
-                  double *Cs, float *Ctab, cudaStream_t st);
-int launch_frozen_drift(const double *lam, const double *x, const double *W, const double *w0,
-                        int n, int S, int Q, double c, double h, const double *L0, double delta, double *b0,
-                        float4 *row, float4 *brow, cudaStream_t st);
+// Tables of the rule (x, W, Q), padded to QP nodes; see tables_kernel.
+int launch_tables(const double *lam, const double *x, const double *W, int Q, int n, int S, int QP, double h, double c,
+                  const double *w0, float4 *tab, float *cn, float4 *row, float4 *brow, float *Ctab, double *b0,
+                  cudaStream_t st);
+// D0 and b0 h into the rows, and the weight exponent's constant into brow (may be null).
+int launch_prefix(const double *b0, int n, int S, double h, const double *L0, double delta, float4 *row, float4 *brow,
+                  cudaStream_t st);
 int launch_finalize(const double *partials, int grid, int n_out, double *sums, cudaStream_t st);
 
 // Implemented in lll_gemm_tc.cu: read and clear the error word of the tcgen05
@@ -153,6 +151,7 @@ namespace lll {
 int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, uint64_t seed,
                 LaunchPlan *plan, bool allow_tenor = true, bool given_rule = false, bool allow_pipe = true);
 int record_error(lll_ctx *ctx, int code, const char *msg);
+void dev_free(lll_ctx *ctx, void *p); // cudaFree, unless p lies in the context's arena
 int ensure_full_tables(lll_ctx *ctx); // the tables of the rule as given
 int use_full_tables(lll_ctx *ctx);    // every sweep of this context takes them from now on
 // Implemented in lll_quadrature.cpp.

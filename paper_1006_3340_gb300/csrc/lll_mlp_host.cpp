@@ -602,7 +602,7 @@ int simulate_mlp_layered(lll_ctx *ctx, MlpState *m, uint64_t first_path, uint64_
     if (rc != LLL_OK) return rc;
     const size_t state_need = (size_t)n * Pc;
     if (state_need > ctx->state_cap) {
-        cudaFree(ctx->d_state);
+        dev_free(ctx, ctx->d_state);
         ctx->d_state = nullptr;
         ctx->state_cap = 0;
         if (cudaMalloc((void **)&ctx->d_state, 4 * state_need) != cudaSuccess) return err(ctx, LLL_ENOMEM, "state");
@@ -618,14 +618,14 @@ int simulate_mlp_layered(lll_ctx *ctx, MlpState *m, uint64_t first_path, uint64_
     }
     const size_t nout = (size_t)plan.n_out;
     if ((size_t)grid * nout > ctx->partials_cap) {
-        cudaFree(ctx->d_partials);
+        dev_free(ctx, ctx->d_partials);
         ctx->d_partials = nullptr;
         ctx->partials_cap = 0;
         if (cudaMalloc((void **)&ctx->d_partials, 8 * grid * nout) != cudaSuccess) return err(ctx, LLL_ENOMEM, "partials");
         ctx->partials_cap = (size_t)grid * nout;
     }
     if (nout > ctx->sums_cap) {
-        cudaFree(ctx->d_sums);
+        dev_free(ctx, ctx->d_sums);
         ctx->d_sums = nullptr;
         ctx->sums_cap = 0;
         if (cudaMalloc((void **)&ctx->d_sums, 8 * nout) != cudaSuccess) return err(ctx, LLL_ENOMEM, "sums");
@@ -681,14 +681,14 @@ int simulate_mlp_wide(lll_ctx *ctx, MlpState *m, uint64_t first_path, uint64_t p
     }
     const size_t nout = (size_t)plan.n_out;
     if ((size_t)grid * nout > ctx->partials_cap) {
-        cudaFree(ctx->d_partials);
+        dev_free(ctx, ctx->d_partials);
         ctx->d_partials = nullptr;
         ctx->partials_cap = 0;
         if (cudaMalloc((void **)&ctx->d_partials, 8 * grid * nout) != cudaSuccess) return err(ctx, LLL_ENOMEM, "partials");
         ctx->partials_cap = (size_t)grid * nout;
     }
     if (nout > ctx->sums_cap) {
-        cudaFree(ctx->d_sums);
+        dev_free(ctx, ctx->d_sums);
         ctx->d_sums = nullptr;
         ctx->sums_cap = 0;
         if (cudaMalloc((void **)&ctx->d_sums, 8 * nout) != cudaSuccess) return err(ctx, LLL_ENOMEM, "sums");
@@ -781,7 +781,7 @@ int simulate_mlp(lll_ctx *ctx, uint64_t first_path, uint64_t paths, uint64_t see
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)occ * ctx->sm_count);
     const size_t state_need = (size_t)grid * ctx->n * T;
     if (state_need > ctx->state_cap) {
-        cudaFree(ctx->d_state);
+        dev_free(ctx, ctx->d_state);
         ctx->d_state = nullptr;
         ctx->state_cap = 0;
         if (cudaMalloc((void **)&ctx->d_state, 4 * state_need) != cudaSuccess) return err(ctx, LLL_ENOMEM, "state");
@@ -789,14 +789,14 @@ int simulate_mlp(lll_ctx *ctx, uint64_t first_path, uint64_t paths, uint64_t see
     }
     const size_t nout = (size_t)plan.n_out;
     if ((size_t)grid * nout > ctx->partials_cap) {
-        cudaFree(ctx->d_partials);
+        dev_free(ctx, ctx->d_partials);
         ctx->d_partials = nullptr;
         ctx->partials_cap = 0;
         if (cudaMalloc((void **)&ctx->d_partials, 8 * grid * nout) != cudaSuccess) return err(ctx, LLL_ENOMEM, "partials");
         ctx->partials_cap = (size_t)grid * nout;
     }
     if (nout > ctx->sums_cap) {
-        cudaFree(ctx->d_sums);
+        dev_free(ctx, ctx->d_sums);
         ctx->d_sums = nullptr;
         ctx->sums_cap = 0;
         if (cudaMalloc((void **)&ctx->d_sums, 8 * nout) != cudaSuccess) return err(ctx, LLL_ENOMEM, "sums");

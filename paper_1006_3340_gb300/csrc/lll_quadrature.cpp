@@ -51,46 +51,57 @@ double x2nu(double x, double alpha, double beta, double dbar)
     return dbar * alpha / M_PI * ax * std::exp(beta * x) * std::cyl_bessel_k(1.0, alpha * ax);
 }
 
-// Recurrence coefficients al[0..Q), bt[1..Q) of the polynomials orthonormal for
+// Recurrence coefficients al[0..K), bt[1..K) of the polynomials orthonormal for
 // the measure sum_i v_i delta_{y_i} (Stieltjes procedure with orthonormal
-// vectors q_k(y_i) sqrt(v_i) and full re-orthogonalisation).  0 on success.
-int jacobi_of_measure(const std::vector<double> &y, const std::vector<double> &v, int Q, std::vector<double> &al,
-                      std::vector<double> &bt, double &mu0)
-{
-    const size_t M = y.size();
-    al.assign(Q, 0.0);
-    bt.assign(Q + 1, 0.0);
-    mu0 = 0.0;
-    for (size_t i = 0; i < M; ++i) mu0 += v[i];
-    if (!(mu0 > 0.0)) return -1;
+// vectors q_k(y_i) sqrt(v_i) and full re-orthogonalisation), extended on demand.
+struct Jacobi {
+    const std::vector<double> &y;
+    double mu0 = 0.0;
+    std::vector<double> al, bt; // bt[0] unused
     std::vector<std::vector<double>> qs;
-    std::vector<double> q(M), r(M);
-    for (size_t i = 0; i < M; ++i) q[i] = std::sqrt(v[i] / mu0);
-    qs.push_back(q);
-    for (int k = 0; k < Q; ++k) {
-        const std::vector<double> &qk = qs[k];
-        double a_k = 0.0;
-        for (size_t i = 0; i < M; ++i) a_k += y[i] * qk[i] * qk[i];
-        al[k] = a_k;
-        if (k + 1 == Q) break;
-        for (size_t i = 0; i < M; ++i)
-            r[i] = (y[i] - a_k) * qk[i] - (k > 0 ? bt[k] * qs[k - 1][i] : 0.0);
-        for (int pass = 0; pass < 2; ++pass)
-            for (const auto &qq : qs) {
-                double d = 0.0;
-                for (size_t i = 0; i < M; ++i) d += qq[i] * r[i];
-                for (size_t i = 0; i < M; ++i) r[i] -= d * qq[i];
-            }
-        double nr = 0.0;
-        for (size_t i = 0; i < M; ++i) nr += r[i] * r[i];
-        nr = std::sqrt(nr);
-        if (!(nr > 0.0)) return -2;
-        bt[k + 1] = nr;
-        for (size_t i = 0; i < M; ++i) r[i] /= nr;
-        qs.push_back(r);
+
+    Jacobi(const std::vector<double> &y_, const std::vector<double> &v) : y(y_)
+    {
+        for (double w : v) mu0 += w;
+        std::vector<double> q(v.size());
+        for (size_t i = 0; i < v.size(); ++i) q[i] = std::sqrt(v[i] / mu0);
+        qs.push_back(q);
+        bt.push_back(0.0);
     }
-    return 0;
-}
+
+    // Coefficients up to al[K-1]; 0 on success.
+    int extend(int K)
+    {
+        if (!(mu0 > 0.0)) return -1;
+        const size_t M = y.size();
+        while ((int)al.size() < K) {
+            const int k = (int)al.size();
+            if (k > 0) { // the next vector
+                const std::vector<double> &qk = qs[k - 1];
+                std::vector<double> r(M);
+                for (size_t i = 0; i < M; ++i)
+                    r[i] = (y[i] - al[k - 1]) * qk[i] - (k > 1 ? bt[k - 1] * qs[k - 2][i] : 0.0);
+                for (int pass = 0; pass < 2; ++pass)
+                    for (const auto &qq : qs) {
+                        double d = 0.0;
+                        for (size_t i = 0; i < M; ++i) d += qq[i] * r[i];
+                        for (size_t i = 0; i < M; ++i) r[i] -= d * qq[i];
+                    }
+                double nr = 0.0;
+                for (size_t i = 0; i < M; ++i) nr += r[i] * r[i];
+                nr = std::sqrt(nr);
+                if (!(nr > 0.0)) return -2;
+                for (size_t i = 0; i < M; ++i) r[i] /= nr;
+                bt.push_back(nr);
+                qs.push_back(r);
+            }
+            double a = 0.0;
+            for (size_t i = 0; i < M; ++i) a += y[i] * qs[k][i] * qs[k][i];
+            al.push_back(a);
+        }
+        return 0;
+    }
+};
 
 // The Q-point Gauss rule of those coefficients (Q at most their number).
 void gauss_of_jacobi(const std::vector<double> &al, const std::vector<double> &bt, double mu0, int Q, double *nodes,
@@ -163,11 +174,10 @@ int build_nig_rule(double alpha, double beta, double dbar, double a, int Q, doub
                 v.push_back(half * gw[g] * x2nu(xx, alpha, beta, dbar));
             }
         }
-    std::vector<double> al, bt;
-    double mu0 = 0.0;
-    const int rc = jacobi_of_measure(y, v, Q, al, bt, mu0);
+    Jacobi J(y, v);
+    const int rc = J.extend(Q);
     if (rc != 0) return rc;
-    gauss_of_jacobi(al, bt, mu0, Q, nodes, weights);
+    gauss_of_jacobi(J.al, J.bt, J.mu0, Q, nodes, weights);
     return 0;
 }
 
@@ -197,9 +207,9 @@ constexpr double kRuleTol = 1.0 / 268435456.0;
 static bool same_generating_function(const double *x, const double *W, int Q, const double *xr, const double *Wr,
                                      int q, double lo, double hi)
 {
-    constexpr int kGrid = 32; // the relative error grows smoothly away from tau = 0
-    for (int g = 0; g <= 2 * kGrid; ++g) {
-        const double tau = g <= kGrid ? lo * g / kGrid : hi * (g - kGrid) / kGrid;
+    constexpr int kGrid = 32; // the relative error grows smoothly away from tau = 0: the ends first
+    for (int g = 2 * kGrid + 1; g >= 0; --g) {
+        const double tau = (g & 1 ? lo : hi) * (g >> 1) / kGrid;
         if (tau == 0.0 && g > 0) continue;
         double top = 0.0; // largest exponent, taken out against overflow
         for (int j = 0; j < Q; ++j) top = std::max(top, tau * x[j]);
@@ -224,16 +234,15 @@ int shorter_rule(const double *x, const double *W, int Q, int Qpad, double lo, d
         spread += W[j] / std::fabs(x[j]);
     }
     if (!std::isfinite(lo) || !std::isfinite(hi) || !std::isfinite(spread)) return 0;
-    std::vector<double> y(x, x + Q), v(W, W + Q), al, bt;
-    double mu0 = 0.0;
+    std::vector<double> y(x, x + Q), v(W, W + Q);
     const int most = std::min(Q, 32);
-    if (jacobi_of_measure(y, v, most, al, bt, mu0) != 0) return 0;
+    Jacobi J(y, v);
     const int pads[] = {4, 8, 12, 16, 20, 24, 32};
     int below = 0;
     for (int p : pads) {
-        if (p >= Qpad) break;
+        if (p >= Qpad || J.extend(std::min(p, most)) != 0) break;
         for (int q = std::min(p, most); q > below; --q) {
-            gauss_of_jacobi(al, bt, mu0, q, xr, Wr);
+            gauss_of_jacobi(J.al, J.bt, J.mu0, q, xr, Wr);
             if (!same_generating_function(x, W, Q, xr, Wr, q, lo, hi)) break; // fewer nodes are no nearer
             double s = 0.0;
             bool fine = true;

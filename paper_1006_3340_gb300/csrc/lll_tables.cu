@@ -6,151 +6,134 @@
 //   constant K_l = C_l - sum_j fl32(E_lj c_j) with
 //   C_l = sum_j W_j (E_lj - lambda_l x_j) / x_j^2, so that
 //   A_l = K_l + sum_j E_lj (c_j P_j) reproduces C_l when P = 1 up to the FP32
-//   sum.  C_l itself (the compensator with all later weights zero) is kept too.
-// frozen_drift_kernel: the drift b(t_k, T_l; Z(0)) of Eq. (Picard-2), i.e.
-//   Eq. (LIBOR-drift-PT) with L frozen at L(0).
+//   sum.  C_l itself (the compensator with all later weights zero) is kept too,
+//   and the drift b(t_k, T_l; Z(0)) of Eq. (Picard-2), i.e. Eq. (LIBOR-drift-PT)
+//   with L frozen at L(0).
 // prefix_kernel: D0_l(t_k) = sum_{m<k} b0_l(t_m) h, the deterministic drift
 //   integral of Z^(1).
 // finalize_kernel: sum of the per-block payoff partials in a fixed order.
 #include <cuda_runtime.h>
 
 #include "lll_internal.h"
-#include "lll_sweep.cuh"
 
 namespace lll {
 namespace {
 
-// One block per Euler step k, one warp per live rate: lanes over the nodes.
-// FP64 runs at about 2 lanes per SM and clock, so the expm1 of every (rate,
-// node) pair is the cost; only the rates live at the step are built (rows of
-// rates already fixed hold lambda alone, nothing reads the rest), and the
-// warps of a block and the blocks are independent.
-__global__ void tables_kernel(const double *lam, const double *x, const double *W, int Q, const double *xr,
-                              const double *Wr, int Qr, int n, int s, int QP, double scale, float4 *tab, float *cn,
-                              float4 *row, float4 *brow, double *Cs, float *Ctab)
+// One block per Euler step k, over the rates live at it (rows of rates already
+// fixed hold lambda alone; nothing reads the rest) in chunks of kTabRates:
+//   1. E_ij of every (rate, node) pair, a thread a pair: FP64 runs at about 2
+//      lanes per SM and clock, so these expm1 are the cost, and they are formed
+//      once for the table, C, the frozen drift and K;
+//   2. a thread a node carries P_j down the rates and leaves the drift's terms;
+//   3. a thread a rate adds up its terms over the nodes.
+// C and the frozen drift are formed with the sweeps' rule, like the table: both
+// are integrals of its generating function (lll_quadrature.cpp), C over [0,
+// lambda] alone.  short_rule: the sweeps' rule is a shorter one; its rows brow
+// then hold K' = -h C less the dot product at zero weights as sweep_dot forms it.
+// w0, b0 null: the table alone (rows of another rule of the same model).
+constexpr int kTabRates = 32;
+
+__global__ void tables_kernel(const double *lam, const double *x, const double *W, int Q, int n, int s, int QP, double h,
+                              double c, const double *w0, float4 *tab, float *cn, float4 *row, float4 *brow, float *Ctab,
+                              double *b0)
 {
-    const int k = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    extern __shared__ double sm_tab[];
+    double *E = sm_tab, *term = E + kTabRates * Q, *P = term + kTabRates * Q, *cj = P + Q; // [kTabRates][Q] twice, [Q] twice
+    const int k = blockIdx.x, tid = threadIdx.x, T = blockDim.x;
     const int imin = k / s + 1;
-    if (k == 0)
-        for (int j = threadIdx.x; j < QP; j += blockDim.x)
-            cn[j] = (j < Qr) ? (float)(scale * (Wr[j] / (xr[j] * xr[j]))) : 0.0f;
-    for (int i = warp + 1; i <= n; i += nw) {
+    const double scale = brow ? -h : 1.0;
+    for (int j = tid; j < QP; j += T) {
+        if (j < Q) {
+            P[j] = 1.0;
+            cj[j] = W[j] / (x[j] * x[j]);
+        }
+        if (k == 0) cn[j] = j < Q ? (float)(scale * cj[j]) : 0.0f;
+    }
+    for (int i = tid + 1; i < imin; i += T) {
         const size_t idx = (size_t)k * n + (i - 1);
-        const double li = lam[idx];
-        double C = 0.0, sa = 0.0;
-        float *out = reinterpret_cast<float *>(tab + idx * (QP / 4));
-        if (i >= imin)
-            for (int j = lane; j < Q; j += 32) {
-                const double xj = x[j];
-                C += W[j] / (xj * xj) * (expm1(li * xj) - li * xj);
-            }
-        for (int j = lane; j < QP; j += 32) {
-            float e = 0.0f;
-            if (i >= imin && j < Qr) {
-                e = (float)expm1(li * xr[j]);
-                sa += (double)__fmul_rn(e, (float)(scale * (Wr[j] / (xr[j] * xr[j]))));
-            }
-            out[j] = e;
+        row[idx] = make_float4((float)lam[idx], 0.0f, 0.0f, 0.0f);
+        if (brow) brow[idx] = make_float4((float)lam[idx], 0.0f, 0.0f, 0.0f);
+        Ctab[idx] = 0.0f;
+    }
+    double scont = 0.0; // sum of w_l lambda_l over the rates above (every thread)
+    for (int i0 = n; i0 >= imin; i0 -= kTabRates) {
+        const int cnt = min(kTabRates, i0 - imin + 1);
+        for (int e = tid; e < cnt * Q; e += T) E[e] = expm1(lam[(size_t)k * n + (i0 - e / Q - 1)] * x[e % Q]);
+        __syncthreads();
+        for (int e = tid; e < cnt * QP; e += T) {
+            const int u = e / QP, j = e % QP;
+            reinterpret_cast<float *>(tab)[((size_t)k * n + (i0 - u - 1)) * QP + j] = j < Q ? (float)E[u * Q + j] : 0.0f;
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            C += __shfl_xor_sync(0xffffffffu, C, o);
-            sa += __shfl_xor_sync(0xffffffffu, sa, o);
-        }
-        if (lane == 0) {
-            *reinterpret_cast<float2 *>(&row[idx]) = make_float2((float)li, (float)(C - sa / scale));
+        if (b0)
+            for (int j = tid; j < Q; j += T) {
+                double p = P[j];
+                const double cc = cj[j], xj = x[j];
+                for (int u = 0; u < cnt; ++u) {
+                    const int i = i0 - u;
+                    const double e = E[u * Q + j];
+                    term[u * Q + j] = cc * (e * p - lam[(size_t)k * n + (i - 1)] * xj);
+                    p *= 1.0 + w0[i - 1] * e;
+                }
+                P[j] = p;
+            }
+        __syncthreads();
+        for (int u = tid; u < cnt; u += T) {
+            const int i = i0 - u;
+            const size_t idx = (size_t)k * n + (i - 1);
+            const double li = lam[idx];
+            double C = 0.0, sa = 0.0, A = 0.0;
+            float2 a = make_float2(0.0f, 0.0f), b = make_float2(0.0f, 0.0f); // the sums of sweep_dot
+            for (int j = 0; j < Q; ++j) {
+                const double e = E[u * Q + j];
+                const float ef = (float)e, cf = (float)(scale * cj[j]);
+                C += cj[j] * (e - li * x[j]);
+                if (b0) A += term[u * Q + j];
+                if (!brow) sa += (double)__fmul_rn(ef, cf);
+                float &acc = (j & 3) == 0 ? a.x : (j & 3) == 1 ? a.y : (j & 3) == 2 ? b.x : b.y;
+                acc = fmaf(ef, cf, acc);
+            }
+            row[idx] = make_float4((float)li, (float)(C - sa), 0.0f, 0.0f);
             if (brow) {
-                brow[idx].x = (float)li;
-                brow[idx].w = 0.0f;
-                Cs[idx] = scale * C;
+                const float dot = __fadd_rn(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+                brow[idx] = make_float4((float)li, 0.0f, (float)(scale * C - (double)dot), 0.0f);
             }
             Ctab[idx] = (float)C;
-        }
-    }
-}
-
-// K' = -h C less the dot product at zero weights, formed by the sweeps' own FP32
-// operations.  One thread a row.
-template <int QP>
-__global__ void close_kernel(const float4 *tab, const float *cn, const double *Cs, int rows, float4 *brow)
-{
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= rows) return;
-    float4 E[QP / 4];
-    float2 P[QP / 2];
-#pragma unroll
-    for (int j = 0; j < QP / 4; ++j) E[j] = tab[(size_t)r * (QP / 4) + j];
-#pragma unroll
-    for (int j = 0; j < QP / 2; ++j) P[j] = reinterpret_cast<const float2 *>(cn)[j];
-    brow[r].z = (float)(Cs[r] - (double)sweep_dot<QP>(E, P));
-}
-
-// One block per step, one thread per node carrying its product P_j down the
-// live rates; the contributions of kDriftRates rates at a time go through
-// shared memory, where one warp sums each rate over the nodes.
-constexpr int kDriftRates = 16;
-
-__global__ void frozen_drift_kernel(const double *lam, const double *x, const double *W,
-                                    const double *w0, int n, int s, int Q, double c, double *b0)
-{
-    __shared__ double contrib[kDriftRates][kMaxQP + 1];
-    __shared__ double cont[kDriftRates]; // sum of w_l lambda_l over the rates above
-    const int k = blockIdx.x, j = threadIdx.x, lane = j & 31, warp = j >> 5, nw = blockDim.x >> 5;
-    const int imin = k / s + 1;
-    double P = 1.0, scont = 0.0;
-    const double xj = (j < Q) ? x[j] : 0.0;
-    const double inv = (j < Q) ? W[j] / (xj * xj) : 0.0;
-    for (int i0 = n; i0 >= imin; i0 -= kDriftRates) {
-        const int cnt = min(kDriftRates, i0 - imin + 1);
-        for (int u = 0; u < cnt; ++u) {
-            const int i = i0 - u;
-            const double li = lam[(size_t)k * n + (i - 1)], wi = w0[i - 1];
-            if (j < Q) {
-                const double e = expm1(li * xj);
-                contrib[u][j] = inv * (e * P - li * xj);
-                P *= 1.0 + wi * e;
+            if (b0) {
+                double sc = scont;
+                for (int v = 0; v < u; ++v) sc += w0[i0 - v - 1] * lam[(size_t)k * n + (i0 - v - 1)];
+                b0[idx] = -A - 0.5 * c * li * li - c * li * sc;
             }
-            if (j == 0) cont[u] = scont;
-            scont += wi * li;
         }
-        __syncthreads();
-        for (int u = warp; u < cnt; u += nw) {
-            double A = 0.0;
-            for (int t = lane; t < Q; t += 32) A += contrib[u][t];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) A += __shfl_xor_sync(0xffffffffu, A, o);
-            const int i = i0 - u;
-            const double li = lam[(size_t)k * n + (i - 1)];
-            if (lane == 0) b0[(size_t)k * n + (i - 1)] = -A - 0.5 * c * li * li - c * li * cont[u];
-        }
+        if (b0 && c != 0.0)
+            for (int v = 0; v < cnt; ++v) scont += w0[i0 - v - 1] * lam[(size_t)k * n + (i0 - v - 1)];
         __syncthreads();
     }
 }
 
-// Thread per rate: the running integral over the steps it lives, eight steps'
-// loads ahead of their additions.
+// Warp per rate: the running integral over the steps it lives, 32 steps at a
+// time by a scan over the lanes.
 __global__ void prefix_kernel(const double *b0, int n, int s, double h, const double *L0, double delta, float4 *row,
                               float4 *brow)
 {
-    constexpr int U = 8;
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= n) return;
+    const int l = blockIdx.x, lane = threadIdx.x;
     const int K = (l + 1) * s;
     const double c0 = brow ? log(delta * L0[l + 1]) : 0.0;
     double D = 0.0;
-    for (int k0 = 0; k0 < K; k0 += U) {
-        double b[U];
+    for (int k0 = 0; k0 < K; k0 += 32) {
+        const int k = k0 + lane;
+        const double bh = k < K ? b0[(size_t)k * n + l] * h : 0.0;
+        double t = bh;
 #pragma unroll
-        for (int u = 0; u < U; ++u) b[u] = k0 + u < K ? b0[(size_t)(k0 + u) * n + l] : 0.0;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (k0 + u >= K) break;
-            const double bh = b[u] * h;
-            float2 *out = reinterpret_cast<float2 *>(&row[(size_t)(k0 + u) * n + l].z);
-            *out = make_float2((float)D, (float)bh);
-            if (brow) brow[(size_t)(k0 + u) * n + l].y = (float)(-1.4426950408889634 * (c0 + D));
-            D += bh;
+        for (int o = 1; o < 32; o <<= 1) {
+            const double v = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += v;
         }
+        if (k < K) {
+            float2 *out = reinterpret_cast<float2 *>(&row[(size_t)k * n + l].z);
+            *out = make_float2((float)(D + (t - bh)), (float)bh);
+            if (brow) brow[(size_t)k * n + l].y = (float)(-1.4426950408889634 * (c0 + D + (t - bh)));
+        }
+        D += __shfl_sync(0xffffffffu, t, 31);
     }
 }
 
@@ -217,38 +200,23 @@ int batch_finalize(const double *partials, const size_t *seg_off, const int *ins
     return (int)cudaGetLastError();
 }
 
-int launch_tables(const double *lam, const double *x, const double *W, int Q, const double *xr, const double *Wr,
-                  int Qr, int n, int S, int QP, double h, float4 *tab, float *cn, float4 *row, float4 *brow,
-                  double *Cs, float *Ctab, cudaStream_t st)
+int launch_tables(const double *lam, const double *x, const double *W, int Q, int n, int S, int QP, double h, double c,
+                  const double *w0, float4 *tab, float *cn, float4 *row, float4 *brow, float *Ctab, double *b0,
+                  cudaStream_t st)
 {
-    const int warps = n < 8 ? n : 8;
-    tables_kernel<<<S, 32 * warps, 0, st>>>(lam, x, W, Q, xr, Wr, Qr, n, S / n, QP, brow ? -h : 1.0, tab, cn, row,
-                                            brow, Cs, Ctab);
-    if (brow) {
-        const int rows = S * n, blocks = (rows + 127) / 128;
-        switch (QP) {
-        case 4: close_kernel<4><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
-        case 8: close_kernel<8><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
-        case 12: close_kernel<12><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
-        case 16: close_kernel<16><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
-        case 20: close_kernel<20><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
-        case 24: close_kernel<24><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
-        case 32: close_kernel<32><<<blocks, 128, 0, st>>>(tab, cn, Cs, rows, brow); break;
-        default: return (int)cudaErrorInvalidValue;
-        }
+    const size_t smem = sizeof(double) * ((size_t)2 * kTabRates * Q + 2 * (size_t)Q);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return (int)e;
     }
+    tables_kernel<<<S, 128, smem, st>>>(lam, x, W, Q, n, S / n, QP, h, c, w0, tab, cn, row, brow, Ctab, b0);
     return (int)cudaGetLastError();
 }
 
-int launch_frozen_drift(const double *lam, const double *x, const double *W, const double *w0,
-                        int n, int S, int Q, double c, double h, const double *L0, double delta, double *b0,
-                        float4 *row, float4 *brow, cudaStream_t st)
+int launch_prefix(const double *b0, int n, int S, double h, const double *L0, double delta, float4 *row, float4 *brow,
+                  cudaStream_t st)
 {
-    const int threads = Q <= 0 ? 32 : (Q + 31) / 32 * 32;
-    frozen_drift_kernel<<<S, threads, 0, st>>>(lam, x, W, w0, n, S / n, Q, c, b0);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return (int)e;
-    prefix_kernel<<<(n + 31) / 32, 32, 0, st>>>(b0, n, S / n, h, L0, delta, row, brow);
+    prefix_kernel<<<n, 32, 0, st>>>(b0, n, S / n, h, L0, delta, row, brow);
     return (int)cudaGetLastError();
 }
 
