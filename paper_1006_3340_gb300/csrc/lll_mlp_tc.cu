@@ -662,7 +662,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_vec_kernel(const PathArgs 
         auto col_of = [&](int c) { return (c < 8 ? 8 * cq : 8 * cq + 24) + c; };
         const uint32_t dq = tmem + ((uint32_t)(q4 * 32) << 16);
         float *st = reinterpret_cast<float *>(sm + lay.state) + row; // [rate][path]: + (m - 1) T + gi * kRows
-        float *lw = reinterpret_cast<float *>(sm + lay.lc) + warp * 32; // lambda, C of this warp's 16 rates
+        // this warp's 16 rates: lambda and -h (C + s_y b_out), so that an Euler step is
+        // z + (lambda dH + (-h s_y) f + that), f the accumulator
+        float2 *lw = reinterpret_cast<float2 *>(sm + lay.lc) + warp * 16;
+        const float hs = -a.h * g.sc.y_scale;
         const float h = a.h;
         uint32_t phd = 0, php = 0, phe = 0, phh = 0; // bit gi: phase parity of dnb[gi]; bit b: of dhb[b]
         int mcount = 0;
@@ -725,10 +728,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_vec_kernel(const PathArgs 
                 const int imin = k / s + 1;
                 const bool mat = (k + 1) % s == 0;
                 const int gb = (int)(gstep++ & 1);
-                if (lane < 16) {
-                    lw[lane] = lam_next;
-                    lw[16 + lane] = c_next;
-                }
+                if (lane < 16) lw[lane] = make_float2(lam_next, in ? -h * fmaf(g.sc.y_scale, bout[col_of(lane)], c_next) : 0.0f);
                 __syncwarp();
                 if (in && k + 1 < S) {
                     lam_next = a.row[(size_t)(k + 1) * n + (mine - 1)].x;
@@ -788,33 +788,53 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_tc_vec_kernel(const PathArgs 
                     tmem_ld8(dq + gi * kH + 8 * cq + 32, ro + 8);
                     tmem_wait(ro);
                     const uint64_t lp = lp0 + gi * kRows;
+                    const bool snap = mat && a.snap != nullptr && lp < a.paths && lp % a.snap_stride == 0 &&
+                                      lp / a.snap_stride < a.n_snap;
+                    // the rates' step and, from the same registers, their feature columns of
+                    // the next step (a rate already fixed keeps its column)
+                    uint32_t pk[8];
+                    float fprev = 0.0f;
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
                         const int m = col_of(c) - 1;
-                        if (m < imin || m > n) continue; // also m < 1: imin >= 1
-                        const float f = __uint_as_float(ro[c]) + bout[col_of(c)];
-                        const float A = lw[16 + c] + g.sc.y_scale * f;
-                        float *sp = st + (size_t)(m - 1) * T + gi * kRows;
-                        const float z = sp[0] + fmaf(lw[c], dH[gi], -A * h);
-                        sp[0] = z;
-                        if (mat && a.snap != nullptr && lp < a.paths && lp % a.snap_stride == 0 &&
-                            lp / a.snap_stride < a.n_snap)
-                            a.snap[((size_t)(imin - 1) * n + (m - 1)) * a.snap_pitch + lp / a.snap_stride] = z + a.Z0[m - 1];
+                        float f = m < 0 ? (float)(k + 1) * h * g.sc.t_scale : 0.0f;
+                        if (m >= 1 && m <= n) {
+                            float *sp = st + (size_t)(m - 1) * T + gi * kRows;
+                            float z = sp[0];
+                            if (m >= imin) {
+                                const float2 lc = lw[c];
+                                z += fmaf(lc.x, dH[gi], fmaf(hs, __uint_as_float(ro[c]), lc.y));
+                                sp[0] = z;
+                                if (snap)
+                                    a.snap[((size_t)(imin - 1) * n + (m - 1)) * a.snap_pitch + lp / a.snap_stride] = z + a.Z0[m - 1];
+                            }
+                            f = z * g.sc.u_scale;
+                        }
+                        if (c & 1) pk[c >> 1] = pack2(fprev, f);
+                        fprev = f;
+                    }
+                    // this tile's columns are handed over before the other tile's step, so
+                    // that its first-layer product runs under it (this and the fused
+                    // columns: N = 40, 2^18 paths 20.1 -> 19.5 ms; two tiles still leave
+                    // 17k cycles a step against 6.1k of the tanh rate)
+                    if (k + 1 < S) {
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const int c8 = cq + 4 * q;
+                            if (c8 < KB0 * 8)
+                                *reinterpret_cast<uint4 *>(sm + lay.u + gi * KB0 * kTileBytes + chunk_off(row, c8 >> 3, c8 & 7)) =
+                                    make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+                        }
+                        fence_async_smem();
+                        tc_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&opu[gi]);
+                    } else {
+                        tc_before();
                     }
                 }
                 if (!ok) break;
-                // next step's feature columns of these rates; accumulators read
-                if (k + 1 < S) {
-                    for (int gi = 0; gi < kGroups; ++gi) write_features(k + 1, gi);
-                    fence_async_smem();
-                    tc_before();
-                    __syncwarp();
-                    if (lane == 0)
-                        for (int gi = 0; gi < kGroups; ++gi) mbar_arrive(&opu[gi]);
-                    if (drawer) draw_share(k + 1, (int)(gstep & 1));
-                } else {
-                    tc_before();
-                }
+                if (k + 1 < S && drawer) draw_share(k + 1, (int)(gstep & 1));
                 if (mat) {
                     // the owner warps price with every rate of the row's paths
                     if (!owner) {
