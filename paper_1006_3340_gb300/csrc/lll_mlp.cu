@@ -341,6 +341,16 @@ __global__ void to_bf16(const float *x, size_t count, __nv_bfloat16 *y)
     if (e < count) y[e] = __float2bfloat16(x[e]);
 }
 
+// Rows of `dim` numbers into BF16 rows of `pad`, the rest zero.
+__global__ void pack_rows(const float *x, int rows, int dim, int pad, __nv_bfloat16 *y)
+{
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (size_t)rows * pad) return;
+    const size_t r = e / pad;
+    const int c = (int)(e % pad);
+    y[e] = __float2bfloat16(c < dim ? x[r * dim + c] : 0.0f);
+}
+
 unsigned blocks_for(size_t count, int threads) { return (unsigned)((count + threads - 1) / threads); }
 
 }  // namespace
@@ -457,6 +467,12 @@ int mlp_adam(float *p, const float *g, float *m, float *v, void *ph, size_t coun
     const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
     adam<<<blocks_for(count, 256), 256, 0, st>>>(p, g, m, v, static_cast<__nv_bfloat16 *>(ph), count,
                                                  lr, b1, b2, eps, c1, c2);
+    return (int)cudaGetLastError();
+}
+
+int mlp_pack_rows(const float *x, int rows, int dim, int pad, void *y, cudaStream_t st)
+{
+    pack_rows<<<blocks_for((size_t)rows * pad, 256), 256, 0, st>>>(x, rows, dim, pad, static_cast<__nv_bfloat16 *>(y));
     return (int)cudaGetLastError();
 }
 

@@ -51,6 +51,7 @@ int mlp_reduce_splits(const float *part, int splits, size_t count, float *out, c
 int mlp_adam(float *p, const float *g, float *m, float *v, void *ph, size_t count, float lr, float b1,
              float b2, float eps, int t, cudaStream_t st);
 int mlp_to_bf16(const float *x, size_t count, void *y, cudaStream_t st);
+int mlp_pack_rows(const float *x, int rows, int dim, int pad, void *y, cudaStream_t st);
 
 // Feature scaling of the network input row (see lll_mlp.cu).
 struct MlpScales {

@@ -50,8 +50,15 @@ struct MlpState {
     float *d_Y = nullptr, *d_out = nullptr, *d_dout = nullptr;
     std::vector<void *> d_H;        // bf16 [cap][hidden], layers
     std::vector<float *> d_Z;       // fp32 [cap][hidden], layers
-    float *d_dZ[2] = {nullptr, nullptr};
-    void *d_dZh[2] = {nullptr, nullptr};
+    // gradient buffers, one per layer (so that a layer's weight gradients may still
+    // be read on the side stream while the next layer's are formed), for `gcap` rows
+    int gcap = 0;
+    std::vector<float *> d_dZ;
+    std::vector<void *> d_dZh;
+    cudaStream_t side = nullptr;              // weight gradients beside the chain of dX products
+    std::vector<cudaEvent_t> ready;           // dZ of each layer, then the join
+    float *d_xin = nullptr;                   // lll_mlp_eval: feature rows as given
+    size_t xin_cap = 0;
     float *d_split = nullptr;       // split-K partials
     size_t split_cap = 0;
     double *d_loss = nullptr;       // per-block loss partials
@@ -73,7 +80,11 @@ void mlp_free_buffers(MlpState *m)
     for (float *p : m->d_Z) cudaFree(p);
     m->d_H.clear();
     m->d_Z.clear();
-    for (int i = 0; i < 2; ++i) { cudaFree(m->d_dZ[i]); cudaFree(m->d_dZh[i]); m->d_dZ[i] = nullptr; m->d_dZh[i] = nullptr; }
+    for (float *p : m->d_dZ) cudaFree(p);
+    for (void *p : m->d_dZh) cudaFree(p);
+    m->d_dZ.clear();
+    m->d_dZh.clear();
+    m->gcap = 0;
     cudaFree(m->d_split); cudaFree(m->d_loss); cudaFree(m->d_colpart);
     m->d_colpart = nullptr;
     m->d_X = nullptr; m->d_Y = m->d_out = m->d_dout = nullptr; m->d_split = nullptr; m->d_loss = nullptr;
@@ -85,7 +96,9 @@ void mlp_free(MlpState *m)
     if (!m) return;
     mlp_free_buffers(m);
     cudaFree(m->d_p); cudaFree(m->d_g); cudaFree(m->d_m); cudaFree(m->d_v); cudaFree(m->d_ph); cudaFree(m->d_phT);
-    cudaFree(m->d_acc);
+    cudaFree(m->d_acc); cudaFree(m->d_xin);
+    for (cudaEvent_t e : m->ready) cudaEventDestroy(e);
+    if (m->side) cudaStreamDestroy(m->side);
     delete m;
 }
 
@@ -152,9 +165,6 @@ int ensure_rows(lll_ctx *ctx, MlpState *m, int rows)
         m->d_H.push_back(hp);
         m->d_Z.push_back(zp);
     }
-    for (int i = 0; ok && i < 2; ++i)
-        ok = cudaMalloc((void **)&m->d_dZ[i], 4 * (size_t)rows * H) == cudaSuccess &&
-             cudaMalloc(&m->d_dZh[i], 2 * (size_t)rows * H) == cudaSuccess;
     // loss partials: one per 8 rows (per-rate head), one per 128 outputs (vector head)
     const size_t lb = m->head ? ((size_t)rows * O + 127) / 128 : ((size_t)rows + 7) / 8;
     ok = ok && cudaMalloc((void **)&m->d_loss, sizeof(double) * lb) == cudaSuccess;
@@ -166,6 +176,31 @@ int ensure_rows(lll_ctx *ctx, MlpState *m, int rows)
     }
     m->cap = rows;
     m->loss_cap = lb;
+    return LLL_OK;
+}
+
+// What a backward pass over `rows` (at most cap) rows needs besides.
+int ensure_grads(lll_ctx *ctx, MlpState *m, int rows)
+{
+    if (!m->side) {
+        MTRY(cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking));
+        for (int l = 0; l <= m->layers + 1; ++l) {
+            cudaEvent_t e;
+            MTRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+            m->ready.push_back(e);
+        }
+    }
+    if (rows <= m->gcap) return LLL_OK;
+    for (float *p : m->d_dZ) cudaFree(p);
+    for (void *p : m->d_dZh) cudaFree(p);
+    m->d_dZ.assign(m->layers, nullptr);
+    m->d_dZh.assign(m->layers, nullptr);
+    m->gcap = 0;
+    for (int l = 0; l < m->layers; ++l)
+        if (cudaMalloc((void **)&m->d_dZ[l], 4 * (size_t)rows * m->hidden) != cudaSuccess ||
+            cudaMalloc(&m->d_dZh[l], 2 * (size_t)rows * m->hidden) != cudaSuccess)
+            return err(ctx, LLL_ENOMEM, "MLP gradient buffers");
+    m->gcap = rows;
     return LLL_OK;
 }
 
@@ -215,72 +250,82 @@ int forward(lll_ctx *ctx, MlpState *m, int rows, const float *y)
     return LLL_OK;
 }
 
-// Backward pass after forward(y): gradients into d_g.
+// Backward pass after forward(y): gradients into d_g.  The chain dZ_{L-1} ..
+// dZ_0 runs on the context's stream; every layer's weight and bias gradients
+// only read it, and run on the side stream as soon as their dZ is formed (the
+// products of 8,192 rows fill 64 to 128 of the SMs, so the two overlap).  The
+// join at the end orders what follows on the context's stream behind both.
 int backward(lll_ctx *ctx, MlpState *m, int rows)
 {
-    cudaStream_t st = ctx->stream;
+    int rc = ensure_grads(ctx, m, rows);
+    if (rc != LLL_OK) return rc;
+    cudaStream_t st = ctx->stream, sd = m->side;
     const char *ph = static_cast<const char *>(m->d_ph);
     const char *phT = static_cast<const char *>(m->d_phT);
-    const int H = m->hidden, L = m->layers;
+    const int H = m->hidden, L = m->layers, O = m->outputs;
     // dW products: K = rows split into ranges of 64 rows (at most 128 CTAs), so
     // that the 128 x din products fill the GPU
     const int splits_req = std::max(1, std::min(128, rows / 64));
-    // transposed weights: the dX products then read K-contiguous rows
+    const int splits = mlp_splits_used(rows, splits_req);
     const bool tc = mlp_gemm_kind() == LLL_GEMM_TC;
+    rc = ensure_split(ctx, m, (size_t)splits * H * std::max({H, m->in_pad, m->head ? O : 1}));
+    if (rc != LLL_OK) return rc;
+    MTRY(cudaEventRecord(m->ready[L], st)); // forward's outputs
+    MTRY(cudaStreamWaitEvent(sd, m->ready[L], 0));
+    // transposed weights: the dX products then read K-contiguous rows
     if (tc) {
         size_t off[6];
         int rr[6], cc[6], cnt = 0;
         for (int l = 1; l < L; ++l) { off[cnt] = m->offW[l]; rr[cnt] = H; cc[cnt] = H; ++cnt; }
-        if (m->head) { off[cnt] = m->off_wout; rr[cnt] = m->outputs; cc[cnt] = H; ++cnt; }
+        if (m->head) { off[cnt] = m->off_wout; rr[cnt] = O; cc[cnt] = H; ++cnt; }
         if (cnt > 0) MTRY(mlp_transpose_weights(m->d_ph, m->d_phT, off, rr, cc, cnt, st));
     }
     if (m->head) {
-        const int O = m->outputs;
-        // dW_out = dout^T H_{L-1} (O x H), db_out = column sums, dZ_{L-1} = (dout W_out) * SiLU'(Z_{L-1})
-        const int splits = mlp_splits_used(rows, splits_req);
-        int rc = ensure_split(ctx, m, (size_t)splits * O * H);
-        if (rc != LLL_OK) return rc;
-        MTRY(mlp_gemm(1, 0, 0, m->d_douth, O, m->d_H[L - 1], H, O, H, rows, splits_req, m->d_split, nullptr,
-                      nullptr, nullptr, nullptr, st));
-        MTRY(mlp_reduce_splits(m->d_split, splits, (size_t)O * H, m->d_g + m->off_wout, st));
-        MTRY(mlp_column_sums(m->d_dout, rows, O, m->d_g + m->off_bout, m->d_colpart, st));
         // dZ = (dout W_out) SiLU'(Z): B(k = o, n = h) from the transposed copy [H][O]
         // (tcgen05), or read column-wise from W_out (mma.sync)
         if (tc)
             MTRY(mlp_gemm(0, 1, 2, m->d_douth, O, phT + 2 * m->off_wout, O, rows, H, O, 1, nullptr, nullptr,
-                          m->d_Z[L - 1], m->d_dZ[0], m->d_dZh[0], st));
+                          m->d_Z[L - 1], m->d_dZ[L - 1], m->d_dZh[L - 1], st));
         else
             MTRY(mlp_gemm(0, 0, 2, m->d_douth, O, ph + 2 * m->off_wout, H, rows, H, O, 1, nullptr, nullptr,
-                          m->d_Z[L - 1], m->d_dZ[0], m->d_dZh[0], st));
+                          m->d_Z[L - 1], m->d_dZ[L - 1], m->d_dZh[L - 1], st));
+    } else {
+        MTRY(mlp_out_backward(m->d_dout, ph + 2 * m->off_wout, m->d_Z[L - 1], rows, H, m->d_dZ[L - 1], m->d_dZh[L - 1], st));
+    }
+    MTRY(cudaEventRecord(m->ready[L - 1], st));
+    for (int l = L - 1; l > 0; --l) {
+        // dZ_{l-1} = (dZ_l W_l) * SiLU'(Z_{l-1}), W_l read transposed ([in][out]) by the
+        // tcgen05 kernel, column-wise by the mma.sync kernel
+        if (tc)
+            MTRY(mlp_gemm(0, 1, 2, m->d_dZh[l], H, phT + 2 * m->offW[l], H, rows, H, H, 1, nullptr, nullptr,
+                          m->d_Z[l - 1], m->d_dZ[l - 1], m->d_dZh[l - 1], st));
+        else
+            MTRY(mlp_gemm(0, 0, 2, m->d_dZh[l], H, ph + 2 * m->offW[l], H, rows, H, H, 1, nullptr, nullptr,
+                          m->d_Z[l - 1], m->d_dZ[l - 1], m->d_dZh[l - 1], st));
+        MTRY(cudaEventRecord(m->ready[l - 1], st));
+    }
+    if (m->head) {
+        // dW_out = dout^T H_{L-1} (O x H), db_out = column sums
+        MTRY(mlp_gemm(1, 0, 0, m->d_douth, O, m->d_H[L - 1], H, O, H, rows, splits_req, m->d_split, nullptr,
+                      nullptr, nullptr, nullptr, sd));
+        MTRY(mlp_reduce_splits(m->d_split, splits, (size_t)O * H, m->d_g + m->off_wout, sd));
+        MTRY(mlp_column_sums(m->d_dout, rows, O, m->d_g + m->off_bout, m->d_colpart, sd));
     } else {
         MTRY(mlp_out_weight_grad(m->d_dout, m->d_H[L - 1], rows, H, m->d_g + m->off_wout, m->d_g + m->off_bout,
-                                 m->d_colpart, st));
-        MTRY(mlp_out_backward(m->d_dout, ph + 2 * m->off_wout, m->d_Z[L - 1], rows, H, m->d_dZ[0], m->d_dZh[0], st));
+                                 m->d_colpart, sd));
     }
-    int cur = 0;
     for (int l = L - 1; l >= 0; --l) {
         const int din = l == 0 ? m->in_pad : H;
         const void *Hl = l == 0 ? m->d_X : m->d_H[l - 1];
-        const int splits = mlp_splits_used(rows, splits_req);
-        int rc = ensure_split(ctx, m, (size_t)splits * H * din);
-        if (rc != LLL_OK) return rc;
+        MTRY(cudaStreamWaitEvent(sd, m->ready[l], 0));
         // dW_l = dZ_l^T H_l  (M = H, N = din, K = rows)
-        MTRY(mlp_gemm(1, 0, 0, m->d_dZh[cur], H, Hl, din, H, din, rows, splits_req, m->d_split, nullptr,
-                      nullptr, nullptr, nullptr, st));
-        MTRY(mlp_reduce_splits(m->d_split, splits, (size_t)H * din, m->d_g + m->offW[l], st));
-        MTRY(mlp_column_sums(m->d_dZ[cur], rows, H, m->d_g + m->offb[l], m->d_colpart, st));
-        if (l > 0) {
-            // dZ_{l-1} = (dZ_l W_l) * SiLU'(Z_{l-1}), W_l read transposed ([in][out]) by the
-            // tcgen05 kernel, column-wise by the mma.sync kernel
-            if (tc)
-                MTRY(mlp_gemm(0, 1, 2, m->d_dZh[cur], H, phT + 2 * m->offW[l], H, rows, H, H, 1, nullptr, nullptr,
-                              m->d_Z[l - 1], m->d_dZ[cur ^ 1], m->d_dZh[cur ^ 1], st));
-            else
-                MTRY(mlp_gemm(0, 0, 2, m->d_dZh[cur], H, ph + 2 * m->offW[l], H, rows, H, H, 1, nullptr, nullptr,
-                              m->d_Z[l - 1], m->d_dZ[cur ^ 1], m->d_dZh[cur ^ 1], st));
-            cur ^= 1;
-        }
+        MTRY(mlp_gemm(1, 0, 0, m->d_dZh[l], H, Hl, din, H, din, rows, splits_req, m->d_split, nullptr,
+                      nullptr, nullptr, nullptr, sd));
+        MTRY(mlp_reduce_splits(m->d_split, splits, (size_t)H * din, m->d_g + m->offW[l], sd));
+        MTRY(mlp_column_sums(m->d_dZ[l], rows, H, m->d_g + m->offb[l], m->d_colpart, sd));
     }
+    MTRY(cudaEventRecord(m->ready[L + 1], sd));
+    MTRY(cudaStreamWaitEvent(st, m->ready[L + 1], 0));
     return LLL_OK;
 }
 
@@ -442,18 +487,20 @@ int lll_mlp_eval(lll_ctx *ctx, const float *x, const float *y, int rows, float *
     int rc = ensure_rows(ctx, m, rows);
     if (rc != LLL_OK) return rc;
     cudaStream_t st = ctx->stream;
-    std::vector<float> xp((size_t)rows * m->in_pad, 0.0f);
-    for (int r = 0; r < rows; ++r)
-        std::memcpy(&xp[(size_t)r * m->in_pad], &x[(size_t)r * m->in_dim], 4 * m->in_dim);
-    float *tmp = nullptr;
-    MTRY(cudaMalloc((void **)&tmp, 4 * xp.size()));
-    cudaError_t e = cudaMemcpyAsync(tmp, xp.data(), 4 * xp.size(), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = (cudaError_t)mlp_to_bf16(tmp, xp.size(), m->d_X, st);
+    // the rows go over as given; the device pads them and rounds to BF16
+    const size_t given = (size_t)rows * m->in_dim;
+    if (given > m->xin_cap) {
+        cudaFree(m->d_xin);
+        m->d_xin = nullptr;
+        m->xin_cap = 0;
+        if (cudaMalloc((void **)&m->d_xin, 4 * given) != cudaSuccess) return err(ctx, LLL_ENOMEM, "feature rows");
+        m->xin_cap = given;
+    }
+    cudaError_t e = cudaMemcpyAsync(m->d_xin, x, 4 * given, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = (cudaError_t)mlp_pack_rows(m->d_xin, rows, m->in_dim, m->in_pad, m->d_X, st);
     if (e == cudaSuccess && y)
         e = cudaMemcpyAsync(m->d_Y, y, 4 * (size_t)rows * m->outputs, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && y && m->head) e = cudaMemsetAsync(m->d_kr, 0, 4 * (size_t)rows, st); // all rates live
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(tmp);
     if (e != cudaSuccess) return cerr(ctx, e, "staging feature rows");
     rc = forward(ctx, m, rows, y ? m->d_Y : nullptr);
     if (rc != LLL_OK) return rc;
@@ -463,7 +510,7 @@ int lll_mlp_eval(lll_ctx *ctx, const float *x, const float *y, int rows, float *
         MTRY(cudaMemcpyAsync(grads, m->d_g, 4 * m->n_params, cudaMemcpyDeviceToHost, st));
     }
     if (out) MTRY(cudaMemcpyAsync(out, m->d_out, 4 * (size_t)rows * m->outputs, cudaMemcpyDeviceToHost, st));
-    MTRY(cudaStreamSynchronize(st));
+    if (!(loss && y)) MTRY(cudaStreamSynchronize(st)); // reading the loss waits
     if (loss && y) {
         bool ok;
         *loss = read_loss(ctx, m, rows, &ok);
