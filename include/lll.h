@@ -108,7 +108,7 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
  *     is (1 - B(T_m,T_N) - K delta sum_{j>m} B(T_m,T_j))^+, priced under the
  *     terminal measure as B(0,T_N) E[((1 + delta L_m) P - 1 - K delta S)^+]
  *     with P = prod_{l>m} (1 + delta L_l(T_m)) and S = sum_{j=m+1}^{N}
- *     prod_{l>=j} (1 + delta L_l(T_m)) (FP64 on the GPU).  lll_price_caplets
+ *     prod_{l>=j} (1 + delta L_l(T_m)) (48 bits or more on the GPU).  lll_price_caplets
  *     then returns swaption prices.  The batched launch prices caplets only. */
 #define LLL_PRODUCT_CAPLET 0
 #define LLL_PRODUCT_SWAPTION 1
@@ -184,7 +184,9 @@ int lll_set_launch(lll_ctx *ctx, int threads_per_block, int blocks_per_sm, int c
  *     gives the log-rates at every maturity.  Same arithmetic per unit as the
  *     path mapping; intermediate arrays of about 4 (S + 2 S n + n^2) bytes per
  *     path, processed in chunks within 2 GiB of device memory.  For small
- *     path budgets (a single term structure of 2^12 paths).  LLL_FULL
+ *     path budgets (a single term structure of 2^12 paths).  With the default
+ *     launch shape the path mapping's kernels run instead, with the same
+ *     log-rates, where they are faster.  LLL_FULL
  *     returns LLL_EUNSUPPORTED under it: the full scheme's drift reads the
  *     simulated rates, so its steps are sequential.  lll_simulate_noalloc
  *     ignores it (path mapping).
@@ -212,10 +214,12 @@ int lll_kernel_ms(lll_ctx *ctx, float *path_kernel_ms, float *simulate_ms);
  *   d_sums     : caller-owned device buffer of n * n_strikes * 2 doubles,
  *                d_sums[2*(m*n_strikes + q)] = sum of payoffs and [... + 1] =
  *                sum of squared payoffs of maturity m+1, strike q.
- * Makes the same launch as lll_simulate, so the sums equal lll_get_sums'.
+ * Makes the same launch as lll_simulate (with fewer blocks where the scratch
+ * would not hold the state of all), so the sums equal lll_get_sums'.
  * Scratch (per-block path state and payoff partials) comes from one static
  * 32 MiB device array that every GPU loading the library holds until exit;
- * a launch needing more returns LLL_EUNSUPPORTED with the byte counts in
+ * a launch of the rule as given that needs more returns LLL_EUNSUPPORTED with
+ * the byte counts in
  * lll_last_error.  Each call made outside a stream capture looks the array's
  * address up (cudaGetSymbolAddress), so a module reloaded after
  * cudaDeviceReset is found at its new address; a call made while the
@@ -243,7 +247,8 @@ int lll_build_nig_quadrature(lll_nig nig, double xmax, int Q, double *nodes, dou
  * volatilities over the steps, every compensator of Eq. (LIBOR-drift-PT) then
  * agrees to 2^-28 of its terms, whatever the rates.  lo <= 0 <= hi.
  *   count : nodes of the shorter rule; 0 where the given rule is swept (a
- *           weight <= 0, or no shorter rule agrees);
+ *           weight <= 0, a node within 4e-5 of 0 as a share of the farthest,
+ *           or no shorter rule agrees);
  *   padded: nodes the kernels process (the given rule padded where count = 0);
  *   x, w  : [32] outputs, the first `count` used.
  * Host computation. */

@@ -213,7 +213,7 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     size_t pipe_smem = 0;
     const int pipe = allow_pipe && block && ctx->threads == 0 && ctx->blocks_per_sm == 0 && ctx->ppt == 0 &&
                              ctx->chunk_rows == 0 && ctx->product == LLL_PRODUCT_CAPLET
-                         ? pipe_steps(scheme, ctx->QR, ctx->n, ctx->s, ctx->S, (paths + 31) / 32, ctx->sm_count, &pipe_smem)
+                         ? pipe_shape(scheme, ctx->QR, ctx->n, ctx->s, ctx->S, (paths + 31) / 32, ctx->sm_count, &pipe_smem)
                          : 0;
     int occ = 0;
     cudaError_t e;
@@ -524,7 +524,7 @@ int lll_set_launch(lll_ctx *ctx, int threads_per_block, int blocks_per_sm, int c
     }
     ctx->ppt = paths_per_thread;
     ctx->lpp = lanes_per_path;
-    if (threads_per_block) ctx->threads = threads_per_block;
+    ctx->threads = threads_per_block;
     ctx->blocks_per_sm = blocks_per_sm;
     ctx->chunk_rows = std::min(chunk_rows, ctx->n);
     return LLL_OK;

@@ -61,7 +61,7 @@ struct LaunchPlan {
     PathArgs args;
     int scheme, qp, ppt, lpp, threads, grid; // lpp: lanes per group of paths (1, 2 or 4)
     bool block;                              // time-blocked kernel (lll_paths_block.cu)
-    int pipe;                                // > 0: its pipeline for few paths (lll_paths_pipe.cu), steps per block
+    int pipe;                                // != 0: its pipeline for few paths (pipe_shape in lll_paths_pipe.cu)
     int tenor;                               // > 0: tenor-parallel kernel with this many lanes per path
     size_t smem;
     // scratch per block: path state; payoff sums (block kernel: and their compensations,
@@ -95,8 +95,8 @@ int launch_batch_block_kernel(int scheme, int QMAX, int R, int grid, int threads
 
 // Launchers implemented in lll_paths_pipe.cu (few paths: 32 paths a block, a
 // pipeline of warps over the rates).
-int pipe_steps(int scheme, int QP, int n, int s, int S, uint64_t tiles, int sms, size_t *smem);
-int launch_pipe_kernel(int scheme, int QP, int B, size_t smem, uint64_t paths, cudaStream_t st, const PathArgs &a);
+int pipe_shape(int scheme, int QP, int n, int s, int S, uint64_t tiles, int sms, size_t *smem);
+int launch_pipe_kernel(int scheme, int QP, int shape, size_t smem, uint64_t paths, cudaStream_t st, const PathArgs &a);
 
 // Launchers implemented in lll_paths_group.cu (four lanes per group of four paths).
 bool group_kernel_supported(int scheme, int QP, int G);

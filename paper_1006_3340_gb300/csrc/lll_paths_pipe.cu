@@ -225,9 +225,9 @@ __global__ void __launch_bounds__(32 * kPipeWarps, QP <= 8 && B == 4 ? 2 : 1) pi
                 st[0] = z[0];
                 if (NST == 2) st[NST - 1] = z[1];
                 if (mat) {
-                    const float off = NST == 2 ? z[0] + z[1] : z[0], e = expf(off), L0 = sm.L0[i - 1];
-                    if (i > m) Pf *= fmaf(a.delta * L0, e, 1.0f);
-                    else sm.pay[(m - 1) * 32 + lane] = lp < a.paths ? make_float2(a.dBN * Pf, L0 * e) : make_float2(0.0f, 0.0f);
+                    const float off = NST == 2 ? z[0] + z[1] : z[0], L = sm.L0[i - 1] * expf(off);
+                    if (i > m) Pf *= fmaf(a.delta, L, 1.0f);
+                    else sm.pay[(m - 1) * 32 + lane] = lp < a.paths ? make_float2(a.dBN * Pf, L) : make_float2(0.0f, 0.0f);
                     if (a.snap != nullptr && lp < a.paths && lp % a.snap_stride == 0 && lp / a.snap_stride < a.n_snap)
                         a.snap[((size_t)(m - 1) * n + (i - 1)) * a.snap_pitch + lp / a.snap_stride] = off + a.Z0[i - 1];
                 }
@@ -283,50 +283,56 @@ PipeFn pick_pipe(int QP, int B)
     }
 }
 
-int pipe_lg_warps(int n)
-{
-    int lg = 0;
-    while ((2 << lg) <= n && (2 << lg) <= kPipeWarps) ++lg;
-    return lg;
-}
-
 }  // namespace
 
-// Steps per block for `tiles` blocks of 32 paths, 0 where the block kernel is the
-// better one or shared memory does not hold the pipeline.
-//  * One block an SM: as many steps as the registers of the products and of the
-//    rows in work allow (8 or 5 up to 8 nodes, 4 up to 16, else 2), preferring a
-//    divisor of the steps per period: 4096 paths of N = 40 take 0.139 ms (full)
-//    with 8 steps, 0.157 with 4, and 0.55 in the block kernel.
-//  * More blocks: 4 steps leave room for two blocks an SM (up to 8 nodes): 9000
-//    paths 0.207 ms, 0.267 with 8 steps.
-//  * Up to three waves of resident blocks, one wave below 24 rates, where the
-//    block kernel's threads are short: N = 40, 29,000 paths 0.59 against 0.65 ms,
-//    38,912 paths 0.79 against 0.66; N = 10, 9000 paths 0.058 against 0.095,
-//    20,000 paths 0.126 against 0.103; N = 120 (one block an SM), 4096 paths 0.83
-//    against 3.1, 16,384 paths 3.29 against 3.11.
-int pipe_steps(int scheme, int QP, int n, int s, int S, uint64_t tiles, int sms, size_t *smem)
+// The pipeline's shape for `tiles` blocks of 32 paths: B steps per block and 2^lg
+// warps, as B | lg << 8; 0 where the block kernel is the better one or shared
+// memory does not hold the pipeline.  Full scheme, ms:
+//  * One block an SM: eight warps and as many steps as the registers of the
+//    products and of the rows in work allow (8 or 5 up to 8 nodes, 4 up to 16,
+//    else 2), preferring a divisor of the steps per period: 4096 paths of N = 40
+//    0.119 with 8 steps, 0.158 with 4, and 0.56 in the block kernel.
+//  * More blocks, 24 rates and more: 4 steps leave room for two blocks an SM (up
+//    to 8 nodes), 9000 paths 0.209 (0.233 with 8 steps, 0.231 with four warps);
+//    up to three waves: 29,000 paths 0.59 against 0.65, 38,000 paths 0.78 against
+//    0.66; N = 120 (one block an SM), 4096 paths 0.74 against 2.74, 9000 paths
+//    1.45, 16,000 paths 2.88 against 2.74.
+//  * Fewer rates: fewer warps a block, and more blocks an SM, in one wave.  N = 10
+//    (4 nodes), 10,000 paths: 0.083 with eight warps, 0.053 with four, against
+//    0.098; 20,000 paths 0.073 with two against 0.103; 30,000 paths 0.090 against
+//    0.107; 40,000 paths 0.128 against 0.120.  The heavy-tailed example (32
+//    nodes): 5000 paths 0.081, 0.045 with four, against 0.086; 10,000 paths 0.054
+//    with two against 0.087; 20,000 paths 0.095 against 0.102.
+int pipe_shape(int scheme, int QP, int n, int s, int S, uint64_t tiles, int sms, size_t *smem)
 {
-    const int G = 1 << pipe_lg_warps(n), nst = scheme == PICARD ? 2 : 1;
-    const bool pairs = QP <= 8 && tiles > (uint64_t)sms; // two blocks an SM
-    int B = QP <= 8 ? (pairs ? 4 : s % 8 == 0 ? 8 : s % 5 == 0 ? 5 : 4) : QP <= 16 ? 4 : 2;
-    *smem = pipe_smem_bytes(QP, B, nst, n, S, G);
+    const int nst = scheme == PICARD ? 2 : 1;
+    const uint64_t per_sm = (tiles + sms - 1) / sms; // blocks an SM
+    int B = QP <= 8 ? (per_sm > 1 ? 4 : s % 8 == 0 ? 8 : s % 5 == 0 ? 5 : 4) : QP <= 16 ? 4 : 2;
+    int most = 8; // warps
+    if (n < 24 && per_sm > 1) {
+        most = per_sm <= (QP <= 8 ? 4 : 2) ? 4 : 2;
+        if (per_sm > (QP <= 8 ? 8 : 6)) return 0;
+    }
+    int lg = 0;
+    while ((2 << lg) <= n && (2 << lg) <= most) ++lg;
+    *smem = pipe_smem_bytes(QP, B, nst, n, S, 1 << lg);
     if (QP > 8 && B == 4 && *smem > 227 * 1024) {
         B = 2;
-        *smem = pipe_smem_bytes(QP, B, nst, n, S, G);
+        *smem = pipe_smem_bytes(QP, B, nst, n, S, 1 << lg);
     }
-    if (*smem > 227 * 1024) return 0;
-    const uint64_t wave = (uint64_t)sms * (pairs && *smem <= 113 * 1024 ? 2 : 1);
-    return tiles <= wave * (n >= 24 ? 3 : 1) ? B : 0;
+    const uint64_t room = 227 * 1024 / *smem; // blocks an SM by shared memory
+    if (room < 1 || (n < 24 && per_sm > room)) return 0;
+    if (n >= 24 && per_sm > 3 * (QP <= 8 && B == 4 && room >= 2 ? 2 : 1)) return 0;
+    return B | lg << 8;
 }
 
-int launch_pipe_kernel(int scheme, int QP, int B, size_t smem, uint64_t paths, cudaStream_t st, const PathArgs &a)
+int launch_pipe_kernel(int scheme, int QP, int shape, size_t smem, uint64_t paths, cudaStream_t st, const PathArgs &a)
 {
+    const int B = shape & 255, lg = shape >> 8;
     PipeFn f = scheme == FULL ? pick_pipe<FULL>(QP, B) : scheme == PICARD ? pick_pipe<PICARD>(QP, B) : nullptr;
     if (!f) return (int)cudaErrorInvalidValue;
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
-    const int lg = pipe_lg_warps(a.n);
     f<<<(unsigned)((paths + 31) / 32), 32 << lg, smem, st>>>(a, lg);
     return (int)cudaGetLastError();
 }

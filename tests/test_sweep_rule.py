@@ -73,10 +73,12 @@ def test_short_for_ordinary_rules_and_none_where_it_does_not_stand(lll):
     # one node of the measure: the rule is that node
     one = lll.lll_sweep_rule([0.5], [1.0], 0.0, 2.0)
     assert len(one[0]) == 1 and abs(one[0][0] - 0.5) < 1e-14 and abs(one[1][0] - 1.0) < 1e-14 and one[2] == 4
-    # no Gauss rule of a signed measure; sums beyond any short rule; overflow
+    # no Gauss rule of a signed measure; a node next to 0; sums beyond any short rule; overflow
     V = W.copy()
     V[5] = -V[5]
-    for args in ((x, V, 0.0, 4.3), (x, W, 0.0, 1e3), (x, W, -1e300, 1e300)):
+    y = x.copy()
+    y[np.argmin(np.abs(x))] = 3e-5
+    for args in ((x, V, 0.0, 4.3), (y, W, 0.0, 4.3), (x, W, 0.0, 1e3), (x, W, -1e300, 1e300)):
         xr, wr, padded = lll.lll_sweep_rule(*args)
         assert len(xr) == 0 and padded == 64
     with pytest.raises(lll.LLLError):
