@@ -285,7 +285,7 @@ def run_batch(args, steps, warmup, with_cpu=True, with_e2e=True, rates=None):
         x, W = lll.lll_build_nig_quadrature(wl.alpha, wl.beta, wl.dbar, wl.a, wl.Q)
         inst.append((wl, x, W))
     units = sum(wl.paths * wl.units_per_path() for wl in wls)          # per scheme
-    lane_ops = sum(wl.paths * wl.units_per_path() * 3 * wl.Q for wl in wls)
+    lane_ops = sum(wl.paths * wl.units_per_path() * 3 * _nodes(lll, wl, x, W) for wl, x, W in inst)
     caplets = sum(wl.n * wl.strikes.shape[1] for wl in wls)
     b, keep = lll.lll_batch_init(inst)  # default stream, the one torch's events record on
     own = args.workload == "batch256"  # not the batch256 block of the default run
@@ -343,7 +343,7 @@ def run_batch(args, steps, warmup, with_cpu=True, with_e2e=True, rates=None):
     ach = lane_ops / (statistics.mean(kernel_ms[dom]) * 1e-3) / 1e12
     roofline = {"bound": "alu", "achieved": ach, "peak": pk["fp32"], "unit": "TFP32-lane-op/s",
                 "frac": ach / pk["fp32"], "frac_of_nominal_128_lanes": ach / pk["fp32_nominal"], "traffic": None,
-                "kernel": f"batch_kernel ({dom}), 3Q FP32 lane-ops per unit, Q=64",
+                "kernel": f"batch_kernel ({dom}), 3Q FP32 lane-ops per unit, Q the nodes swept per instance",
                 "peak_basis": pk["fp32_basis"]}
 
     # end to end through the C ABI from host arrays: batch init (instance inputs
@@ -605,7 +605,7 @@ def run_single(args, wl, schemes, steps, warmup, dev, rank, world, local, with_c
             per[f"{s}_vs_full_max_bp"] = float(np.abs(pv - pf).max() * 1e4)
 
     # Rooflines.  Quadrature kernels: 3Q FP32 lane-ops per unit (one FMA into
-    # A, one multiply w*E, one FMA into P) against the measured packed-FMA
+    # A, one multiply w*E, one FMA into P), Q the nodes they sweep, against the measured packed-FMA
     # rate.  MLP kernels: one tanh.approx per SiLU against the measured MUFU
     # rate (the binding pipe), with the tensor rate (2 x multiply-adds of the
     # network) beside it against the measured sustained BF16 rate.
@@ -615,17 +615,18 @@ def run_single(args, wl, schemes, steps, warmup, dev, rank, world, local, with_c
 
     def quad_roofline(s):
         ms = statistics.mean(per_scheme_ms[s])
-        ach = units * 3 * wl.Q / (ms * 1e-3) / 1e12
         shape = tuned.get(s, {}).get("launch(threads,bps,chunk,ppt,lanes[,tenor])")
         lanes = shape[4] if shape and shape[4] else 1
         ppt = shape[3] if shape and shape[3] else 1
         tenor = shape[5] if shape and len(shape) > 5 else 0
-        key = f"{s}/QP{wl.Q}/lanes{lanes}" + (f"/ppt{ppt}" if ppt > 1 else "")
+        q = _nodes(lll, wl, x, W, given=tenor > 0 or lanes > 1)
+        ach = units * 3 * q / (ms * 1e-3) / 1e12
+        key = f"{s}/QP{q}/lanes{lanes}" + (f"/ppt{ppt}" if ppt > 1 else "")
         traffic = (_traffic(key) if wl.paths == 1 << 20 and not tenor else None)
         r = {"bound": "alu", "achieved": ach, "peak": pk["fp32"], "unit": "TFP32-lane-op/s",
              "frac": ach / pk["fp32"], "frac_of_nominal_128_lanes": ach / pk["fp32_nominal"], "traffic": traffic,
-             "kernel": (f"{s} tenor-parallel kernel ({tenor} lanes per path), QP={wl.Q}" if tenor
-                        else f"{s} path kernel, QP={wl.Q}"), "peak_basis": pk["fp32_basis"]}
+             "kernel": (f"{s} tenor-parallel kernel ({tenor} lanes per path), QP={q}" if tenor > 0
+                        else f"{s} path kernel, QP={q} (rule as given: {wl.Q})"), "peak_basis": pk["fp32_basis"]}
         if clocks and clocks.get("sm_mhz"):
             r["frac_at_sampled_clock"] = r["frac"] * pk["sm_max_mhz"] / clocks["sm_mhz"]
         return r
@@ -762,7 +763,7 @@ def run_mappings(args, rates=None):
 
     dev = torch.device("cuda", 0)
     pk = _alu_peaks(lll, torch, dev, rates)
-    shapes = [("path, 128 threads", (128, 0, 0, 1, 1)), ("path, 256 threads", (256, 0, 0, 1, 1)),
+    shapes = [("default", (0, 0, 0, 0, 0)), ("path, 128 threads", (128, 0, 0, 1, 1)), ("path, 256 threads", (256, 0, 0, 1, 1)),
               ("path, 2 paths/thread", (128, 0, 0, 2, 1))] + \
              [(f"tenor, {g} lanes/path", (0, 0, 0, 0, 0, g)) for g in (4, 8, 16, 32)] + \
              [("step-parallel (Picard)", (0, 0, 0, 0, 0, -1))]
@@ -785,14 +786,25 @@ def run_mappings(args, rates=None):
                         sim.simulate(scheme)
                         ms.append(sim.kernel_ms()[0])
                     t = statistics.median(ms)
-                    ach = paths * wl.units_per_path() * 3 * wl.Q / (t * 1e-3) / 1e12
-                    rows.append({"paths": paths, "scheme": scheme, "mapping": name, "kernel_ms": t,
+                    q = _nodes(lll, wl, x, W, given=name.startswith("tenor"))
+                    ach = paths * wl.units_per_path() * 3 * q / (t * 1e-3) / 1e12
+                    rows.append({"paths": paths, "scheme": scheme, "mapping": name, "kernel_ms": t, "nodes": q,
                                  "units_per_s": paths * wl.units_per_path() / (t * 1e-3),
                                  "fp32_frac": ach / pk["fp32"]})
         finally:
             sim.close()
     return {"metric": "path-kernel device time per mapping", "workload": "large_single (N=40, Q=64)",
             "fp32_peak_basis": pk["fp32_basis"], "rows": rows}
+
+
+def _nodes(lll, wl, x, W, given=False):
+    """Nodes per unit that the full and Picard sweeps process for the rule (x, W) of ``wl``:
+    those of its shorter equivalent, or (``given``: lane groups, tenor-parallel) its own."""
+    if given:
+        return wl.Q
+    i = np.arange(1, wl.n + 1) * wl.s
+    lam = np.where(np.arange(wl.steps)[:, None] < i[None, :], wl.lam, 0.0)
+    return lll.lll_sweep_rule(x, W, np.minimum(lam, 0.0).sum(axis=1).min(), np.maximum(lam, 0.0).sum(axis=1).max())[2]
 
 
 def run_by_length(args, rates=None):
@@ -833,7 +845,7 @@ def run_by_length(args, rates=None):
                     sim.simulate(scheme)
                     ms.append(sim.kernel_ms()[0])
                 t = statistics.median(ms)
-                ach = paths * wl.units_per_path() * 3 * wl.Q / (t * 1e-3) / 1e12
+                ach = paths * wl.units_per_path() * 3 * _nodes(lll, wl, x, W) / (t * 1e-3) / 1e12
                 row[scheme] = {"kernel_ms": t, "units_per_s": paths * wl.units_per_path() / (t * 1e-3),
                                "fp32_frac": ach / pk["fp32"]}
             rows.append(row)

@@ -22,7 +22,10 @@ from . import lll
 CACHE = os.path.join(_build.BUILD, "autotune.json")
 
 DEFAULT_CANDIDATES = [
-    # (threads, blocks_per_sm, chunk_rows, paths_per_thread, lanes_per_path[, tenor lanes])
+    # (threads, blocks_per_sm, chunk_rows, paths_per_thread, lanes_per_path[, tenor lanes]);
+    # all zero: the library's own choice, which for few paths is the pipeline over the rates
+    (0, 0, 0, 0, 0)
+] + [
     (t, 0, c, 1, l) for t, c, l in itertools.product((64, 128, 256), (0, 16), (1, 2, 4))
 ] + [(t, 0, c, 2, 1) for t, c in itertools.product((64, 128), (0, 16))] \
   + [(0, 0, 0, 0, 0, g) for g in (4, 8, 16, 32, -1)]
