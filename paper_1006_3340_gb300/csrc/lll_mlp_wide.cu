@@ -410,6 +410,14 @@ __global__ void __launch_bounds__(kThreadsW, 1)
                     if (mlo >= 1 && mlo >= imin && mhi <= n) chunk(std::integral_constant<int, 0>{}, ro[i & 1], c8, i);
                     else if (mlo >= 1 && mhi < imin && mhi <= n) chunk(std::integral_constant<int, 1>{}, ro[i & 1], c8, i);
                     else if (mlo <= n || (feat && c8 < KB0 * 8)) chunk(std::integral_constant<int, 2>{}, ro[i & 1], c8, i);
+                    // feature columns 0 .. 63 are complete: the next first layer starts on
+                    // them (into the other accumulator) under the second half of the rates
+                    // (N = 120, 50,000 paths: 19.9 -> 19.6 ms)
+                    if (i == 1 && feat) {
+                        fence_async_smem();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&actb[0]);
+                    }
                 }
                 // the accumulator has been read; the feature chunks are written
                 if (feat) {
@@ -417,7 +425,7 @@ __global__ void __launch_bounds__(kThreadsW, 1)
                     tc_before();
                     __syncwarp();
                     if (lane == 0)
-                        for (int j = 0; j < KB0; ++j) mbar_arrive(&actb[j]);
+                        for (int j = 1; j < KB0; ++j) mbar_arrive(&actb[j]);
                 } else {
                     tc_before();
                 }
