@@ -229,7 +229,7 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
         e = (cudaError_t)group_kernel_prepare(scheme, QPk, lpp, smem, T, &occ);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "group kernel attributes");
     } else if (block) {
-        e = (cudaError_t)block_kernel_prepare(scheme, ctx->QR, R, smem, T, &occ);
+        e = (cudaError_t)block_kernel_prepare(scheme, ctx->QR, R, paths, smem, T, &occ);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "block kernel attributes");
     } else {
         e = (cudaError_t)path_kernel_prepare(scheme, QPk, R, T, smem);

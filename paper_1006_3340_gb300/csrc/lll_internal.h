@@ -86,7 +86,7 @@ size_t path_kernel_smem(int QP, int n, int ns, int threads, int chunk_rows);
 // QMAX = 8 or 32).
 int block_chunk_rates(int QP, int R, int n, int rows);
 size_t block_kernel_smem(int QP, int R, int n, int threads, int chunk_rates);
-int block_kernel_prepare(int scheme, int QP, int R, size_t smem, int threads, int *blocks_per_sm);
+int block_kernel_prepare(int scheme, int QP, int R, uint64_t paths, size_t smem, int threads, int *blocks_per_sm);
 int launch_block_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st,
                         const PathArgs &a);
 int batch_block_prepare(int scheme, int QMAX, int R, size_t smem, int threads, int *blocks_per_sm);

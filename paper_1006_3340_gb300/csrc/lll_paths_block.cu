@@ -29,15 +29,15 @@ __host__ __device__ constexpr int steps_of(int QP, int R)
 }
 
 // Blocks of 256 threads per SM the registers are budgeted for.  (With 20 nodes
-// and four steps the Picard kernel gains by 128 registers, 15.6 -> 14.0 ms, and
-// the full one loses, 13.4 -> 14.8.)
+// and four steps the Picard kernel gains by 128 registers, 15.6 -> 14.0 ms; the
+// full one from kManyPaths on.)
 __host__ __device__ constexpr int blocks_of(int scheme, int QP, int R)
 {
     return R * steps_of(QP, R) * QP <= 64 || (scheme == PICARD && R == 1 && QP == 20) ? 2 : 1;
 }
 
-template <int SCHEME, int QP, int R>
-__global__ void __launch_bounds__(kMaxThreads, blocks_of(SCHEME, QP, R)) block_kernel(const PathArgs a)
+template <int SCHEME, int QP, int R, int BL = blocks_of(SCHEME, QP, R)>
+__global__ void __launch_bounds__(kMaxThreads, BL) block_kernel(const PathArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int B = steps_of(QP, R), NST = (SCHEME == PICARD) ? 2 : 1;
@@ -109,6 +109,14 @@ __global__ void __launch_bounds__(kMaxThreads, blocks_of(FULL, QMAX > 8 ? 24 : 8
 }
 
 typedef void (*KernelFn)(const PathArgs);
+
+// The full scheme on 20 nodes runs as well in two blocks of 128 threads an SM at
+// 192 registers as in four at 128 (a wave of 38,912 paths 3.9 ms, of 77,824 paths
+// 7.4); the two differ by how many paths the last wave is short of, and from here
+// on the larger wave wins throughout: N = 120, 140,000 paths 14.8 against 15.5 ms,
+// 2^20 paths 99.7 against 108.7.  (Below, either may: 116,000 paths 12.9 against
+// 11.6, 55,000 paths 6.0 against 7.7.)
+constexpr uint64_t kManyPaths = 140000;
 typedef void (*BatchFn)(const BatchArgs);
 
 template <int SCHEME, int R>
@@ -126,8 +134,9 @@ KernelFn pick_qp(int QP)
     }
 }
 
-KernelFn pick(int scheme, int QP, int R)
+KernelFn pick(int scheme, int QP, int R, uint64_t paths)
 {
+    if (scheme == FULL && QP == 20 && R == 1 && paths >= kManyPaths) return block_kernel<FULL, 20, 1, 2>;
     if (scheme == FULL) return R == 1 ? pick_qp<FULL, 1>(QP) : R == 2 ? pick_qp<FULL, 2>(QP) : nullptr;
     if (scheme == PICARD) return R == 1 ? pick_qp<PICARD, 1>(QP) : R == 2 ? pick_qp<PICARD, 2>(QP) : nullptr;
     return nullptr;
@@ -167,14 +176,14 @@ size_t block_kernel_smem(int QP, int R, int n, int threads, int chunk_rates)
     return block_smem_bytes(QP, steps_of(QP, R), R, n, threads, chunk_rates);
 }
 
-int block_kernel_prepare(int scheme, int QP, int R, size_t smem, int threads, int *blocks_per_sm)
+int block_kernel_prepare(int scheme, int QP, int R, uint64_t paths, size_t smem, int threads, int *blocks_per_sm)
 {
-    return prepare(pick(scheme, QP, R), smem, threads, blocks_per_sm);
+    return prepare(pick(scheme, QP, R, paths), smem, threads, blocks_per_sm);
 }
 
 int launch_block_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st, const PathArgs &a)
 {
-    KernelFn f = pick(scheme, QP, R);
+    KernelFn f = pick(scheme, QP, R, a.paths);
     if (!f) return (int)cudaErrorInvalidValue;
     f<<<grid, threads, smem, st>>>(a);
     return (int)cudaGetLastError();
