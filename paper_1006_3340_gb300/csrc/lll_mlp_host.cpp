@@ -182,13 +182,22 @@ int ensure_rows(lll_ctx *ctx, MlpState *m, int rows)
 // What a backward pass over `rows` (at most cap) rows needs besides.
 int ensure_grads(lll_ctx *ctx, MlpState *m, int rows)
 {
-    if (!m->side) {
-        MTRY(cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking));
-        for (int l = 0; l <= m->layers + 1; ++l) {
-            cudaEvent_t e;
-            MTRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-            m->ready.push_back(e);
+    if (!m->side) { // the stream with all its events, or neither
+        cudaStream_t side = nullptr;
+        std::vector<cudaEvent_t> ready;
+        cudaError_t e = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking);
+        while (e == cudaSuccess && (int)ready.size() < m->layers + 2) {
+            cudaEvent_t ev = nullptr;
+            e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+            if (e == cudaSuccess) ready.push_back(ev);
         }
+        if (e != cudaSuccess) {
+            for (cudaEvent_t ev : ready) cudaEventDestroy(ev);
+            if (side) cudaStreamDestroy(side);
+            return cerr(ctx, e, "side stream and events");
+        }
+        m->side = side;
+        m->ready.swap(ready);
     }
     if (rows <= m->gcap) return LLL_OK;
     for (float *p : m->d_dZ) cudaFree(p);
