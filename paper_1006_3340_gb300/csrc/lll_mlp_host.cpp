@@ -224,6 +224,14 @@ int ensure_split(lll_ctx *ctx, MlpState *m, size_t floats)
     return LLL_OK;
 }
 
+// After a failed call: wait for what it enqueued on either stream.  Its copies may
+// still read or write the caller's arrays, and the next call uses the same buffers.
+void drain(lll_ctx *ctx, MlpState *m)
+{
+    if (m->side) cudaStreamSynchronize(m->side);
+    cudaStreamSynchronize(ctx->stream);
+}
+
 // Forward pass over `rows` rows already in d_X.  y != nullptr: also residual,
 // dL/dout and loss partials.
 int forward(lll_ctx *ctx, MlpState *m, int rows, const float *y)
@@ -370,6 +378,44 @@ float lambda_ref(const lll_ctx *ctx)
     return mx > 0 ? (float)(1.0 / mx) : 1.0f;
 }
 
+// lll_mlp_eval on checked arguments.
+int evaluate(lll_ctx *ctx, MlpState *m, const float *x, const float *y, int rows, float *out, float *grads, double *loss)
+{
+    int rc = ensure_rows(ctx, m, rows);
+    if (rc != LLL_OK) return rc;
+    cudaStream_t st = ctx->stream;
+    // the rows go over as given; the device pads them and rounds to BF16
+    const size_t given = (size_t)rows * m->in_dim;
+    if (given > m->xin_cap) {
+        cudaFree(m->d_xin);
+        m->d_xin = nullptr;
+        m->xin_cap = 0;
+        if (cudaMalloc((void **)&m->d_xin, 4 * given) != cudaSuccess) return err(ctx, LLL_ENOMEM, "feature rows");
+        m->xin_cap = given;
+    }
+    cudaError_t e = cudaMemcpyAsync(m->d_xin, x, 4 * given, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = (cudaError_t)mlp_pack_rows(m->d_xin, rows, m->in_dim, m->in_pad, m->d_X, st);
+    if (e == cudaSuccess && y)
+        e = cudaMemcpyAsync(m->d_Y, y, 4 * (size_t)rows * m->outputs, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && y && m->head) e = cudaMemsetAsync(m->d_kr, 0, 4 * (size_t)rows, st); // all rates live
+    if (e != cudaSuccess) return cerr(ctx, e, "staging feature rows");
+    rc = forward(ctx, m, rows, y ? m->d_Y : nullptr);
+    if (rc != LLL_OK) return rc;
+    if (grads) {
+        rc = backward(ctx, m, rows);
+        if (rc != LLL_OK) return rc;
+        MTRY(cudaMemcpyAsync(grads, m->d_g, 4 * m->n_params, cudaMemcpyDeviceToHost, st));
+    }
+    if (out) MTRY(cudaMemcpyAsync(out, m->d_out, 4 * (size_t)rows * m->outputs, cudaMemcpyDeviceToHost, st));
+    if (!(loss && y)) MTRY(cudaStreamSynchronize(st)); // reading the loss waits
+    if (loss && y) {
+        bool ok;
+        *loss = read_loss(ctx, m, rows, &ok);
+        if (!ok) return err(ctx, LLL_ECUDA, "loss readback");
+    }
+    return LLL_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -492,40 +538,9 @@ int lll_mlp_eval(lll_ctx *ctx, const float *x, const float *y, int rows, float *
     if (!ctx || !ctx->mlp) return err(ctx, LLL_ESTATE, "no network (lll_mlp_init first)");
     if (!x || rows < 1) return err(ctx, LLL_EINVAL, "need x and rows >= 1");
     if (grads && !y) return err(ctx, LLL_EINVAL, "gradients need targets");
-    MlpState *m = ctx->mlp;
-    int rc = ensure_rows(ctx, m, rows);
-    if (rc != LLL_OK) return rc;
-    cudaStream_t st = ctx->stream;
-    // the rows go over as given; the device pads them and rounds to BF16
-    const size_t given = (size_t)rows * m->in_dim;
-    if (given > m->xin_cap) {
-        cudaFree(m->d_xin);
-        m->d_xin = nullptr;
-        m->xin_cap = 0;
-        if (cudaMalloc((void **)&m->d_xin, 4 * given) != cudaSuccess) return err(ctx, LLL_ENOMEM, "feature rows");
-        m->xin_cap = given;
-    }
-    cudaError_t e = cudaMemcpyAsync(m->d_xin, x, 4 * given, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = (cudaError_t)mlp_pack_rows(m->d_xin, rows, m->in_dim, m->in_pad, m->d_X, st);
-    if (e == cudaSuccess && y)
-        e = cudaMemcpyAsync(m->d_Y, y, 4 * (size_t)rows * m->outputs, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && y && m->head) e = cudaMemsetAsync(m->d_kr, 0, 4 * (size_t)rows, st); // all rates live
-    if (e != cudaSuccess) return cerr(ctx, e, "staging feature rows");
-    rc = forward(ctx, m, rows, y ? m->d_Y : nullptr);
-    if (rc != LLL_OK) return rc;
-    if (grads) {
-        rc = backward(ctx, m, rows);
-        if (rc != LLL_OK) return rc;
-        MTRY(cudaMemcpyAsync(grads, m->d_g, 4 * m->n_params, cudaMemcpyDeviceToHost, st));
-    }
-    if (out) MTRY(cudaMemcpyAsync(out, m->d_out, 4 * (size_t)rows * m->outputs, cudaMemcpyDeviceToHost, st));
-    if (!(loss && y)) MTRY(cudaStreamSynchronize(st)); // reading the loss waits
-    if (loss && y) {
-        bool ok;
-        *loss = read_loss(ctx, m, rows, &ok);
-        if (!ok) return err(ctx, LLL_ECUDA, "loss readback");
-    }
-    return LLL_OK;
+    const int rc = evaluate(ctx, ctx->mlp, x, y, rows, out, grads, loss);
+    if (rc != LLL_OK) drain(ctx, ctx->mlp);
+    return rc;
 }
 
 int lll_mlp_train(lll_ctx *ctx, const lll_mlp_cfg *cfg, double *final_loss)
@@ -608,7 +623,7 @@ int lll_mlp_train(lll_ctx *ctx, const lll_mlp_cfg *cfg, double *final_loss)
         if (e != cudaSuccess) { cleanup(); return cerr(ctx, e, "gather"); }
         rc = forward(ctx, m, B, m->d_Y);
         if (rc == LLL_OK) rc = backward(ctx, m, B);
-        if (rc != LLL_OK) { cleanup(); return rc; }
+        if (rc != LLL_OK) { drain(ctx, m); cleanup(); return rc; }
         ++m->adam_t;
         e = (cudaError_t)mlp_adam(m->d_p, m->d_g, m->d_m, m->d_v, m->d_ph, m->n_params, lr, 0.9f, 0.999f,
                                   1e-8f, m->adam_t, st);

@@ -1,6 +1,8 @@
 """lll_mlp_eval's host code on a fake CUDA runtime (tests/host_helpers), on the
-CPU: what a failing call leaves behind.  An evaluation that could not create an
-event leaves a network that the next evaluation can use."""
+CPU: what a failing call leaves behind.  An evaluation whose n-th call fails
+reports it and returns with no work in flight on either of its streams (its
+copies read and write the caller's arrays); one that could not create an event
+leaves a network that the next evaluation can use."""
 import os
 import shutil
 import subprocess
@@ -29,4 +31,9 @@ def helper(tmp_path_factory):
 @pytest.mark.parametrize("n", range(1, 6))
 def test_failed_event_leaves_a_usable_network(helper, n):
     r = subprocess.run([helper, "events", str(n)], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, (r.returncode, r.stderr)
+
+
+def test_failed_call_returns_with_nothing_in_flight(helper):
+    r = subprocess.run([helper, "calls"], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, (r.returncode, r.stderr)
