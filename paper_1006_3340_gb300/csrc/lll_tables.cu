@@ -206,7 +206,10 @@ int launch_tables(const double *lam, const double *x, const double *W, int Q, in
 {
     const size_t smem = sizeof(double) * ((size_t)2 * kTabRates * Q + 2 * (size_t)Q);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // always the need of the longest rule: the limit is the kernel's, and another
+        // thread's launch (a context of its own) may need more than this one
+        constexpr int most = sizeof(double) * (2 * kTabRates * kMaxQP + 2 * kMaxQP);
+        const cudaError_t e = cudaFuncSetAttribute(tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e != cudaSuccess) return (int)e;
     }
     tables_kernel<<<S, 128, smem, st>>>(lam, x, W, Q, n, S / n, QP, h, c, w0, tab, cn, row, brow, Ctab, b0);
