@@ -153,7 +153,7 @@ int expand_occupancy(int order, size_t smem, int *blocks_per_sm)
 {
     void (*f)(const PathArgs, const float *, const float *, const float *) =
         order == 2 ? expand_kernel<2> : expand_kernel<1>;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, kT, smem);
 }

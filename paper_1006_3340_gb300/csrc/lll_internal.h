@@ -15,6 +15,16 @@ constexpr int kMaxQP = 128;
 // Maximum threads per block of the path kernels.
 constexpr int kMaxThreads = 256;
 
+// Shared memory a block may have.  A kernel's limit is set to it, never to one
+// launch's need: the limit is the kernel's, and a launch of the same kernel from
+// another thread may need more.  A need above `most` is refused, as by the device.
+constexpr size_t kMaxSmem = 227 * 1024;
+template <class F>
+cudaError_t allow_smem(F kernel, size_t need, size_t most = kMaxSmem)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(need > most ? need : most));
+}
+
 // Arguments of the path kernels (one simulation of one scheme).
 struct PathArgs {
     const float4 *tab;    // [S][n][QP/4]: (E_j .. E_j+3), E_lj = e^{lambda_l(t_k) x_j} - 1

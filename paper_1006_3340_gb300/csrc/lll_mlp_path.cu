@@ -332,7 +332,7 @@ int mlp_path_occupancy(int layers, int in_pad, size_t smem, int *blocks_per_sm)
 {
     MlpKernelFn f = pick_mlp(layers, in_pad / 16);
     if (!f) return (int)cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, kWarps * 32, smem);
 }

@@ -957,7 +957,7 @@ int mlp_tc_vec_occupancy(int layers, int in_pad, size_t smem, int *blocks_per_sm
 {
     TcKernelFn f = pick_tc_vec(layers, (in_pad + 63) / 64);
     if (!f) return (int)cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, kThreads, smem);
 }
@@ -988,7 +988,7 @@ int mlp_tc_occupancy(int layers, int in_pad, size_t smem, int *blocks_per_sm)
 {
     TcKernelFn f = pick_tc(layers, (in_pad + 63) / 64);
     if (!f) return (int)cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, kThreads, smem);
 }

@@ -562,7 +562,7 @@ int launch_mlp_wide(int layers, int in_pad, int outputs, int grid, cudaStream_t 
     }
     if (!make_tmap(&maps.w[layers], g.wh + g.off_wout, outputs, kHW, kHW, kOutW)) return (int)cudaErrorInvalidValue;
     const size_t smem = wide_layout(a.n, a.ns).total;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return (int)e;
     f<<<grid, kThreadsW, smem, st>>>(a, g, maps, acc);
     return (int)cudaGetLastError();

@@ -482,7 +482,7 @@ int batch_kernel_prepare(int scheme, int QP, int R, size_t smem, int threads, in
 {
     BatchFn f = pick_batch(scheme, QP, R);
     if (!f) return (int)cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem, kMaxSmem - 1024); // less its static shared memory
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }
@@ -507,7 +507,7 @@ int path_kernel_prepare(int scheme, int QP, int R, int threads, size_t smem)
 {
     KernelFn f = pick(scheme, QP, R, threads);
     if (!f) return (int)cudaErrorInvalidValue;
-    return (int)cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return (int)allow_smem(f, smem);
 }
 
 int path_kernel_occupancy(int scheme, int QP, int R, int threads, size_t smem, int *blocks_per_sm)

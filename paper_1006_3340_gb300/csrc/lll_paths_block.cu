@@ -152,13 +152,11 @@ BatchFn pick_batch(int scheme, int QMAX, int R)
     return R == 1 ? batch_block_kernel<PICARD, 32, 1> : batch_block_kernel<PICARD, 32, 2>;
 }
 
-// most: the shared memory allowed from now on (launches of the same kernel from
-// other threads may need more than this one's smem).
 template <class F>
 int prepare(F f, size_t smem, size_t most, int threads, int *blocks_per_sm)
 {
     if (!f) return (int)cudaErrorInvalidValue;
-    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    const cudaError_t e = allow_smem(f, smem, most);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }
@@ -180,7 +178,7 @@ size_t block_kernel_smem(int QP, int R, int n, int threads, int chunk_rates)
 
 int block_kernel_prepare(int scheme, int QP, int R, uint64_t paths, size_t smem, int threads, int *blocks_per_sm)
 {
-    return prepare(pick(scheme, QP, R, paths), smem, 227 * 1024, threads, blocks_per_sm);
+    return prepare(pick(scheme, QP, R, paths), smem, kMaxSmem, threads, blocks_per_sm);
 }
 
 int launch_block_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st, const PathArgs &a)
@@ -193,8 +191,8 @@ int launch_block_kernel(int scheme, int QP, int R, int grid, int threads, size_t
 
 int batch_block_prepare(int scheme, int QMAX, int R, size_t smem, int threads, int *blocks_per_sm)
 {
-    // (less its static shared memory)
-    return prepare(pick_batch(scheme, QMAX, R), smem, 226 * 1024, threads, blocks_per_sm);
+    // less its static shared memory
+    return prepare(pick_batch(scheme, QMAX, R), smem, kMaxSmem - 1024, threads, blocks_per_sm);
 }
 
 int launch_batch_block_kernel(int scheme, int QMAX, int R, int grid, int threads, size_t smem, cudaStream_t st,

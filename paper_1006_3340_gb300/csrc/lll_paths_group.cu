@@ -348,7 +348,7 @@ int group_kernel_prepare(int scheme, int QP, int G, size_t smem, int threads, in
 {
     GroupFn f = pick_group(scheme, QP, G);
     if (!f) return (int)cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }

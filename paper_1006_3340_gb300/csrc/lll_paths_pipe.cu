@@ -331,8 +331,7 @@ int launch_pipe_kernel(int scheme, int QP, int shape, size_t smem, uint64_t path
     const int B = shape & 255, lg = shape >> 8;
     PipeFn f = scheme == FULL ? pick_pipe<FULL>(QP, B) : scheme == PICARD ? pick_pipe<PICARD>(QP, B) : nullptr;
     if (!f) return (int)cudaErrorInvalidValue;
-    // always the most: another thread's launch of the same kernel may need more than this one
-    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    const cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return (int)e;
     f<<<(unsigned)((paths + 31) / 32), 32 << lg, smem, st>>>(a, lg);
     return (int)cudaGetLastError();

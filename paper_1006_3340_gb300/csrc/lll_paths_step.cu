@@ -288,7 +288,7 @@ int launch_step_chunk(int QP, bool shorter, const PathArgs &a, uint64_t chunk_fi
     sp_draw<<<blocks_of((size_t)S * Pc), kSpT, 0, st>>>(a, chunk_first, Pc, dH);
     sp_scan_y<<<blocks_of((size_t)n * Pc), kSpT, 0, st>>>(a, Pc, dH, Y);
     const size_t smem = step_sweep_smem(QP, n);
-    cudaError_t e = cudaFuncSetAttribute(sw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(sw, smem);
     if (e != cudaSuccess) return (int)e;
     sw<<<dim3(blocks_of((size_t)Pc), S), kSpT, smem, st>>>(a, Pc, Y, Bh);
     const auto scan_d = shorter ? sp_scan_d<true> : sp_scan_d<false>;

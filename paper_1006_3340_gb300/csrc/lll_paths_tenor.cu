@@ -370,7 +370,7 @@ int tenor_kernel_prepare(int scheme, int QP, int G, size_t smem, int *blocks_per
 {
     TenorFn f = pick_tenor(scheme, QP, G);
     if (!f) return (int)cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, kTenorThreads, smem);
 }
