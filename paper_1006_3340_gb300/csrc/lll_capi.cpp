@@ -71,7 +71,7 @@ cudaError_t dalloc(T **p, size_t count)
 void free_all(lll_ctx *c)
 {
     for (void *p : {(void *)c->d_tab, (void *)c->d_row, (void *)c->d_brow, (void *)c->d_cn, (void *)c->d_tab_full,
-                    (void *)c->d_row_full, (void *)c->d_cn_full, (void *)c->d_partials, (void *)c->d_sums,
+                    (void *)c->d_row_full, (void *)c->d_cn_full, (void *)c->d_C_full, (void *)c->d_partials, (void *)c->d_sums,
                     (void *)c->d_state, (void *)c->d_snap, (void *)c->d_err, (void *)c->d_K1, (void *)c->d_K2,
                     (void *)c->d_K3})
         dev_free(c, p);
@@ -103,25 +103,28 @@ int ensure_full_tables(lll_ctx *ctx)
     if (ctx->QR == ctx->QP || ctx->d_tab_full) return LLL_OK;
     const size_t rows = (size_t)ctx->S * ctx->n;
     float4 *tab = nullptr, *row = nullptr;
-    float *cn = nullptr;
+    float *cn = nullptr, *C = nullptr;
     cudaError_t e = dalloc(&tab, rows * (ctx->QP / 4));
     if (e == cudaSuccess) e = dalloc(&row, rows);
     if (e == cudaSuccess) e = dalloc(&cn, ctx->QP);
+    if (e == cudaSuccess) e = dalloc(&C, rows);
     const bool room = e == cudaSuccess;
     if (room)
         e = (cudaError_t)launch_tables(ctx->d_lam, ctx->d_x, ctx->d_W, ctx->Q, ctx->n, ctx->S, ctx->QP, ctx->h, ctx->c,
-                                       nullptr, tab, cn, row, nullptr, ctx->d_C, nullptr, ctx->stream);
+                                       nullptr, tab, cn, row, nullptr, C, nullptr, ctx->stream);
     if (e == cudaSuccess)
         e = (cudaError_t)launch_prefix(ctx->d_b0, ctx->n, ctx->S, ctx->h, nullptr, ctx->delta, row, nullptr, ctx->stream);
     if (e != cudaSuccess) {
         cudaFree(tab);
         cudaFree(row);
         cudaFree(cn);
+        cudaFree(C);
         return room ? cuda_fail(ctx, e, "tables of the given rule") : fail(ctx, LLL_ENOMEM, "tables of the given rule");
     }
     ctx->d_tab_full = tab;
     ctx->d_row_full = row;
     ctx->d_cn_full = cn;
+    ctx->d_C_full = C;
     return LLL_OK;
 }
 

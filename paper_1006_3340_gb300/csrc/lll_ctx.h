@@ -35,7 +35,9 @@ struct lll_ctx {
     // sweeps' rule is the given one.
     float4 *d_tab_full = nullptr, *d_row_full = nullptr;
     float *d_cn_full = nullptr;
-    float *d_C = nullptr; // [S][n]: C_l(t_k), the compensator at zero weights (FP64-built)
+    // [S][n]: C_l(t_k), the compensator at zero weights, summed in FP64: of the sweeps'
+    // rule (LLL_MLP), written by lll_init alone; of the rule as given (training targets)
+    float *d_C = nullptr, *d_C_full = nullptr;
     float *d_Z0 = nullptr, *d_L0 = nullptr, *d_c0 = nullptr, *d_strikes = nullptr;
     double *d_partials = nullptr, *d_sums = nullptr;
     size_t partials_cap = 0, sums_cap = 0;

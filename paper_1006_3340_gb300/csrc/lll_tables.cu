@@ -30,7 +30,7 @@ namespace {
 // are integrals of its generating function (lll_quadrature.cpp), C over [0,
 // lambda] alone.  short_rule: the sweeps' rule is a shorter one; its rows brow
 // then hold K' = -h C less the dot product at zero weights as sweep_dot forms it.
-// w0, b0 null: the table alone (rows of another rule of the same model).
+// w0, b0 null: the table and C alone (of another rule of the same model).
 constexpr int kTabRates = 32;
 
 __global__ void tables_kernel(const double *lam, const double *x, const double *W, int Q, int n, int s, int QP, double h,

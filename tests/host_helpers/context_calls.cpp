@@ -1,0 +1,133 @@
+// Test helper: the host code of the C ABI's contexts (lll_capi.cpp) on a fake
+// CUDA runtime and fake kernel launchers that record what they are asked, on the
+// CPU.  Built and run by tests/test_context_calls.py only; the first argument
+// names the check.  Exit code 0: as expected; otherwise a message on stderr.
+#include "../../paper_1006_3340_gb300/csrc/lll_capi.cpp"
+#include "../../paper_1006_3340_gb300/csrc/lll_quadrature.cpp"
+
+#include <cstdlib>
+
+namespace {
+struct Tables {
+    const void *tab, *Ctab;
+    int QP;
+};
+std::vector<Tables> g_tables;              // launches of the table kernel
+const void *g_path_tab = nullptr;          // table of the last path kernel
+long g_mallocs = 0, g_frees = 0, g_launches = 0, g_copies = 0;
+bool g_capturing = false;
+
+int check(bool ok, const char *what)
+{
+    if (!ok) std::fprintf(stderr, "%s\n", what);
+    return ok ? 0 : 1;
+}
+}  // namespace
+
+extern "C" {
+cudaError_t cudaMalloc(void **p, size_t bytes)
+{
+    ++g_mallocs;
+    *p = std::calloc(bytes, 1);
+    return *p ? cudaSuccess : cudaErrorMemoryAllocation;
+}
+cudaError_t cudaFree(void *p)
+{
+    g_frees += p != nullptr;
+    std::free(p);
+    return cudaSuccess;
+}
+cudaError_t cudaMemcpyAsync(void *dst, const void *src, size_t bytes, cudaMemcpyKind, cudaStream_t)
+{
+    ++g_copies;
+    std::memcpy(dst, src, bytes);
+    return cudaSuccess;
+}
+cudaError_t cudaMemcpy(void *dst, const void *src, size_t bytes, cudaMemcpyKind k) { return cudaMemcpyAsync(dst, src, bytes, k, nullptr); }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s)
+{
+    *s = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t *e) { return *e = (cudaEvent_t)std::malloc(1), cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t e) { return std::free(e), cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+const char *cudaGetErrorString(cudaError_t) { return "fake"; }
+}
+
+namespace lll {
+void mlp_free(MlpState *) {}
+bool path_kernel_supported(int, int, int) { return true; }
+size_t path_kernel_smem(int, int, int, int, int) { return 1024; }
+int path_kernel_prepare(int, int, int, int, size_t) { return 0; }
+int path_kernel_occupancy(int, int, int, int, size_t, int *b) { return *b = 4, 0; }
+int launch_path_kernel(int, int, int, int, int, size_t, cudaStream_t, const PathArgs &a) { return ++g_launches, g_path_tab = a.tab, 0; }
+int block_chunk_rates(int, int, int n, int) { return n; }
+size_t block_kernel_smem(int, int, int, int, int) { return 1024; }
+int block_kernel_prepare(int, int, int, uint64_t, size_t, int, int *b) { return *b = 4, 0; }
+int launch_block_kernel(int, int, int, int, int, size_t, cudaStream_t, const PathArgs &a) { return ++g_launches, g_path_tab = a.tab, 0; }
+int pipe_shape(int, int, int, int, int, uint64_t, int, size_t *) { return 0; }
+bool group_kernel_supported(int, int, int) { return true; }
+size_t group_kernel_smem(int, int, int, int, int) { return 1024; }
+int group_kernel_prepare(int, int, int, size_t, int, int *b) { return *b = 4, 0; }
+int launch_group_kernel(int, int, int, int, int, size_t, cudaStream_t, const PathArgs &a) { return ++g_launches, g_path_tab = a.tab, 0; }
+bool tenor_kernel_supported(int, int, int) { return true; }
+size_t tenor_kernel_smem(int, int, int, int) { return 1024; }
+int tenor_kernel_threads() { return 128; }
+int tenor_kernel_prepare(int, int, int, size_t, int *b) { return *b = 4, 0; }
+int launch_tenor_kernel(int, int, int, int, size_t, cudaStream_t, const PathArgs &a) { return ++g_launches, g_path_tab = a.tab, 0; }
+int launch_tables(const double *, const double *, const double *, int, int, int, int QP, double, double, const double *,
+                  float4 *tab, float *, float4 *, float4 *, float *Ctab, double *, cudaStream_t)
+{
+    ++g_launches;
+    g_tables.push_back({tab, Ctab, QP});
+    return 0;
+}
+int launch_prefix(const double *, int, int, double, const double *, double, float4 *, float4 *, cudaStream_t) { return ++g_launches, 0; }
+int launch_finalize(const double *, int, int, double *, cudaStream_t) { return ++g_launches, 0; }
+}  // namespace lll
+
+namespace {
+// A 9-rate model whose 32-node rule has a shorter equivalent.
+lll_ctx *model()
+{
+    const int N = 10, s = 2, n = N - 1, S = n * s, Q = 32;
+    std::vector<double> L0(N, 0.03), lam((size_t)S * n, 0.05), x(Q), W(Q), K(n * 3, 0.03);
+    const lll_nig nig{12.0, -3.0, 0.8, NAN};
+    lll_ctx *c = nullptr;
+    if (lll_build_nig_quadrature(nig, 1.5, Q, x.data(), W.data()) != LLL_OK ||
+        lll_init(&c, N, 0.5, L0.data(), s, lam.data(), LLL_DRIVER_NIG, nig, Q, x.data(), W.data(), (void *)&g_launches) != LLL_OK ||
+        lll_set_strikes(c, 3, K.data()) != LLL_OK || c->QR >= c->QP)
+        std::abort();
+    return c;
+}
+
+// The compensators that LLL_MLP reads are written by lll_init alone.
+int compensators()
+{
+    lll_ctx *c = model();
+    int bad = check(g_tables.size() == 1 && g_tables[0].Ctab == c->d_C, "lll_init writes C once");
+    for (int lanes : {8, 0}) {
+        if (lanes) lll_set_mapping(c, LLL_MAP_TENOR, lanes);
+        else lll_set_launch(c, 0, 0, 0, 0, 2);
+        bad += check(lll_simulate(c, LLL_PICARD, 0, 1000, 1) == LLL_OK, "simulate");
+        lll_set_mapping(c, LLL_MAP_PATH, 0);
+    }
+    bad += check(g_tables.size() > 1, "the rule as given has tables of its own");
+    for (size_t q = 1; q < g_tables.size(); ++q) bad += check(g_tables[q].Ctab != c->d_C, "C written by a selection");
+    lll_destroy(c);
+    return bad;
+}
+}  // namespace
+
+int main(int argc, char **argv)
+{
+    const std::string what = argc > 1 ? argv[1] : "";
+    if (what == "compensators") return compensators();
+    return 2;
+}
