@@ -70,10 +70,8 @@ cudaError_t dalloc(T **p, size_t count)
 
 void free_all(lll_ctx *c)
 {
-    for (void *p : {(void *)c->d_tab, (void *)c->d_row, (void *)c->d_brow, (void *)c->d_cn, (void *)c->d_tab_full,
-                    (void *)c->d_row_full, (void *)c->d_cn_full, (void *)c->d_C_full, (void *)c->d_partials, (void *)c->d_sums,
-                    (void *)c->d_state, (void *)c->d_snap, (void *)c->d_err, (void *)c->d_K1, (void *)c->d_K2,
-                    (void *)c->d_K3})
+    for (void *p : {(void *)c->d_partials, (void *)c->d_sums, (void *)c->d_state, (void *)c->d_snap,
+                    (void *)c->d_err, (void *)c->d_K1, (void *)c->d_K2, (void *)c->d_K3})
         dev_free(c, p);
     cudaFree(c->arena);
     mlp_free(c->mlp);
@@ -98,45 +96,32 @@ namespace lll {
 
 int record_error(lll_ctx *ctx, int code, const char *msg) { return fail(ctx, code, msg); }
 
+// In the room that lll_init keeps for them: no allocation, so the selections
+// that need them may come at any time, also while the stream is captured (the
+// two kernels are then part of the graph, and the next call outside builds them).
 int ensure_full_tables(lll_ctx *ctx)
 {
-    if (ctx->QR == ctx->QP || ctx->d_tab_full) return LLL_OK;
-    const size_t rows = (size_t)ctx->S * ctx->n;
-    float4 *tab = nullptr, *row = nullptr;
-    float *cn = nullptr, *C = nullptr;
-    cudaError_t e = dalloc(&tab, rows * (ctx->QP / 4));
-    if (e == cudaSuccess) e = dalloc(&row, rows);
-    if (e == cudaSuccess) e = dalloc(&cn, ctx->QP);
-    if (e == cudaSuccess) e = dalloc(&C, rows);
-    const bool room = e == cudaSuccess;
-    if (room)
-        e = (cudaError_t)launch_tables(ctx->d_lam, ctx->d_x, ctx->d_W, ctx->Q, ctx->n, ctx->S, ctx->QP, ctx->h, ctx->c,
-                                       nullptr, tab, cn, row, nullptr, C, nullptr, ctx->stream);
+    if (ctx->QR == ctx->QP || ctx->full_built) return LLL_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) cudaGetLastError();
+    cudaError_t e = (cudaError_t)launch_tables(ctx->d_lam, ctx->d_x, ctx->d_W, ctx->Q, ctx->n, ctx->S, ctx->QP, ctx->h,
+                                               ctx->c, nullptr, ctx->d_tab_full, ctx->d_cn_full, ctx->d_row_full, nullptr,
+                                               ctx->d_C_full, nullptr, ctx->stream);
     if (e == cudaSuccess)
-        e = (cudaError_t)launch_prefix(ctx->d_b0, ctx->n, ctx->S, ctx->h, nullptr, ctx->delta, row, nullptr, ctx->stream);
-    if (e != cudaSuccess) {
-        cudaFree(tab);
-        cudaFree(row);
-        cudaFree(cn);
-        cudaFree(C);
-        return room ? cuda_fail(ctx, e, "tables of the given rule") : fail(ctx, LLL_ENOMEM, "tables of the given rule");
-    }
-    ctx->d_tab_full = tab;
-    ctx->d_row_full = row;
-    ctx->d_cn_full = cn;
-    ctx->d_C_full = C;
+        e = (cudaError_t)launch_prefix(ctx->d_b0, ctx->n, ctx->S, ctx->h, nullptr, ctx->delta, ctx->d_row_full, nullptr,
+                                       ctx->stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "tables of the given rule");
+    ctx->full_built = cap == cudaStreamCaptureStatusNone;
     return LLL_OK;
 }
 
 int use_full_tables(lll_ctx *ctx)
 {
     const int rc = ensure_full_tables(ctx);
-    if (rc != LLL_OK || !ctx->d_tab_full) return rc;
-    ctx->d_tab = ctx->d_tab_full; // the shorter rule's stay in the arena, unused
+    if (rc != LLL_OK || ctx->QR == ctx->QP) return rc;
+    ctx->d_tab = ctx->d_tab_full;
     ctx->d_row = ctx->d_row_full;
     ctx->d_cn = ctx->d_cn_full;
-    ctx->d_tab_full = ctx->d_row_full = nullptr;
-    ctx->d_cn_full = nullptr;
     ctx->d_brow = nullptr;
     ctx->QR = ctx->QP;
     return LLL_OK;
@@ -247,7 +232,11 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     const int grid = (int)(pipe ? tiles : std::min<uint64_t>(tiles, (uint64_t)bps * ctx->sm_count));
     const int nst = (scheme == LLL_PICARD) ? 2 : 1;
     PathArgs a{};
-    const bool other = !block && ctx->d_tab_full;
+    const bool other = !given_rule && !block && QPk > 0 && ctx->QR < ctx->QP; // the rule as given (lane groups, tenor mapping)
+    if (other) {
+        const int rc = ensure_full_tables(ctx);
+        if (rc != LLL_OK) return rc;
+    }
     a.tab = other ? ctx->d_tab_full : ctx->d_tab;
     a.cn = other ? ctx->d_cn_full : ctx->d_cn;
     a.brow = ctx->d_brow;
@@ -393,7 +382,8 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
         cuda_fail(c, e, "cudaDeviceGetAttribute"); return bail(LLL_ECUDA);
     }
     // One arena: the inputs (one host image, one copy), then the tables, then
-    // strikes, sums and payoff scratch for the usual sizes.
+    // strikes, sums and payoff scratch for the usual sizes, and last room for the
+    // tables of a rule as given beside its shorter one's.
     const size_t rows = (size_t)S * n;
     size_t bytes = 0;
     auto place = [&](size_t size) {
@@ -410,6 +400,9 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
                  at_row = place(16 * rows), at_brow = place(Qr > 0 ? 16 * rows : 0), at_C = place(4 * rows),
                  at_strikes = place(4 * (size_t)n * 64), at_sums = place(16 * (size_t)n * 64),
                  at_part = place(kArenaPartials * 8);
+    const bool two = QR < QP;
+    const size_t at_tabf = place(two ? 4 * rows * QP : 0), at_rowf = place(two ? 16 * rows : 0),
+                 at_cnf = place(two ? 4 * (size_t)QP : 0), at_Cf = place(two ? 4 * rows : 0);
     std::vector<char> in(in_bytes);
     auto host = [&](size_t at) { return reinterpret_cast<double *>(in.data() + at); };
     std::memcpy(host(at_lam), lambda, 8 * rows);
@@ -443,6 +436,10 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
     c->sums_cap = 2 * (size_t)n * 64;
     c->d_partials = (double *)dev(at_part);
     c->partials_cap = kArenaPartials;
+    if (two) {
+        c->d_tab_full = (float4 *)dev(at_tabf); c->d_row_full = (float4 *)dev(at_rowf);
+        c->d_cn_full = (float *)dev(at_cnf); c->d_C_full = (float *)dev(at_Cf);
+    }
     for (auto &ev : c->ev)
         if ((e = cudaEventCreate(&ev)) != cudaSuccess) { cuda_fail(c, e, "cudaEventCreate"); return bail(LLL_ECUDA); }
     cudaStream_t st = c->stream;
@@ -521,10 +518,6 @@ int lll_set_launch(lll_ctx *ctx, int threads_per_block, int blocks_per_sm, int c
         return fail(ctx, LLL_EINVAL, "paths_per_thread must be 0 (automatic), 1 or 2");
     if (lanes_per_path != 0 && lanes_per_path != 1 && lanes_per_path != 2 && lanes_per_path != 4)
         return fail(ctx, LLL_EINVAL, "lanes_per_path must be 0 (default), 1, 2 or 4");
-    if (lanes_per_path > 1) {
-        const int rc = ensure_full_tables(ctx);
-        if (rc != LLL_OK) return rc;
-    }
     ctx->ppt = paths_per_thread;
     ctx->lpp = lanes_per_path;
     ctx->threads = threads_per_block;
@@ -549,8 +542,6 @@ int lll_set_mapping(lll_ctx *ctx, int mapping, int lanes)
     if (mapping != LLL_MAP_TENOR) return fail(ctx, LLL_EINVAL, "unknown mapping");
     if (lanes != 4 && lanes != 8 && lanes != 16 && lanes != 32)
         return fail(ctx, LLL_EINVAL, "lanes must be 4, 8, 16 or 32");
-    const int rc = ensure_full_tables(ctx);
-    if (rc != LLL_OK) return rc;
     ctx->tenor_lanes = lanes;
     ctx->step_map = false;
     return LLL_OK;

@@ -31,8 +31,9 @@ struct lll_ctx {
     float4 *d_brow = nullptr; // rows of the shorter rule (null where the given one is swept)
     float *d_cn = nullptr; // [QR]: c_j = W_j / x_j^2 (shorter rule: -h c_j)
     // The same for the rule as given (lane groups, the tenor-parallel mapping and
-    // training data), built when one of them is first selected; null where the
-    // sweeps' rule is the given one.
+    // training data), built by the first call that reads them (full_built); null
+    // where the sweeps' rule is the given one.
+    bool full_built = false;
     float4 *d_tab_full = nullptr, *d_row_full = nullptr;
     float *d_cn_full = nullptr;
     // [S][n]: C_l(t_k), the compensator at zero weights, summed in FP64: of the sweeps'

@@ -566,7 +566,7 @@ int lll_mlp_train(lll_ctx *ctx, const lll_mlp_cfg *cfg, double *final_loss)
     rc = plan_launch(ctx, LLL_FULL, 0, P, cfg->seed ^ 0x5EED5EEDull, &plan, false);
     if (rc == LLL_OK) rc = ensure_full_tables(ctx); // the targets are integrals of the rule as given
     if (rc != LLL_OK) return rc;
-    if (ctx->d_tab_full) {
+    if (ctx->QR < ctx->QP) {
         plan.args.tab = ctx->d_tab_full;
         plan.args.cn = ctx->d_cn_full;
         plan.args.row = ctx->d_row_full;
@@ -585,7 +585,7 @@ int lll_mlp_train(lll_ctx *ctx, const lll_mlp_cfg *cfg, double *final_loss)
         cleanup();
         return err(ctx, LLL_ENOMEM, "training data buffers");
     }
-    cudaError_t e = (cudaError_t)mlp_datagen(ctx->QP, plan.args, ctx->d_C_full ? ctx->d_C_full : ctx->d_C, R, (uint32_t)(cfg->seed * 2654435761u),
+    cudaError_t e = (cudaError_t)mlp_datagen(ctx->QP, plan.args, ctx->QR < ctx->QP ? ctx->d_C_full : ctx->d_C, R, (uint32_t)(cfg->seed * 2654435761u),
                                              state, rec_u, rec_y, rec_k, st);
     std::vector<double> hpart(mb);
     if (e == cudaSuccess) e = (cudaError_t)mlp_target_moments(rec_y, rec_k, nrec, n, ctx->s, part, mb, st);

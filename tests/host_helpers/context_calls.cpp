@@ -123,11 +123,44 @@ int compensators()
     lll_destroy(c);
     return bad;
 }
+// Selecting lane groups or a mapping makes no CUDA call; the first simulation
+// under the selection builds the tables that it needs without allocating, and
+// once.  Built in a capture they belong to the graph: the next call builds them.
+int selections()
+{
+    int bad = 0;
+    for (int capture = 0; capture < 2; ++capture)
+        for (int lanes : {8, 0}) {
+            lll_ctx *c = model();
+            bad += check(lll_simulate(c, LLL_PICARD, 0, 100000, 1) == LLL_OK, "scratch of a larger call");
+            const void *sweeps = g_path_tab;
+            const long mallocs = g_mallocs, launches = g_launches, copies = g_copies;
+            g_tables.clear();
+            g_capturing = capture;
+            const int rc = lanes ? lll_set_mapping(c, LLL_MAP_TENOR, lanes) : lll_set_launch(c, 0, 0, 0, 0, 2);
+            bad += check(rc == LLL_OK && g_mallocs == mallocs && g_launches == launches && g_copies == copies, "a selection called CUDA");
+            for (int call = 0; call < 2; ++call) {
+                bad += check(lll_simulate(c, LLL_PICARD, 0, 1000, 1) == LLL_OK, "simulate");
+                bad += check(g_mallocs == mallocs, "a simulation under a selection allocated");
+                bad += check(!g_tables.empty() && g_path_tab == g_tables[0].tab && g_path_tab != sweeps, "not the given rule's table");
+                bad += check((int)g_tables.size() == (capture ? call + 1 : 1), "table launches");
+            }
+            g_capturing = false;
+            bad += check(lll_simulate(c, LLL_PICARD, 0, 1000, 1) == LLL_OK && g_path_tab == g_tables[0].tab, "simulate");
+            bad += check((int)g_tables.size() == (capture ? 3 : 1), "tables of a capture taken as built");
+            lll_set_mapping(c, LLL_MAP_PATH, 0);
+            lll_set_launch(c, 0, 0, 0, 0, 0);
+            bad += check(lll_simulate(c, LLL_PICARD, 0, 1000, 1) == LLL_OK && g_path_tab == sweeps, "set back");
+            lll_destroy(c);
+        }
+    return bad;
+}
 }  // namespace
 
 int main(int argc, char **argv)
 {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "compensators") return compensators();
+    if (what == "selections") return selections();
     return 2;
 }

@@ -1,5 +1,5 @@
 """What a context was asked before must not change what it answers: selecting a
-mapping and setting it back."""
+mapping and setting it back, and the same selections inside a stream capture."""
 import numpy as np
 import pytest
 
@@ -46,3 +46,37 @@ def test_learned_drift_prices_do_not_depend_on_earlier_selections(env, maker, hi
         sim.close()
     assert np.array_equal(z, z2, equal_nan=True)
     assert np.array_equal(sums[0], sums2[0]) and np.array_equal(sums[1], sums2[1])
+
+
+@pytest.mark.parametrize("how", ["tenor", "lanes"])
+def test_selection_inside_a_capture(env, how):
+    """The selection and the simulation captured into one graph: the graph gives the
+    sums of the same calls outside, and the context is sound afterwards."""
+    torch, lll = env
+    wl = workloads.large_single(paths=3000)
+    stream = torch.cuda.Stream()
+    ref, sim = lll.LevyLibor(wl), lll.LevyLibor(wl, stream=stream.cuda_stream)
+    out = torch.zeros((wl.n, wl.strikes.shape[1], 2), dtype=torch.float64, device="cuda")
+    noalloc = lambda s, seed: lll.lll_simulate_noalloc(s.ctx, lll.LLL_PICARD, 0, wl.paths, seed, out.data_ptr())  # noqa: E731
+    try:
+        SELECT[how](ref)
+        ref.simulate("picard", seed=5)
+        want = ref.sums()
+        noalloc(sim, 1)  # finds the scratch array
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            SELECT[how](sim)
+            noalloc(sim, 5)
+        for _ in range(2):
+            out.fill_(float("nan"))
+            graph.replay()
+            torch.cuda.synchronize()
+            assert np.allclose(out[..., 0].cpu().numpy(), want[0], rtol=1e-12, atol=0)
+            assert np.allclose(out[..., 1].cpu().numpy(), want[1], rtol=1e-12, atol=0)
+        sim.simulate("picard", seed=5)
+        got = sim.sums()
+        assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+    finally:
+        ref.close()
+        sim.close()
