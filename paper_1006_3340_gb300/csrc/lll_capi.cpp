@@ -217,7 +217,7 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
         e = (cudaError_t)group_kernel_prepare(scheme, QPk, lpp, smem, T, &occ);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "group kernel attributes");
     } else if (block) {
-        e = (cudaError_t)block_kernel_prepare(scheme, ctx->QR, R, paths, smem, T, &occ);
+        e = (cudaError_t)block_kernel_prepare(scheme, ctx->product, ctx->QR, R, paths, smem, T, &occ);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "block kernel attributes");
     } else {
         e = (cudaError_t)path_kernel_prepare(scheme, QPk, R, T, smem);
@@ -251,6 +251,7 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     a.h = (float)ctx->h; a.sqrt_h = (float)std::sqrt(ctx->h); a.delta = (float)ctx->delta;
     a.dBN = (float)(ctx->delta * ctx->BN);
     a.product = ctx->product;
+    a.wide_strikes = ctx->wide_strikes;
     if (ctx->driver == LLL_DRIVER_NIG) {
         const double m = ctx->nig.delta * ctx->h / ctx->gam;
         const double l = (ctx->nig.delta * ctx->h) * (ctx->nig.delta * ctx->h);
@@ -478,14 +479,17 @@ int lll_set_strikes(lll_ctx *ctx, int n_strikes, const double *strikes)
     if (n_strikes < 1 || n_strikes > 64 || !strikes) return fail(ctx, LLL_EINVAL, "need 1..64 strikes");
     const size_t cnt = (size_t)ctx->n * n_strikes;
     std::vector<float> f(cnt);
+    bool wide = false;
     for (size_t e = 0; e < cnt; ++e) {
         if (!isfin(strikes[e])) return fail(ctx, LLL_EINVAL, "strike is NaN/Inf");
         f[e] = (float)strikes[e];
+        wide = wide || !(std::fabs(strikes[e]) < kPairStrike);
     }
     CUDA_TRY(ctx, cudaMemcpyAsync(ctx->d_strikes, f.data(), sizeof(float) * cnt, cudaMemcpyHostToDevice,
                                   ctx->stream));
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
     ctx->ns = n_strikes;
+    ctx->wide_strikes = wide;
     ctx->simulated = false;
     return LLL_OK;
 }

@@ -47,6 +47,7 @@ struct lll_ctx {
     float *d_snap = nullptr;
     uint64_t n_snap = 0, snap_stride = 1;
     int ns = 0;
+    bool wide_strikes = false; // some strike is of kPairStrike or more
     int product = 0; // LLL_PRODUCT_*
     bool simulated = false;
     uint64_t last_paths = 0;

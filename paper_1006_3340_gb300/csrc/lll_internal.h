@@ -25,6 +25,9 @@ cudaError_t allow_smem(F kernel, size_t need, size_t most = kMaxSmem)
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(need > most ? need : most));
 }
 
+// Strikes up to which swaption payoffs may be formed in pairs of FP32 numbers.
+constexpr double kPairStrike = 1e3;
+
 // Arguments of the path kernels (one simulation of one scheme).
 struct PathArgs {
     const float4 *tab;    // [S][n][QP/4]: (E_j .. E_j+3), E_lj = e^{lambda_l(t_k) x_j} - 1
@@ -46,6 +49,7 @@ struct PathArgs {
     int driver;           // 0 NIG, 1 Brownian
     float h, sqrt_h, delta, dBN; // dBN = delta * B(0, T_N)
     int product;          // 0: caplets, 1: co-terminal payer swaptions (see lll_device.cuh)
+    int wide_strikes;     // some strike is of kPairStrike or more (see beyond_pairs in lll_device.cuh)
     // NIG increment over one step: IG(mean m, shape l) mixing variable.
     float ig_m, ig_m2, ig_hl, ig_fl; // m, m^2, m / (2 l), 4 m l
     float nig_beta, nig_muh;         // beta, mu * h
@@ -96,7 +100,7 @@ size_t path_kernel_smem(int QP, int n, int ns, int threads, int chunk_rows);
 // QMAX = 8 or 32).
 int block_chunk_rates(int QP, int R, int n, int rows);
 size_t block_kernel_smem(int QP, int R, int n, int threads, int chunk_rates);
-int block_kernel_prepare(int scheme, int QP, int R, uint64_t paths, size_t smem, int threads, int *blocks_per_sm);
+int block_kernel_prepare(int scheme, int product, int QP, int R, uint64_t paths, size_t smem, int threads, int *blocks_per_sm);
 int launch_block_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st,
                         const PathArgs &a);
 int batch_block_prepare(int scheme, int QMAX, int R, size_t smem, int threads, int *blocks_per_sm);

@@ -14,44 +14,10 @@
 // N = 40, 4096 paths 2.11 -> 0.66 ms (1.02).
 #include <cuda_runtime.h>
 
-#include "lll_device.cuh"
-#include "lll_internal.h"
-#include "lll_sweep.cuh"
+#include "lll_paths_block.cuh"
 
 namespace lll {
 namespace {
-
-// Steps per block for QP nodes and R paths per thread.  N = 120 (20 nodes, four
-// steps a period), 2^17 paths: 14.7 ms with two steps, 13.4 with four.
-__host__ __device__ constexpr int steps_of(int QP, int R)
-{
-    return R == 2 ? (QP <= 4 ? 8 : QP <= 8 ? 4 : QP <= 24 ? 2 : 1) : (QP <= 8 ? 8 : QP <= 20 ? 4 : 2);
-}
-
-// Blocks of 256 threads per SM the registers are budgeted for.  (With 20 nodes
-// and four steps the Picard kernel gains by 128 registers, 15.6 -> 14.0 ms; the
-// full one from kManyPaths on.)
-__host__ __device__ constexpr int blocks_of(int scheme, int QP, int R)
-{
-    return R * steps_of(QP, R) * QP <= 64 || (scheme == PICARD && R == 1 && QP == 20) ? 2 : 1;
-}
-
-template <int SCHEME, int QP, int R, int BL = blocks_of(SCHEME, QP, R)>
-__global__ void __launch_bounds__(kMaxThreads, BL) block_kernel(const PathArgs a)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int B = steps_of(QP, R), NST = (SCHEME == PICARD) ? 2 : 1;
-    const int T = blockDim.x, tid = threadIdx.x;
-    const BlockSmem sm = block_carve(smem_raw, QP, B, R, a.n, T, a.chunk_rows);
-    for (int e = tid; e < a.n; e += T) sm.c0[e] = -1.4426950408889634f * a.c0[e];
-    for (int e = tid; e < QP; e += T) reinterpret_cast<float *>(sm.cn)[e] = a.cn[e];
-    State<NST * R> *st = reinterpret_cast<State<NST * R> *>(a.state) + (size_t)blockIdx.x * a.n * T + tid;
-    const size_t nout = (size_t)a.n * a.ns * 2;
-    double *acc = a.partials + blockIdx.x * nout, *comp = a.partials + (gridDim.x + blockIdx.x) * nout;
-    const uint64_t TP = (uint64_t)T * R, ntiles = (a.paths + TP - 1) / TP;
-    for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-        block_tile<SCHEME, QP, B, R>(a, sm, st, tile, acc, comp, tile == blockIdx.x);
-}
 
 // A batch: the blocks claim items as in batch_kernel (lll_paths.cu), and take
 // each instance at its own rule's length, up to QMAX nodes.
@@ -65,8 +31,9 @@ __device__ __forceinline__ void batch_item(const PathArgs &a, unsigned char *sme
     for (int e = tid; e < a.n; e += T) sm.c0[e] = -1.4426950408889634f * a.c0[e];
     for (int e = tid; e < QP; e += T) reinterpret_cast<float *>(sm.cn)[e] = a.cn[e];
     State<NST * R> *st = reinterpret_cast<State<NST * R> *>(state) + tid;
+    bool beyond; // (of swaptions)
     for (uint32_t t = tiles.x; t < tiles.y; ++t)
-        block_tile<SCHEME, QP, B, R>(a, sm, st, t, acc, comp, t == tiles.x);
+        block_tile<SCHEME, QP, B, R, CAPLETS>(a, sm, st, t, acc, comp, t == tiles.x, beyond);
 }
 
 template <int SCHEME, int QMAX, int R>
@@ -108,39 +75,7 @@ __global__ void __launch_bounds__(kMaxThreads, blocks_of(FULL, QMAX > 8 ? 24 : 8
     }
 }
 
-typedef void (*KernelFn)(const PathArgs);
-
-// The full scheme on 20 nodes runs as well in two blocks of 128 threads an SM at
-// 192 registers as in four at 128 (a wave of 38,912 paths 3.9 ms, of 77,824 paths
-// 7.4); the two differ by how many paths the last wave is short of, and from here
-// on the larger wave wins throughout: N = 120, 140,000 paths 14.8 against 15.5 ms,
-// 2^20 paths 99.7 against 108.7.  (Below, either may: 116,000 paths 12.9 against
-// 11.6, 55,000 paths 6.0 against 7.7.)
-constexpr uint64_t kManyPaths = 140000;
 typedef void (*BatchFn)(const BatchArgs);
-
-template <int SCHEME, int R>
-KernelFn pick_qp(int QP)
-{
-    switch (QP) {
-    case 4: return block_kernel<SCHEME, 4, R>;
-    case 8: return block_kernel<SCHEME, 8, R>;
-    case 12: return block_kernel<SCHEME, 12, R>;
-    case 16: return block_kernel<SCHEME, 16, R>;
-    case 20: return block_kernel<SCHEME, 20, R>;
-    case 24: return block_kernel<SCHEME, 24, R>;
-    case 32: return block_kernel<SCHEME, 32, R>;
-    default: return nullptr;
-    }
-}
-
-KernelFn pick(int scheme, int QP, int R, uint64_t paths)
-{
-    if (scheme == FULL && QP == 20 && R == 1 && paths >= kManyPaths) return block_kernel<FULL, 20, 1, 2>;
-    if (scheme == FULL) return R == 1 ? pick_qp<FULL, 1>(QP) : R == 2 ? pick_qp<FULL, 2>(QP) : nullptr;
-    if (scheme == PICARD) return R == 1 ? pick_qp<PICARD, 1>(QP) : R == 2 ? pick_qp<PICARD, 2>(QP) : nullptr;
-    return nullptr;
-}
 
 BatchFn pick_batch(int scheme, int QMAX, int R)
 {
@@ -150,6 +85,11 @@ BatchFn pick_batch(int scheme, int QMAX, int R)
     }
     if (scheme == FULL) return R == 1 ? batch_block_kernel<FULL, 32, 1> : batch_block_kernel<FULL, 32, 2>;
     return R == 1 ? batch_block_kernel<PICARD, 32, 1> : batch_block_kernel<PICARD, 32, 2>;
+}
+
+BlockFn pick_kernel(int scheme, int product, int QP, int R, uint64_t paths)
+{
+    return product == 0 ? pick<CAPLETS>(scheme, QP, R, paths) : pick_swaption_kernel(scheme, QP, R, paths);
 }
 
 template <class F>
@@ -176,16 +116,21 @@ size_t block_kernel_smem(int QP, int R, int n, int threads, int chunk_rates)
     return block_smem_bytes(QP, steps_of(QP, R), R, n, threads, chunk_rates);
 }
 
-int block_kernel_prepare(int scheme, int QP, int R, uint64_t paths, size_t smem, int threads, int *blocks_per_sm)
+int block_kernel_prepare(int scheme, int product, int QP, int R, uint64_t paths, size_t smem, int threads,
+                         int *blocks_per_sm)
 {
-    return prepare(pick(scheme, QP, R, paths), smem, kMaxSmem, threads, blocks_per_sm);
+    return prepare(pick_kernel(scheme, product, QP, R, paths), smem, kMaxSmem, threads, blocks_per_sm);
 }
 
 int launch_block_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st, const PathArgs &a)
 {
-    KernelFn f = pick(scheme, QP, R, a.paths);
+    BlockFn f = pick_kernel(scheme, a.product, QP, R, a.paths);
     if (!f) return (int)cudaErrorInvalidValue;
-    f<<<grid, threads, smem, st>>>(a);
+    if (a.product == 0 || !a.wide_strikes) f<<<grid, threads, smem, st>>>(a);
+    if (a.product != 0) {
+        const int e = launch_wide_swaptions(scheme, QP, R, grid, threads, st, a);
+        if (e != 0) return e;
+    }
     return (int)cudaGetLastError();
 }
 

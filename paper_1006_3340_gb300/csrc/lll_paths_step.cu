@@ -204,13 +204,25 @@ __global__ void __launch_bounds__(kSpT) sp_payoff(const PathArgs a, int Pc, uint
     float Lm = 0.0f;
     float4 mv = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (lp < Pc) {
-        if constexpr (SHORT) mv = maturity_values(a, m, z);
+        if constexpr (SHORT) mv = maturity_values(a, a.product, m, z);
         else maturity_products(a, m, z, Pp, Sp, Lm);
     }
+    bool wide = false; // swaptions of the shorter rule beyond the pairs' range: FP64
+    if (SHORT && a.product != 0) wide = __syncthreads_or(a.wide_strikes || (active && beyond_pairs(mv)));
+    double2 xv = make_double2(0.0, 0.0);
+    if (wide && active)
+        xv = swaption_values(a.delta, n, m, [&](int i) { return __ldg(a.L0 + i - 1) * expf(z(i)); });
     for (int q = 0; q < ns; ++q) {
         const float K = a.strikes[(size_t)(m - 1) * ns + q];
         const size_t slot = (size_t)warp * ns + q;
-        if (SHORT || a.product == 0) {
+        if (wide) {
+            const double X = xv.x - (double)K * xv.y, v = X > 0.0 ? payoff_scale(a) * X : 0.0;
+            const double s1 = warp_sum(v), s2 = warp_sum(v * v);
+            if (lane == 0) {
+                red[2 * slot + 0] = s1;
+                red[2 * slot + 1] = s2;
+            }
+        } else if (SHORT || a.product == 0) {
             DFloat v{0.0f, 0.0f};
             if (active) {
                 if constexpr (SHORT) v = payoff_of(a.product, mv, K);
@@ -230,8 +242,8 @@ __global__ void __launch_bounds__(kSpT) sp_payoff(const PathArgs a, int Pc, uint
     __syncthreads();
     if (threadIdx.x < ns) {
         double s1, s2;
-        block_payoff_sums(a.product == 0 || SHORT, red, kSpT / 32, ns, threadIdx.x, s1, s2);
-        if (SHORT) {
+        block_payoff_sums(a.product == 0 || (SHORT && !wide), red, kSpT / 32, ns, threadIdx.x, s1, s2);
+        if (SHORT && !wide) {
             s1 *= payoff_scale(a);
             s2 *= payoff_scale(a) * payoff_scale(a);
         }

@@ -1,0 +1,75 @@
+// lll_paths_swaption.cu -- the time-blocked path kernels (lll_paths_block.cuh) of
+// co-terminal swaptions.
+//
+// Payoffs are formed in pairs of FP32 numbers (maturity_values): in FP64, of which
+// GB300 has a 64th of the FP32 rate, the N = 40 workload takes a fifth longer.  The
+// pairs have FP32's exponents, so a block that meets a value beyond their range
+// (beyond_pairs) marks its sums, and wide_kernel, launched behind, runs that block's
+// tiles again with FP64 payoffs.  It ends at once where there is no mark.  (Formed in
+// FP64 within the first kernel instead, the code for it alone cost 2.5 % there:
+// 300,007 paths 3.97 against 3.87 ms.)
+#include "lll_paths_block.cuh"
+
+namespace lll {
+namespace {
+
+// The marked blocks' tiles of a launch with R paths a thread, as R tiles each of one
+// path a thread.  Strikes beyond the range are known on the host: then every block.
+template <int SCHEME, int QP>
+__global__ void __launch_bounds__(kMaxThreads, 1) wide_kernel(const PathArgs a, int R)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int B = steps_of(QP, 1), NST = (SCHEME == PICARD) ? 2 : 1;
+    const int T = blockDim.x, tid = threadIdx.x;
+    const size_t nout = (size_t)a.n * a.ns * 2;
+    double *acc = a.partials + blockIdx.x * nout, *comp = a.partials + (gridDim.x + blockIdx.x) * nout;
+    if (!a.wide_strikes && !isnan(comp[0])) return; // the same for the whole block
+    __syncthreads();                                // before the mark is written over
+    const BlockSmem sm = block_carve(smem_raw, QP, B, 1, a.n, T, a.chunk_rows);
+    for (int e = tid; e < a.n; e += T) sm.c0[e] = -1.4426950408889634f * a.c0[e];
+    for (int e = tid; e < QP; e += T) reinterpret_cast<float *>(sm.cn)[e] = a.cn[e];
+    State<NST> *st = reinterpret_cast<State<NST> *>(a.state) + (size_t)blockIdx.x * a.n * T + tid;
+    const uint64_t TP = (uint64_t)T * R, ntiles = (a.paths + TP - 1) / TP;
+    bool beyond, first = true;
+    for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+        for (int q = 0; q < R; ++q) {
+            block_tile<SCHEME, QP, B, 1, WIDE_SWAPTIONS>(a, sm, st, tile * R + q, acc, comp, first, beyond);
+            first = false;
+        }
+}
+
+typedef void (*WideFn)(const PathArgs, int);
+
+template <int SCHEME>
+WideFn pick_wide(int QP)
+{
+    switch (QP) {
+    case 4: return wide_kernel<SCHEME, 4>;
+    case 8: return wide_kernel<SCHEME, 8>;
+    case 12: return wide_kernel<SCHEME, 12>;
+    case 16: return wide_kernel<SCHEME, 16>;
+    case 20: return wide_kernel<SCHEME, 20>;
+    case 24: return wide_kernel<SCHEME, 24>;
+    case 32: return wide_kernel<SCHEME, 32>;
+    default: return nullptr;
+    }
+}
+
+}  // namespace
+
+BlockFn pick_swaption_kernel(int scheme, int QP, int R, uint64_t paths) { return pick<SWAPTIONS>(scheme, QP, R, paths); }
+
+int launch_wide_swaptions(int scheme, int QP, int R, int grid, int threads, cudaStream_t st, const PathArgs &a)
+{
+    WideFn f = scheme == FULL ? pick_wide<FULL>(QP) : scheme == PICARD ? pick_wide<PICARD>(QP) : nullptr;
+    if (!f) return (int)cudaErrorInvalidValue;
+    PathArgs w = a;
+    w.chunk_rows = block_chunk_rates(QP, 1, a.n, 0);
+    const size_t smem = block_kernel_smem(QP, 1, a.n, threads, w.chunk_rows);
+    const cudaError_t e = allow_smem(f, smem);
+    if (e != cudaSuccess) return (int)e;
+    f<<<grid, threads, smem, st>>>(w, R);
+    return (int)cudaGetLastError();
+}
+
+}  // namespace lll

@@ -175,17 +175,28 @@ struct alignas(4 * N) State {
     float v[N];
 };
 
+// What a kernel prices: caplets; swaptions in pairs of FP32 numbers; swaptions in
+// FP64 (values beyond the pairs' range, see beyond_pairs).
+enum { CAPLETS = 0, SWAPTIONS = 1, WIDE_SWAPTIONS = 2 };
+
 // Payoffs of the block's paths at T_m into the block's FP64 Kahan sums
 // acc[(m-1) ns + q][2] with compensations comp[..][2].  Every thread leaves its
 // paths' values in shared memory; then thread (strike q, slice g) adds up the
-// payoffs of every G-th path in double-float pairs, and thread q the G slices.
-// (Reducing each strike over the warp's lanes instead, by shuffles, took 0.25
-// of 2.08 ms on the N = 40 workload and three times the latency.)
-template <int NST, int R>
+// payoffs of every G-th path in double-float pairs (FP64: WIDE_SWAPTIONS), and
+// thread q the G slices.  (Reducing each strike over the warp's lanes instead, by
+// shuffles, took 0.25 of 2.08 ms on the N = 40 workload and three times the
+// latency.)  beyond: set where a swaption of this thread's paths is beyond the pairs.
+template <int NST, int R, int PRICES>
 __device__ __forceinline__ void block_maturity(const PathArgs &a, const BlockSmem &sm, const State<NST * R> *st, int T,
-                                               int m, const uint64_t (&lp)[R], double *acc, double *comp, bool first)
+                                               int m, const uint64_t (&lp)[R], double *acc, double *comp, bool first,
+                                               bool &beyond)
 {
+    constexpr bool WIDE = PRICES == WIDE_SWAPTIONS;
     const int n = a.n, ns = a.ns, tid = threadIdx.x;
+    // (the caplets' kernels keep the run-time product: with a constant in its place the
+    // N = 40 Picard kernel took 12.88 ms for 2^20 paths, not 12.74)
+    const int product = PRICES == CAPLETS ? a.product : 1;
+    double2 *const values = reinterpret_cast<double2 *>(sm.pay), *const sums = reinterpret_cast<double2 *>(sm.part);
 #pragma unroll
     for (int u = 0; u < R; ++u) {
         auto z = [&](int i) {
@@ -194,9 +205,15 @@ __device__ __forceinline__ void block_maturity(const PathArgs &a, const BlockSme
             if constexpr (NST == 2) x += v.v[2 * u + 1];
             return x;
         };
-        float4 v = maturity_values(a, m, z);
-        if (lp[u] >= a.paths) v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        sm.pay[u * T + tid] = v;
+        if constexpr (WIDE) {
+            auto rate = [&](int i) { return __ldg(a.L0 + i - 1) * expf(z(i)); };
+            values[u * T + tid] = lp[u] < a.paths ? swaption_values(a.delta, n, m, rate) : make_double2(0.0, 0.0);
+        } else {
+            float4 v = maturity_values(a, product, m, z);
+            if (lp[u] >= a.paths) v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if constexpr (PRICES == SWAPTIONS) beyond = beyond || beyond_pairs(v);
+            sm.pay[u * T + tid] = v;
+        }
         if (a.snap != nullptr && lp[u] < a.paths && lp[u] % a.snap_stride == 0 && lp[u] / a.snap_stride < a.n_snap)
             for (int i = n; i >= m; --i)
                 a.snap[((size_t)(m - 1) * n + (i - 1)) * a.snap_pitch + lp[u] / a.snap_stride] = z(i) + a.Z0[i - 1];
@@ -209,25 +226,47 @@ __device__ __forceinline__ void block_maturity(const PathArgs &a, const BlockSme
         const int q = tid % nq, g = tid / nq;
         if (g < G) {
             const float K = a.strikes[(size_t)(m - 1) * ns + q0 + q];
-            DFloat s1{0.0f, 0.0f}, s2{0.0f, 0.0f};
-            for (int p = g; p < R * T; p += G) {
-                const DFloat v = payoff_of(a.product, sm.pay[p], K);
-                s1 = df_add(s1, v);
-                s2 = df_add(s2, df_square_pair(v));
+            if constexpr (WIDE) {
+                const double scale = payoff_scale(a);
+                double s1 = 0.0, s2 = 0.0;
+                for (int p = g; p < R * T; p += G) {
+                    const double X = values[p].x - (double)K * values[p].y, v = X > 0.0 ? scale * X : 0.0;
+                    s1 += v;
+                    s2 += v * v;
+                }
+                sums[g * nq + q] = make_double2(s1, s2);
+            } else {
+                DFloat s1{0.0f, 0.0f}, s2{0.0f, 0.0f};
+                for (int p = g; p < R * T; p += G) {
+                    const DFloat v = payoff_of(product, sm.pay[p], K);
+                    s1 = df_add(s1, v);
+                    s2 = df_add(s2, df_square_pair(v));
+                }
+                sm.part[g * nq + q] = make_float4(s1.hi, s1.lo, s2.hi, s2.lo);
             }
-            sm.part[g * nq + q] = make_float4(s1.hi, s1.lo, s2.hi, s2.lo);
         }
         __syncthreads();
         if (tid < nq) {
-            float4 r = sm.part[tid];
-            DFloat x{r.x, r.y}, y{r.z, r.w};
-            for (int k = 1; k < G; ++k) {
-                r = sm.part[k * nq + tid];
-                x = df_add(x, DFloat{r.x, r.y});
-                y = df_add(y, DFloat{r.z, r.w});
+            double v1, v2;
+            if constexpr (WIDE) {
+                v1 = sums[tid].x;
+                v2 = sums[tid].y;
+                for (int k = 1; k < G; ++k) {
+                    v1 += sums[k * nq + tid].x;
+                    v2 += sums[k * nq + tid].y;
+                }
+            } else {
+                float4 r = sm.part[tid];
+                DFloat x{r.x, r.y}, y{r.z, r.w};
+                for (int k = 1; k < G; ++k) {
+                    r = sm.part[k * nq + tid];
+                    x = df_add(x, DFloat{r.x, r.y});
+                    y = df_add(y, DFloat{r.z, r.w});
+                }
+                const double c = payoff_scale(a);
+                v1 = c * ((double)x.hi + (double)x.lo);
+                v2 = c * c * ((double)y.hi + (double)y.lo);
             }
-            const double c = payoff_scale(a);
-            const double v1 = c * ((double)x.hi + (double)x.lo), v2 = c * c * ((double)y.hi + (double)y.lo);
             const size_t e = 2 * ((size_t)(m - 1) * ns + q0 + tid);
             if (first) {
                 acc[e] = v1;
@@ -284,10 +323,10 @@ __device__ __forceinline__ void sweep_chunk(const PathArgs &a, const BlockSmem &
 
 // One tile: all Euler steps and payoffs.  st: this thread's column of the
 // block's state slot [n][T]; acc, comp: the block's payoff sums; first: they
-// hold nothing yet.
-template <int SCHEME, int QP, int B, int R>
+// hold nothing yet; beyond: see block_maturity.
+template <int SCHEME, int QP, int B, int R, int PRICES>
 __device__ __forceinline__ void block_tile(const PathArgs &a, const BlockSmem &sm, State<(SCHEME == PICARD ? 2 : 1) * R> *st,
-                                           uint64_t tile, double *acc, double *comp, bool first)
+                                           uint64_t tile, double *acc, double *comp, bool first, bool &beyond)
 {
     constexpr int NST = (SCHEME == PICARD) ? 2 : 1;
     const int T = blockDim.x, tid = threadIdx.x;
@@ -347,7 +386,7 @@ __device__ __forceinline__ void block_tile(const PathArgs &a, const BlockSmem &s
                 buf ^= 1;
             }
         }
-        block_maturity<NST, R>(a, sm, st, T, m, lp, acc, comp, first);
+        block_maturity<NST, R, PRICES>(a, sm, st, T, m, lp, acc, comp, first, beyond);
     }
     cp_wait_0();
 }
