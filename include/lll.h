@@ -214,13 +214,16 @@ int lll_kernel_ms(lll_ctx *ctx, float *path_kernel_ms, float *simulate_ms);
  *   d_sums     : caller-owned device buffer of n * n_strikes * 2 doubles,
  *                d_sums[2*(m*n_strikes + q)] = sum of payoffs and [... + 1] =
  *                sum of squared payoffs of maturity m+1, strike q.
- * Makes the same launch as lll_simulate (with fewer blocks where the scratch
- * would not hold the state of all), so the sums equal lll_get_sums'.
- * Scratch (per-block path state and payoff partials) comes from one static
- * 32 MiB device array that every GPU loading the library holds until exit;
- * a launch of the rule as given that needs more returns LLL_EUNSUPPORTED with
- * the byte counts in
- * lll_last_error.  Each call made outside a stream capture looks the array's
+ * Makes the same launch as lll_simulate, so the sums equal lll_get_sums',
+ * where that launch's scratch fits.  Scratch (per-block path state and payoff
+ * partials) comes from one static 32 MiB device array that every GPU loading
+ * the library holds until exit.  The bound is held against the launch of the
+ * rule as given: one needing more returns LLL_EUNSUPPORTED with the byte counts
+ * in lll_last_error.  Where that one fits and the launch of its shorter
+ * equivalent (lll_sweep_rule) does not, as for 2^18 paths of 39 rates under
+ * LLL_PICARD, fewer blocks run, or the kernel for many paths in place of that
+ * for few; the sums then agree to the grouping of their FP64 partials (1e-12).
+ * Each call made outside a stream capture looks the array's
  * address up (cudaGetSymbolAddress), so a module reloaded after
  * cudaDeviceReset is found at its new address; a call made while the
  * context's stream is captured uses the address the last uncaptured call
