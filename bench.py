@@ -749,6 +749,14 @@ def run_single(args, wl, schemes, steps, warmup, dev, rank, world, local, with_c
     return line
 
 
+# name, candidate of autotune.apply.  The step mapping with a shape of its own: with the
+# default one it may run the path mapping's kernels.
+MAPPING_SHAPES = [("default", (0, 0, 0, 0, 0)), ("path, 128 threads", (128, 0, 0, 1, 1)), ("path, 256 threads", (256, 0, 0, 1, 1)),
+                  ("path, 2 paths/thread", (128, 0, 0, 2, 1))] + \
+                 [(f"tenor, {g} lanes/path", (0, 0, 0, 0, 0, g)) for g in (4, 8, 16, 32)] + \
+                 [("step-parallel (Picard)", (128, 0, 0, 1, 1, -1))]
+
+
 def run_mappings(args, rates=None):
     """Path mapping against the tenor-parallel mapping: device time of one
     simulation of the N=40 term structure (full and Picard) at 2^20 paths and
@@ -763,10 +771,6 @@ def run_mappings(args, rates=None):
 
     dev = torch.device("cuda", 0)
     pk = _alu_peaks(lll, torch, dev, rates)
-    shapes = [("default", (0, 0, 0, 0, 0)), ("path, 128 threads", (128, 0, 0, 1, 1)), ("path, 256 threads", (256, 0, 0, 1, 1)),
-              ("path, 2 paths/thread", (128, 0, 0, 2, 1))] + \
-             [(f"tenor, {g} lanes/path", (0, 0, 0, 0, 0, g)) for g in (4, 8, 16, 32)] + \
-             [("step-parallel (Picard)", (0, 0, 0, 0, 0, -1))]
     rows = []
     sizes = (args.paths,) if args.paths else (1 << 20, 1 << 12)
     schemes = [s for s in args.schemes.split(",") if s in ("picard", "full")] or ["picard", "full"]
@@ -776,7 +780,7 @@ def run_mappings(args, rates=None):
         sim = lll.LevyLibor(wl, x, W)
         try:
             for scheme in schemes:
-                for name, cand in shapes:
+                for name, cand in MAPPING_SHAPES:
                     if scheme == "full" and len(cand) > 5 and cand[5] < 0:
                         continue  # the full scheme's steps are sequential
                     autotune.apply(sim, cand)

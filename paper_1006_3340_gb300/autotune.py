@@ -28,7 +28,8 @@ DEFAULT_CANDIDATES = [
 ] + [
     (t, 0, c, 1, l) for t, c, l in itertools.product((64, 128, 256), (0, 16), (1, 2, 4))
 ] + [(t, 0, c, 2, 1) for t, c in itertools.product((64, 128), (0, 16))] \
-  + [(0, 0, 0, 0, 0, g) for g in (4, 8, 16, 32, -1)]
+  + [(0, 0, 0, 0, 0, g) for g in (4, 8, 16, 32)] \
+  + [(128, 0, 0, 1, 1, -1)]  # a shape of its own: with the default one the step mapping may run the path kernels
 
 
 def apply(sim: "lll.LevyLibor", cand) -> None:
