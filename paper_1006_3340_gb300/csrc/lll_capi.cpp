@@ -151,6 +151,34 @@ static void block_shape(const lll_ctx *ctx, uint64_t paths, int *R, int *T)
     if (ctx->threads == 0) *T = 128;
 }
 
+// Whether a default launch of caplets may take the pipeline (pipe_shape).
+static bool pipe_allowed(const lll_ctx *ctx)
+{
+    return ctx->threads == 0 && ctx->blocks_per_sm == 0 && ctx->ppt == 0 && ctx->chunk_rows == 0 &&
+           ctx->product == LLL_PRODUCT_CAPLET;
+}
+
+// Scratch that smaller calls of this context, on other kernels than this plan's, may
+// need more of: a call with fewer paths than an earlier one then never changes the
+// buffers.  The pipeline's many small blocks have more payoff sums than the block
+// kernel's on more paths; and where the pipeline's shape for one block an SM does not
+// fit shared memory, the block kernel serves fewer paths than the pipeline.
+static void smaller_calls(const lll_ctx *ctx, const LaunchPlan &plan, size_t *state_floats, size_t *partial_doubles)
+{
+    if (!plan.block || !pipe_allowed(ctx)) return;
+    const uint64_t now_per_sm = ((plan.args.paths + 31) / 32 + ctx->sm_count - 1) / ctx->sm_count;
+    const int now = (int)std::min<uint64_t>(now_per_sm, kMaxPipePerSm);
+    for (int scheme : {LLL_FULL, LLL_PICARD})
+        for (int per_sm = 1; per_sm <= now; ++per_sm) {
+            size_t smem;
+            const uint64_t tiles = (uint64_t)per_sm * ctx->sm_count; // of 32 paths
+            const bool pipe = pipe_shape(scheme, ctx->QR, ctx->n, ctx->s, ctx->S, tiles, ctx->sm_count, &smem) != 0;
+            if (pipe && !plan.pipe) *partial_doubles = std::max(*partial_doubles, tiles * plan.n_out);
+            if (!pipe && plan.pipe && per_sm < now)
+                *state_floats = std::max(*state_floats, (tiles + 3) / 4 * ctx->n * 128 * (scheme == LLL_PICARD ? 2 : 1));
+        }
+}
+
 // Same launch shape and arguments as lll_simulate, with no allocation: the
 // per-block scratch sizes are returned for the caller to place.
 int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, uint64_t seed,
@@ -199,8 +227,7 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     }
     // The pipeline serves a default launch of caplets on few paths.
     size_t pipe_smem = 0;
-    const int pipe = allow_pipe && block && ctx->threads == 0 && ctx->blocks_per_sm == 0 && ctx->ppt == 0 &&
-                             ctx->chunk_rows == 0 && ctx->product == LLL_PRODUCT_CAPLET
+    const int pipe = allow_pipe && block && pipe_allowed(ctx)
                          ? pipe_shape(scheme, ctx->QR, ctx->n, ctx->s, ctx->S, (paths + 31) / 32, ctx->sm_count, &pipe_smem)
                          : 0;
     int occ = 0;
@@ -664,7 +691,8 @@ int lll_simulate(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, 
     int rc = plan_launch(ctx, scheme, first_path, paths, seed, &plan);
     if (rc != LLL_OK) return rc;
     const int grid = plan.grid;
-    const size_t state_need = plan.state_floats_per_block * grid;
+    size_t state_need = plan.state_floats_per_block * grid, part_need = plan.partial_doubles_per_block * grid;
+    smaller_calls(ctx, plan, &state_need, &part_need);
     if (state_need > ctx->state_cap) {
         dev_free(ctx, ctx->d_state);
         ctx->d_state = nullptr;
@@ -672,7 +700,7 @@ int lll_simulate(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, 
         if (dalloc(&ctx->d_state, state_need) != cudaSuccess) return fail(ctx, LLL_ENOMEM, "state scratch");
         ctx->state_cap = state_need;
     }
-    const size_t nout = (size_t)plan.n_out, part_need = plan.partial_doubles_per_block * grid;
+    const size_t nout = (size_t)plan.n_out;
     if (part_need > ctx->partials_cap) {
         dev_free(ctx, ctx->d_partials);
         ctx->d_partials = nullptr;

@@ -109,6 +109,7 @@ int launch_batch_block_kernel(int scheme, int QMAX, int R, int grid, int threads
 
 // Launchers implemented in lll_paths_pipe.cu (few paths: 32 paths a block, a
 // pipeline of warps over the rates).
+constexpr int kMaxPipePerSm = 8; // blocks an SM of its largest launch
 int pipe_shape(int scheme, int QP, int n, int s, int S, uint64_t tiles, int sms, size_t *smem);
 int launch_pipe_kernel(int scheme, int QP, int shape, size_t smem, uint64_t paths, cudaStream_t st, const PathArgs &a);
 

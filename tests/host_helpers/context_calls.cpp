@@ -16,6 +16,7 @@ std::vector<Tables> g_tables;              // launches of the table kernel
 const void *g_path_tab = nullptr;          // table of the last path kernel
 long g_mallocs = 0, g_frees = 0, g_launches = 0, g_copies = 0;
 bool g_capturing = false;
+uint64_t g_pipe_tiles = 0, g_pipe_hole = 0; // blocks an SM up to which the pipeline is chosen, and but one
 
 int check(bool ok, const char *what)
 {
@@ -71,7 +72,12 @@ int block_chunk_rates(int, int, int n, int) { return n; }
 size_t block_kernel_smem(int, int, int, int, int) { return 1024; }
 int block_kernel_prepare(int, int, int, int, uint64_t, size_t, int, int *b) { return *b = 4, 0; }
 int launch_block_kernel(int, int, int, int, int, size_t, cudaStream_t, const PathArgs &a) { return ++g_launches, g_path_tab = a.tab, 0; }
-int pipe_shape(int, int, int, int, int, uint64_t, int, size_t *) { return 0; }
+int pipe_shape(int, int, int, int, int, uint64_t tiles, int sms, size_t *) 
+{
+    const uint64_t per_sm = (tiles + sms - 1) / sms;
+    return per_sm <= g_pipe_tiles && per_sm != g_pipe_hole;
+}
+int launch_pipe_kernel(int, int, int, size_t, uint64_t, cudaStream_t, const PathArgs &) { return ++g_launches, 0; }
 bool group_kernel_supported(int, int, int) { return true; }
 size_t group_kernel_smem(int, int, int, int, int) { return 1024; }
 int group_kernel_prepare(int, int, int, size_t, int, int *b) { return *b = 4, 0; }
@@ -155,6 +161,27 @@ int selections()
         }
     return bad;
 }
+// A call with fewer paths than an earlier one allocates and frees nothing,
+// whichever kernel it takes (its launches may be captured, and an earlier capture
+// may hold the buffers).
+int fewer_paths()
+{
+    int bad = 0;
+    for (g_pipe_tiles = 1; g_pipe_tiles <= 8; ++g_pipe_tiles)
+        for (g_pipe_hole = 0; g_pipe_hole < 3; ++g_pipe_hole)
+        for (uint64_t most : {300000ull, 30000ull, 5000ull}) {
+            lll_ctx *c = model();
+            bad += check(lll_simulate(c, LLL_PICARD, 0, most, 1) == LLL_OK, "simulate");
+            const long mallocs = g_mallocs, frees = g_frees;
+            for (uint64_t paths = most; paths > 0; paths = paths * 9 / 10)
+                for (int scheme : {LLL_PICARD, LLL_FULL}) bad += check(lll_simulate(c, scheme, 0, paths, 1) == LLL_OK, "simulate");
+            if (g_mallocs != mallocs || g_frees != frees) std::fprintf(stderr, "pipeline to %d, but %d, from %llu paths: ", (int)g_pipe_tiles, (int)g_pipe_hole, (unsigned long long)most);
+            bad += check(g_mallocs == mallocs && g_frees == frees, "a call with fewer paths changed its buffers");
+            lll_destroy(c);
+        }
+    g_pipe_tiles = 0;
+    return bad;
+}
 }  // namespace
 
 int main(int argc, char **argv)
@@ -162,5 +189,6 @@ int main(int argc, char **argv)
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "compensators") return compensators();
     if (what == "selections") return selections();
+    if (what == "fewer_paths") return fewer_paths();
     return 2;
 }
