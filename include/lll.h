@@ -108,7 +108,8 @@ int lll_init(lll_ctx **out, int N, double tenor_delta, const double *L0, int ste
  *     is (1 - B(T_m,T_N) - K delta sum_{j>m} B(T_m,T_j))^+, priced under the
  *     terminal measure as B(0,T_N) E[((1 + delta L_m) P - 1 - K delta S)^+]
  *     with P = prod_{l>m} (1 + delta L_l(T_m)) and S = sum_{j=m+1}^{N}
- *     prod_{l>=j} (1 + delta L_l(T_m)) (48 bits or more on the GPU).  lll_price_caplets
+ *     prod_{l>=j} (1 + delta L_l(T_m)) (48 bits on the GPU, FP64 where a
+ *     value leaves their range or the rule is swept as given).  lll_price_caplets
  *     then returns swaption prices.  The batched launch prices caplets only. */
 #define LLL_PRODUCT_CAPLET 0
 #define LLL_PRODUCT_SWAPTION 1
@@ -243,10 +244,12 @@ int lll_simulate_noalloc(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t
 int lll_build_nig_quadrature(lll_nig nig, double xmax, int Q, double *nodes, double *weights);
 
 /* lll_sweep_rule -- the rule that the full and Picard sweeps use in place of
- * (nodes, weights), the arguments of lll_init: the shortest Gauss rule of the
- * discrete measure sum_j weights[j] delta_nodes[j] (at most 32 nodes) whose
- * moment generating function agrees with the given rule's to 2^-28 relative
- * on [lo, hi].  With lo (hi) the most negative (positive) sum of the live
+ * (nodes, weights), the arguments of lll_init: a Gauss rule of the discrete
+ * measure sum_j weights[j] delta_nodes[j] whose moment generating function
+ * agrees with the given rule's to 2^-28 relative on [lo, hi] and whose sum of
+ * weights[j] / |nodes[j]| is no larger.  Of the node counts that the kernels
+ * process (4, 8, 12, 16, 20, 24, 32) the first that holds such a rule is taken,
+ * and in it the longest rule.  With lo (hi) the most negative (positive) sum of the live
  * volatilities over the steps, every compensator of Eq. (LIBOR-drift-PT) then
  * agrees to 2^-28 of its terms, whatever the rates.  lo <= 0 <= hi.
  *   count : nodes of the shorter rule; 0 where the given rule is swept (a
@@ -254,6 +257,7 @@ int lll_build_nig_quadrature(lll_nig nig, double xmax, int Q, double *nodes, dou
  *           or no shorter rule agrees);
  *   padded: nodes the kernels process (the given rule padded where count = 0);
  *   x, w  : [32] outputs, the first `count` used.
+ * C_l, the frozen drift and D0 are formed with the shorter rule too, in FP64.
  * Host computation. */
 int lll_sweep_rule(int Q, const double *nodes, const double *weights, double lo, double hi, int *count,
                    int *padded, double *x, double *w);
@@ -267,7 +271,9 @@ int lll_sweep_rule(int Q, const double *nodes, const double *weights, double lo,
  * whatever block ran which item.  Instance q draws its increments
  * from Philox counter (k, q, p_lo, p_hi): independent streams per instance.
  * All instances must use the NIG driver and the same padded Q (16, 32, 64, 96
- * or 128). */
+ * or 128).  Instances sweep their shorter rules (lll_sweep_rule) where every one
+ * has one; a single instance without takes all to the rules as given, at about
+ * five times the time: better priced in a batch of its own. */
 typedef struct {
     int N;                 /* accrual dates (as lll_init) */
     double tenor_delta;

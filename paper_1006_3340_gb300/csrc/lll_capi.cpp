@@ -80,7 +80,10 @@ void free_all(lll_ctx *c)
         if (e) cudaEventDestroy(e);
 }
 
-constexpr size_t kArenaPartials = size_t(1) << 15; // doubles: 608 blocks of 9 rates and 3 strikes
+// Payoff scratch in the arena (doubles, 256 KB): short curves on a few thousand paths
+// need no more (a pipeline of 4,864 paths, 9 rates, 11 strikes), and their fresh
+// contexts, priced once, then allocate nothing else; a larger call allocates its own.
+constexpr size_t kArenaPartials = size_t(1) << 15;
 
 int default_chunk_rows(int n, int QP)
 {
@@ -590,7 +593,8 @@ namespace {
 // kernels, whose threads do not carry products across steps, while their
 // intermediate arrays are small: N = 120 (20 nodes), 2000 paths 0.53 against 0.75
 // ms, 4096 paths (1.2e8 units) 0.89 against 0.75; the 9-rate heavy-tailed example
-// (32 nodes), 8192 paths (1.8e6 units) 0.058 against 0.090.
+// (32 nodes), 8192 paths (1.8e6 units) 0.058 against 0.090.  The two unit counts lie
+// between such pairs of points, one curve each.
 bool step_as_path(const lll_ctx *ctx, uint64_t paths)
 {
     if (ctx->QR >= ctx->QP || ctx->lpp > 1 || ctx->ppt > 0 || ctx->threads > 0 || ctx->blocks_per_sm > 0 ||

@@ -9,9 +9,8 @@
 //
 // Measured on a GB300 (whole call, prices read) against the step-by-step sweep
 // of the rule as given (lll_paths.cu): Picard, N = 40, 64 -> 8 nodes, 2^20
-// paths 59.8 -> 15.0 ms, of which the shorter rule alone in that sweep gave
-// 29.7; full, N = 120, 96 -> 24 nodes, 2^17 paths 63.1 -> 18.3 ms (27.1); full,
-// N = 40, 4096 paths 2.11 -> 0.66 ms (1.02).
+// paths 59.8 -> 12.7 ms; full, N = 120, 96 -> 20 nodes, 2^17 paths 63.1 -> 13.6
+// ms; full, N = 40, 4096 paths 2.11 -> 0.60 ms (the pipeline: 0.15).
 #include <cuda_runtime.h>
 
 #include "lll_paths_block.cuh"

@@ -56,9 +56,10 @@ __global__ void __launch_bounds__(kMaxThreads, BL) block_kernel(const PathArgs a
 // The full scheme on 20 nodes runs as well in two blocks of 128 threads an SM at
 // 192 registers as in four at 128 (a wave of 38,912 paths 3.9 ms, of 77,824 paths
 // 7.4); the two differ by how many paths the last wave is short of, and from here
-// on the larger wave wins throughout: N = 120, 140,000 paths 14.8 against 15.5 ms,
-// 2^20 paths 99.7 against 108.7.  (Below, either may: 116,000 paths 12.9 against
-// 11.6, 55,000 paths 6.0 against 7.7.)
+// on the larger wave wins throughout: N = 120, 140,000 paths 14.8 ms at 128
+// registers, 15.5 at 192, 2^20 paths 99.7 and 108.7.  Below, 192 registers are
+// taken, which is not always the better: 116,000 paths 11.6 ms (12.9 at 128), but
+// 55,000 paths 7.7 (6.0).  Other node counts were not measured for it.
 constexpr uint64_t kManyPaths = 140000;
 
 template <int PRICES, int SCHEME, int R>

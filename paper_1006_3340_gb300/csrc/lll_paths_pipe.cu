@@ -298,7 +298,7 @@ PipeFn pick_pipe(int QP, int B)
 //    0.66; N = 120 (one block an SM), 4096 paths 0.74 against 2.74, 9000 paths
 //    1.45, 16,000 paths 2.88 against 2.74.
 //  * Fewer rates: fewer warps a block, and more blocks an SM, in one wave.  N = 10
-//    (4 nodes), 10,000 paths: 0.083 with eight warps, 0.053 with four, against
+//    (8 nodes), 10,000 paths: 0.083 with eight warps, 0.053 with four, against
 //    0.098; 20,000 paths 0.073 with two against 0.103; 30,000 paths 0.090 against
 //    0.107; 40,000 paths 0.128 against 0.120.  The heavy-tailed example (32
 //    nodes): 5000 paths 0.081, 0.045 with four, against 0.086; 10,000 paths 0.054
