@@ -217,7 +217,7 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
     if (G == 0 && lpp == 1 && !path_kernel_supported(scheme, QPk, R))
         return fail(ctx, LLL_EUNSUPPORTED, "no kernel for this Q and paths per thread");
     int T = G > 0 ? tenor_kernel_threads() : ctx->threads > 0 ? ctx->threads : 128;
-    int CH = ctx->chunk_rows > 0 ? ctx->chunk_rows : default_chunk_rows(ctx->n, QPk);
+    int CH = ctx->chunk_rows > 0 ? ctx->chunk_rows : default_chunk_rows(ctx->n, ctx->QP);
     size_t smem = G > 0 ? tenor_kernel_smem(QPk, ctx->n, ctx->ns, G)
                 : lpp > 1 ? group_kernel_smem(QPk, ctx->n, ctx->ns, T, CH)
                           : path_kernel_smem(QPk, ctx->n, ctx->ns, T, CH);

@@ -3,6 +3,7 @@
 // CPU.  Built and run by tests/test_context_calls.py only; the first argument
 // names the check.  Exit code 0: as expected; otherwise a message on stderr.
 #include "../../paper_1006_3340_gb300/csrc/lll_capi.cpp"
+#include "../../paper_1006_3340_gb300/csrc/lll_batch.cpp"
 #include "../../paper_1006_3340_gb300/csrc/lll_quadrature.cpp"
 
 #include <cstdlib>
@@ -13,6 +14,10 @@ struct Tables {
     int QP;
 };
 std::vector<Tables> g_tables;              // launches of the table kernel
+struct Need {
+    int QP, n, ns, threads, rows;
+};
+std::vector<Need> g_need;                  // shared memory that was asked for
 const void *g_path_tab = nullptr;          // table of the last path kernel
 long g_mallocs = 0, g_frees = 0, g_launches = 0, g_copies = 0;
 bool g_capturing = false;
@@ -52,6 +57,10 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s)
     *s = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
     return cudaSuccess;
 }
+cudaError_t cudaMallocHost(void **p, size_t bytes) { return *p = std::calloc(bytes, 1), cudaSuccess; }
+cudaError_t cudaFreeHost(void *p) { return std::free(p), cudaSuccess; }
+cudaError_t cudaMemsetAsync(void *p, int v, size_t bytes, cudaStream_t) { return std::memset(p, v, bytes), cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
@@ -64,7 +73,11 @@ const char *cudaGetErrorString(cudaError_t) { return "fake"; }
 namespace lll {
 void mlp_free(MlpState *) {}
 bool path_kernel_supported(int, int, int) { return true; }
-size_t path_kernel_smem(int, int, int, int, int) { return 1024; }
+size_t path_kernel_smem(int QP, int n, int ns, int threads, int rows)
+{
+    g_need.push_back({QP, n, ns, threads, rows});
+    return 1024;
+}
 int path_kernel_prepare(int, int, int, int, size_t) { return 0; }
 int path_kernel_occupancy(int, int, int, int, size_t, int *b) { return *b = 4, 0; }
 int launch_path_kernel(int, int, int, int, int, size_t, cudaStream_t, const PathArgs &a) { return ++g_launches, g_path_tab = a.tab, 0; }
@@ -95,6 +108,11 @@ int launch_tables(const double *, const double *, const double *, int, int, int,
     return 0;
 }
 int launch_prefix(const double *, int, int, double, const double *, double, float4 *, float4 *, cudaStream_t) { return ++g_launches, 0; }
+int batch_block_prepare(int, int, int, size_t, int, int *b) { return *b = 4, 0; }
+int batch_kernel_prepare(int, int, int, size_t, int, int *b) { return *b = 4, 0; }
+int launch_batch_block_kernel(int, int, int, int, int, size_t, cudaStream_t, const BatchArgs &) { return ++g_launches, 0; }
+int launch_batch_kernel(int, int, int, int, int, size_t, cudaStream_t, const BatchArgs &) { return ++g_launches, 0; }
+int batch_finalize(const double *, const size_t *, const int *, const int *, const size_t *, int, const int *, double *, cudaStream_t) { return ++g_launches, 0; }
 int launch_finalize(const double *, int, int, double *, cudaStream_t) { return ++g_launches, 0; }
 }  // namespace lll
 
@@ -182,6 +200,36 @@ int fewer_paths()
     g_pipe_tiles = 0;
     return bad;
 }
+// The shared memory by which a call is refused is that of the rule as given and of
+// 128 threads where none are set: 24 KB of staged rows of that rule, and as many rows
+// under the frozen drift.
+int limits()
+{
+    int bad = 0;
+    lll_ctx *c = model();
+    const int rows = 24 * 1024 / (2 * (32 / 4) * 16); // of 32 nodes
+    for (int scheme : {LLL_FULL, LLL_PICARD, LLL_FROZEN}) {
+        g_need.clear();
+        bad += check(lll_simulate(c, scheme, 0, 5000, 1) == LLL_OK, "simulate");
+        for (const Need &q : g_need) bad += check(q.threads == 128 && q.rows == std::min(rows, 9), "context");
+    }
+    lll_destroy(c);
+    for (int N : {60, 400}) { // more rates than rows
+        const int n = N - 1, Q = 128;
+        std::vector<double> L0(N, 0.03), lam((size_t)n * n, 0.001), x(Q), W(Q), K(n, 0.03);
+        const lll_nig nig{12.0, -3.0, 0.8, NAN};
+        lll_build_nig_quadrature(nig, 1.5, Q, x.data(), W.data());
+        bad += check(lll_init(&c, N, 0.25, L0.data(), 1, lam.data(), LLL_DRIVER_NIG, nig, Q, x.data(), W.data(), nullptr) == LLL_OK &&
+                     lll_set_strikes(c, 1, K.data()) == LLL_OK, "init");
+        for (int scheme : {LLL_FULL, LLL_FROZEN}) {
+            g_need.clear();
+            bad += check(lll_simulate(c, scheme, 0, 5000, 1) == LLL_OK, "simulate");
+            for (const Need &q : g_need) bad += check(q.rows == 24 * 1024 / (2 * 32 * 16), "rows of a longer curve");
+        }
+        lll_destroy(c);
+    }
+    return bad;
+}
 }  // namespace
 
 int main(int argc, char **argv)
@@ -190,5 +238,6 @@ int main(int argc, char **argv)
     if (what == "compensators") return compensators();
     if (what == "selections") return selections();
     if (what == "fewer_paths") return fewer_paths();
+    if (what == "limits") return limits();
     return 2;
 }
