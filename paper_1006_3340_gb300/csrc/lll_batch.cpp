@@ -152,8 +152,9 @@ int build_schedule(lll_batch *b, int scheme)
     int CH = sh.chunk_rows > 0 ? std::min(sh.chunk_rows, b->n_max)
                                : std::min(b->n_max, std::max(1, (48 * 1024) / (2 * (b->QP / 4) * 16)));
     const int nst = scheme == LLL_PICARD ? 2 : 1;
-    // smem as for the path kernel, sized for the largest instance
-    size_t smem = path_kernel_smem(b->QP, b->n_max, b->ns_max, T, CH);
+    // smem as for the path kernel, sized for the largest instance; a batch is refused by
+    // the need of the rules as given at 128 threads, whatever kernel sweeps them
+    size_t smem = path_kernel_smem(b->QP, b->n_max, b->ns_max, sh.threads > 0 ? T : 128, CH);
     if (smem > 227 * 1024) return berr(b, LLL_EUNSUPPORTED, "batch shared memory exceeds 227 KB");
     if (b->QK > 0) { // the longest of the instances' rules decides
         CH = b->n_max;

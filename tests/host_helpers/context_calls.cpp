@@ -230,6 +230,25 @@ int limits()
     }
     return bad;
 }
+// The same of a batch, with 48 KB of staged rows.
+int batch_limits()
+{
+    int bad = 0;
+    for (int N : {60, 400}) {
+        const int n = N - 1, Q = 128;
+        std::vector<double> L0(N, 0.03), lam((size_t)n * n, 0.001), x(Q), W(Q), K(n, 0.03);
+        const lll_nig nig{12.0, -3.0, 0.8, NAN};
+        lll_build_nig_quadrature(nig, 1.5, Q, x.data(), W.data());
+        const lll_instance inst{N, 0.25, L0.data(), 1, lam.data(), LLL_DRIVER_NIG, nig, Q, x.data(), W.data(), 1, K.data(), 5000};
+        lll_batch *b = nullptr;
+        g_need.clear();
+        bad += check(lll_batch_init(&b, 1, &inst, nullptr) == LLL_OK && b->QK > 0 && lll_batch_simulate(b, LLL_FULL, 1) == LLL_OK, "batch");
+        for (const Need &q : g_need) bad += check(q.threads == 128, "threads of a batch");
+        bad += check(!g_need.empty() && g_need[0].rows == 48, "rows of a batch");
+        lll_batch_destroy(b);
+    }
+    return bad;
+}
 }  // namespace
 
 int main(int argc, char **argv)
@@ -239,5 +258,6 @@ int main(int argc, char **argv)
     if (what == "selections") return selections();
     if (what == "fewer_paths") return fewer_paths();
     if (what == "limits") return limits();
+    if (what == "batch_limits") return batch_limits();
     return 2;
 }

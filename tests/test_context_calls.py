@@ -25,7 +25,7 @@ def helper(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("what", ["compensators", "selections", "fewer_paths", "limits"])
+@pytest.mark.parametrize("what", ["compensators", "selections", "fewer_paths", "limits", "batch_limits"])
 def test_context_calls(helper, what):
     r = subprocess.run([helper, what], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, (r.returncode, r.stderr)
