@@ -114,27 +114,34 @@ void gauss_of_jacobi(const std::vector<double> &al, const std::vector<double> &b
         lo = std::min(lo, al[k] - rad);
         hi = std::max(hi, al[k] + rad);
     }
-    auto count_below = [&](double lam) {
-        int cnt = 0;
-        double d = 1.0;
+    // All eigenvalues are bisected side by side: a Sturm sequence is a chain of
+    // divisions, and Q independent chains overlap where one after the other waited for
+    // each quotient (the search of shorter_rule that ends without a rule, 64 nodes:
+    // 0.79 -> 0.36 ms).  The numbers are those of one bisection at a time.
+    std::vector<double> a0(Q, lo), b0(Q, hi), mid(Q), d(Q);
+    std::vector<int> below(Q);
+    for (int it = 0; it < 200; ++it) {
+        bool moving = false;
+        for (int j = 0; j < Q; ++j) {
+            mid[j] = 0.5 * (a0[j] + b0[j]);
+            moving = moving || (mid[j] > a0[j] && mid[j] < b0[j]);
+            d[j] = 1.0;
+            below[j] = 0;
+        }
+        if (!moving) break;
         for (int k = 0; k < Q; ++k) {
-            const double off = k > 0 ? bt[k] * bt[k] : 0.0;
-            d = al[k] - lam - (k > 0 ? off / d : 0.0);
-            if (d == 0.0) d = -1e-300;
-            if (d < 0.0) ++cnt;
+            const double off = k > 0 ? bt[k] * bt[k] : 0.0, alk = al[k];
+            for (int j = 0; j < Q; ++j) {
+                double v = alk - mid[j] - off / d[j];
+                v = v == 0.0 ? -1e-300 : v;
+                below[j] += v < 0.0;
+                d[j] = v;
+            }
         }
-        return cnt;
-    };
-    for (int j = 0; j < Q; ++j) {
-        double a0 = lo, b0 = hi;
-        for (int it = 0; it < 200 && b0 - a0 > 0.0; ++it) {
-            const double mid = 0.5 * (a0 + b0);
-            if (mid <= a0 || mid >= b0) break;
-            if (count_below(mid) > j) b0 = mid;
-            else a0 = mid;
-        }
-        nodes[j] = 0.5 * (a0 + b0);
+        for (int j = 0; j < Q; ++j)
+            if (mid[j] > a0[j] && mid[j] < b0[j]) (below[j] > j ? b0 : a0)[j] = mid[j];
     }
+    for (int j = 0; j < Q; ++j) nodes[j] = 0.5 * (a0[j] + b0[j]);
     // Christoffel numbers from the orthonormal recurrence.
     for (int j = 0; j < Q; ++j) {
         const double xx = nodes[j];
