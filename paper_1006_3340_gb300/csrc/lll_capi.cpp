@@ -586,22 +586,29 @@ int lll_set_mapping(lll_ctx *ctx, int mapping, int lanes)
 namespace {
 
 // Whether the step mapping of a default launch runs the path mapping's kernels
-// instead (the same log-rates bit for bit).  Up to 8 nodes the pipeline and the
-// time-blocked kernel are faster at every path count: N = 40, 2000 paths 0.127
-// against 0.153 ms, 4096 paths 0.127 against 0.229, 50,000 paths 0.83 against
-// 1.93; N = 10, 2000 paths 0.040 against 0.052.  Longer rules keep the step
-// kernels, whose threads do not carry products across steps, while their
-// intermediate arrays are small: N = 120 (20 nodes), 2000 paths 0.53 against 0.75
-// ms, 4096 paths (1.2e8 units) 0.89 against 0.75; the 9-rate heavy-tailed example
-// (32 nodes), 8192 paths (1.8e6 units) 0.058 against 0.090.  The two unit counts lie
-// between such pairs of points, one curve each.
+// instead (the same log-rates bit for bit): where they are the faster by the three
+// kernels' estimates.  The step kernels' time is nearly the same from 32 to 1000
+// paths and then grows by the unit; the pipeline's is its ticks, the block kernel's a
+// path's latency, until the paths fill the GPU.  N = 40 (8 nodes), us: 32 paths 121
+// in the pipeline, 102 in the step kernels; 4096 paths 127 and 232; 64,000 paths 977
+// (block) and 2543.  N = 120: 20 nodes 1000 paths 741 and 372, 4096 paths 744 and
+// 902; 8 nodes and 8 steps a period, where the pipeline does not fit shared memory,
+// 2000 paths 4062 (block) and 775.  Over 20 curves (1 to 299 rates, 1 to 500 steps a
+// period, 4 to 32 nodes) and 32 to 130,000 paths the estimates cost 0.7 % against the
+// better choice, a third at worst.
 bool step_as_path(const lll_ctx *ctx, uint64_t paths)
 {
     if (ctx->QR >= ctx->QP || ctx->lpp > 1 || ctx->ppt > 0 || ctx->threads > 0 || ctx->blocks_per_sm > 0 ||
         ctx->chunk_rows > 0)
         return false;
-    const double units = (double)paths * ctx->s * ctx->n * (ctx->n + 1) / 2;
-    return ctx->QR <= 8 || units > (ctx->n >= 24 ? 1e8 : 4e6);
+    const uint64_t tiles = (paths + 31) / 32;
+    size_t smem = 0;
+    const int shape = ctx->product == LLL_PRODUCT_CAPLET
+                          ? pipe_shape(LLL_PICARD, ctx->QR, ctx->n, ctx->s, ctx->S, tiles, ctx->sm_count, &smem)
+                          : 0;
+    const double path_us = shape ? pipe_estimate_us(ctx->QR, shape, smem, ctx->n, ctx->s, tiles, ctx->sm_count)
+                                 : block_estimate_us(ctx->QR, ctx->n, ctx->s, paths);
+    return path_us <= step_estimate_us(ctx->n, ctx->s, paths);
 }
 
 // The Picard scheme with its Euler steps in parallel (lll_paths_step.cu):

@@ -100,6 +100,7 @@ size_t path_kernel_smem(int QP, int n, int ns, int threads, int chunk_rows);
 // QMAX = 8 or 32).
 int block_chunk_rates(int QP, int R, int n, int rows);
 size_t block_kernel_smem(int QP, int R, int n, int threads, int chunk_rates);
+double block_estimate_us(int QP, int n, int s, uint64_t paths);
 int block_kernel_prepare(int scheme, int product, int QP, int R, uint64_t paths, size_t smem, int threads, int *blocks_per_sm);
 int launch_block_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st,
                         const PathArgs &a);
@@ -111,6 +112,7 @@ int launch_batch_block_kernel(int scheme, int QMAX, int R, int grid, int threads
 // pipeline of warps over the rates).
 constexpr int kMaxPipePerSm = 8; // blocks an SM of its largest launch
 int pipe_shape(int scheme, int QP, int n, int s, int S, uint64_t tiles, int sms, size_t *smem);
+double pipe_estimate_us(int QP, int shape, size_t smem, int n, int s, uint64_t tiles, int sms);
 int launch_pipe_kernel(int scheme, int QP, int shape, size_t smem, uint64_t paths, cudaStream_t st, const PathArgs &a);
 
 // Launchers implemented in lll_paths_group.cu (four lanes per group of four paths).
@@ -129,6 +131,7 @@ int launch_tenor_kernel(int scheme, int QP, int G, int grid, size_t smem, cudaSt
 // Launchers implemented in lll_paths_step.cu (Picard with its Euler steps in parallel).
 bool step_kernels_supported(int QP, bool shorter, int ns);
 size_t step_bytes_per_path(int n, int S);
+double step_estimate_us(int n, int s, uint64_t paths);
 int step_blocks_per_chunk(int Pc);
 int launch_step_chunk(int QP, bool shorter, const PathArgs &a, uint64_t chunk_first, int Pc, float *dH, float *Y, float *Bh,
                       float *Zm, int block0, double *partials, cudaStream_t st);

@@ -11,6 +11,8 @@
 // of the rule as given (lll_paths.cu): Picard, N = 40, 64 -> 8 nodes, 2^20
 // paths 59.8 -> 12.7 ms; full, N = 120, 96 -> 20 nodes, 2^17 paths 63.1 -> 13.6
 // ms; full, N = 40, 4096 paths 2.11 -> 0.60 ms (the pipeline: 0.15).
+#include <algorithm>
+
 #include <cuda_runtime.h>
 
 #include "lll_paths_block.cuh"
@@ -113,6 +115,15 @@ int block_chunk_rates(int QP, int R, int n, int rows)
 size_t block_kernel_smem(int QP, int R, int n, int threads, int chunk_rates)
 {
     return block_smem_bytes(QP, steps_of(QP, R), R, n, threads, chunk_rates);
+}
+
+// Time of a launch on default shape in us (see step_as_path): one tile's latency, or all
+// tiles' throughput, by (rate, step block) and by unit.
+double block_estimate_us(int QP, int n, int s, uint64_t paths)
+{
+    const int B = steps_of(QP, 1);
+    const double pairs = 0.5 * n * (n + 1.0), blocks = pairs * ((s + B - 1) / B), units = pairs * s;
+    return 10.0 + std::max(0.25 * blocks + 0.045 * units + 0.4 * n * s, (double)paths * (8e-6 * blocks + 1.3e-6 * units));
 }
 
 int block_kernel_prepare(int scheme, int product, int QP, int R, uint64_t paths, size_t smem, int threads,

@@ -326,6 +326,17 @@ int pipe_shape(int scheme, int QP, int n, int s, int S, uint64_t tiles, int sms,
     return B | lg << 8;
 }
 
+// Time of such a launch in us, for the choice of lll_set_mapping(LLL_MAP_STEP): its
+// ticks by the rates a warp takes through one (see step_as_path).
+double pipe_estimate_us(int QP, int shape, size_t smem, int n, int s, uint64_t tiles, int sms)
+{
+    const int B = shape & 255, G = 1 << (shape >> 8);
+    const double ticks = (double)n * ((s + B - 1) / B) + G - 1, rates = (n + G - 1) / G;
+    const uint64_t per_sm = (tiles + sms - 1) / sms;
+    const uint64_t at_once = n < 24 ? per_sm : QP <= 8 && B == 4 && 227 * 1024 / smem >= 2 ? 2 : 1;
+    return 10.0 + (double)((per_sm + at_once - 1) / at_once) * ticks * (1.0 + (B == 8 ? 0.32 : 0.16) * rates);
+}
+
 int launch_pipe_kernel(int scheme, int QP, int shape, size_t smem, uint64_t paths, cudaStream_t st, const PathArgs &a)
 {
     const int B = shape & 255, lg = shape >> 8;

@@ -280,6 +280,14 @@ bool step_kernels_supported(int QP, bool shorter, int ns) { return pick_sweep(QP
 
 size_t step_bytes_per_path(int n, int S) { return 4 * ((size_t)S + 2 * (size_t)S * n + (size_t)n * n); }
 
+// Time of the five kernels in us for a shorter rule (see step_as_path): their launches,
+// the scans over the steps, the sweep over the rates, and the units of all paths.
+double step_estimate_us(int n, int s, uint64_t paths)
+{
+    const double S = (double)n * s;
+    return 25.0 + 0.16 * S + 0.6 * n + 7e-6 * (double)paths * s * 0.5 * n * (n + 1.0);
+}
+
 int step_blocks_per_chunk(int Pc) { return (int)blocks_of((size_t)Pc); }
 
 size_t step_sweep_smem(int QP, int n)
