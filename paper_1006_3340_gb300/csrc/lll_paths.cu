@@ -107,7 +107,8 @@ __device__ __forceinline__ void issue_chunk(const PathArgs &a, const Smem &sm, i
 
 // One tile of T*R paths of the simulation `a`: all Euler steps, payoffs
 // accumulated into sm.bsum.  st: this thread's column of the block's state slot.
-template <int SCHEME, int QP, int R>
+// INLINE: see draw_increment.
+template <int SCHEME, int QP, int R, bool INLINE>
 __device__ __forceinline__ void run_tile(const PathArgs &a, const Smem &sm, float *st, uint64_t tile)
 {
     constexpr int Q2 = QP > 0 ? QP / 2 : 1; // node pairs
@@ -144,7 +145,7 @@ __device__ __forceinline__ void run_tile(const PathArgs &a, const Smem &sm, floa
             const bool mat = (k + 1) % s == 0;     // rate imin fixes at t_{k+1} = T_imin
             float dH[R];
 #pragma unroll
-            for (int q = 0; q < R; ++q) dH[q] = draw_increment(a, p[q], (uint32_t)k);
+            for (int q = 0; q < R; ++q) dH[q] = draw_increment<INLINE>(a, p[q], (uint32_t)k);
 
             // scaled products P~_j = c_j P_j, P = 1 above the top rate
             float2 P[R][Q2];
@@ -321,9 +322,21 @@ __device__ __forceinline__ void run_tile(const PathArgs &a, const Smem &sm, floa
 //   LB 2: 102 registers, five blocks of at most 128 threads per SM.
 template <int LB>
 struct Bounds {
-    static constexpr int threads = LB == 2 ? 128 : kMaxThreads;
-    static constexpr int blocks = LB == 0 ? 1 : (LB == 1 ? 2 : 5);
+    static constexpr int threads = LB >= 2 ? 128 : kMaxThreads;
+    static constexpr int blocks = LB == 0 ? 1 : LB == 1 ? 2 : LB == 2 ? 5 : 7;
 };
+
+// Kernels that draw with the decision in line (out of line / in line, us): Picard on
+// 64 nodes, 200,000 paths of N = 40 12350 / 11500; Brownian full, 2000 paths 834 / 772.
+// The others: full on 64 nodes, 2000 paths 2030 / 2100; Brownian Picard, 200,000 paths
+// 4740 / 4840; 96 nodes 19700 / 20700 (Picard), 15100 / 17300 (full); 32 nodes 785 / 838
+// (Picard); frozen drift, N = 10, 10,000 paths 116 / 122, once its registers are held to
+// seven blocks of 128 threads an SM (else six fit, and N = 40 on 200,000 paths takes
+// 3350, not 2900).
+__host__ __device__ constexpr bool draws_inline(int scheme, int QP, int R)
+{
+    return R == 1 && ((scheme == PICARD && QP == 64) || (scheme == FULL && QP == 0));
+}
 
 template <int SCHEME, int QP, int R, int LB>
 __global__ void __launch_bounds__(Bounds<LB>::threads, Bounds<LB>::blocks) path_kernel(const PathArgs a)
@@ -339,7 +352,7 @@ __global__ void __launch_bounds__(Bounds<LB>::threads, Bounds<LB>::blocks) path_
     // This block's state slot: [R][NST][n][T]; thread tid owns column tid.
     float *st = a.state + (size_t)blockIdx.x * R * NST * n * T + tid;
     const uint64_t ntiles = (a.paths + (uint64_t)T * R - 1) / ((uint64_t)T * R);
-    for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) run_tile<SCHEME, QP, R>(a, sm, st, tile);
+    for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) run_tile<SCHEME, QP, R, draws_inline(SCHEME, QP, R)>(a, sm, st, tile);
     __syncthreads();
     double *out = a.partials + (size_t)blockIdx.x * n * ns * 2;
     for (int e = tid; e < n * ns; e += T) {
@@ -386,7 +399,7 @@ __global__ void __launch_bounds__(kMaxThreads) batch_kernel(const BatchArgs b)
         }
         for (int e = tid; e < 4 * a->n * a->ns; e += T) sm.bsum[e] = 0.0;
         const uint2 tr = b.item_tiles[it];
-        for (uint32_t t = tr.x; t < tr.y; ++t) run_tile<SCHEME, QP, R>(*a, sm, st, t);
+        for (uint32_t t = tr.x; t < tr.y; ++t) run_tile<SCHEME, QP, R, false>(*a, sm, st, t);
         __syncthreads();
         double *out = b.partials + b.seg_off[it];
         for (int e = tid; e < a->n * a->ns; e += T) {
@@ -408,7 +421,7 @@ KernelFn pick_r(int R, int T)
 {
     if (R == 1) {
         if constexpr (QP <= 32) {
-            if (T <= 128) return path_kernel<SCHEME, QP, 1, 2>;
+            if (T <= 128) return path_kernel<SCHEME, QP, 1, SCHEME == FROZEN ? 3 : 2>;
         }
         if constexpr (QP <= 96) return path_kernel<SCHEME, QP, 1, 1>;
         else return path_kernel<SCHEME, QP, 1, 0>;

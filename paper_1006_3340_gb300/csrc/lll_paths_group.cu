@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kMaxThreads, (QP <= 64 ? 2 : 1)) group_kernel(
             const int imin = k / s + 1;
             const int nch = (n - imin + CH) / CH;
             const bool mat = (k + 1) % s == 0;
-            const float dH = draw_increment(a, p, (uint32_t)k);
+            const float dH = draw_increment<true>(a, p, (uint32_t)k); // N = 40, 100,000 paths 7.74 -> 7.14 ms in line
             // P[q][2j + hf]: scaled product c P of path q of the group, node
             // pair hf of table entry G j + t
             float2 P[G][2 * QL];

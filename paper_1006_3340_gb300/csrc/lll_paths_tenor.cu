@@ -193,7 +193,8 @@ __global__ void __launch_bounds__(kTenorThreads) tenor_kernel(const PathArgs a, 
             // increments: lane g draws step k + g once every G steps
             if (k % G == 0) {
                 const int kk = k + g;
-                dh_mine = (active && kk < S) ? draw_increment(a, pid, (uint32_t)kk) : 0.0f;
+                // (in line: N = 120, eight lanes, 4096 paths 9.82 -> 9.27 ms)
+                dh_mine = (active && kk < S) ? draw_increment<true>(a, pid, (uint32_t)kk) : 0.0f;
             }
             const float dH = __shfl_sync(FULLMASK, dh_mine, gbase + (k % G));
             cp_wait_1();

@@ -32,9 +32,9 @@ __global__ void math_kernel(int what, const float *a, const float *b, int count,
 
 // Draws of `count` paths at step k: how many increments are nearer to the root
 // that the FP64 decision does not take, how many draws lie within `band` of the
-// threshold, and the smallest distance from it seen (relative).
+// threshold (relative), and how many differ between the two forms of the draw.
 __global__ void root_kernel(PathArgs a, uint32_t k, int count, double band, unsigned long long *wrong,
-                            unsigned long long *near)
+                            unsigned long long *near, unsigned long long *differ)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= count) return;
@@ -47,9 +47,11 @@ __global__ void root_kernel(PathArgs a, uint32_t k, int count, double band, unsi
     const bool take_small = u2 <= m / (m + small);
     auto increment = [&](double V) { return (double)a.nig_beta * V + sqrt(V) * z2 + (double)a.nig_muh; };
     const double right = increment(take_small ? small : large), other = increment(take_small ? large : small);
-    const double got = draw_increment(a, (uint64_t)p, k);
+    const float out_of_line = draw_increment<false>(a, (uint64_t)p, k), in_line = draw_increment<true>(a, (uint64_t)p, k);
+    const double got = out_of_line;
     if (fabs(t - m) < band * m) atomicAdd(near, 1ull);
     if (fabs(right - other) > 1e-4 * (fabs(right) + fabs(other)) && fabs(got - right) > fabs(got - other)) atomicAdd(wrong, 1ull);
+    if (__float_as_uint(out_of_line) != __float_as_uint(in_line)) atomicAdd(differ, 1ull);
 }
 
 extern "C" int device_math(int what, const float *a, const float *b, int count, double *err)
@@ -75,7 +77,7 @@ extern "C" int device_math(int what, const float *a, const float *b, int count, 
 // Increments of the normal inverse Gaussian driver (m, l: mean and shape of the
 // mixing variable over a step).
 extern "C" int device_roots(double m, double l, double beta, double muh, unsigned key, unsigned k, int count, double band,
-                            unsigned long long *wrong, unsigned long long *near)
+                            unsigned long long *wrong, unsigned long long *near, unsigned long long *differ)
 {
     PathArgs a{};
     a.driver = 0;
@@ -83,16 +85,17 @@ extern "C" int device_roots(double m, double l, double beta, double muh, unsigne
     a.ig_m = (float)m; a.ig_m2 = (float)(m * m); a.ig_hl = (float)(m / (2.0 * l));
     a.ig_fl = (float)(4.0 * m * l); a.ig_md = m; a.ig_ld = l;
     a.nig_beta = (float)beta; a.nig_muh = (float)muh;
-    unsigned long long *d = nullptr, h[2] = {0, 0};
+    unsigned long long *d = nullptr, h[3] = {0, 0, 0};
     cudaError_t e = cudaMalloc((void **)&d, sizeof h);
     if (e == cudaSuccess) e = cudaMemset(d, 0, sizeof h);
     if (e == cudaSuccess) {
-        root_kernel<<<(count + 127) / 128, 128>>>(a, k, count, band, d, d + 1);
+        root_kernel<<<(count + 127) / 128, 128>>>(a, k, count, band, d, d + 1, d + 2);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpy(h, d, sizeof h, cudaMemcpyDeviceToHost);
     cudaFree(d);
     *wrong = h[0];
     *near = h[1];
+    *differ = h[2];
     return (int)e;
 }

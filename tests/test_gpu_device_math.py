@@ -34,7 +34,7 @@ def dev(tmp_path_factory):
     lib = ctypes.CDLL(so)
     V, D, I, U = ctypes.c_void_p, ctypes.c_double, ctypes.c_int, ctypes.c_uint
     lib.device_math.argtypes = [I, V, V, I, V]
-    lib.device_roots.argtypes = [D, D, D, D, U, U, I, D, V, V]
+    lib.device_roots.argtypes = [D, D, D, D, U, U, I, D, V, V, V]
     return lib
 
 
@@ -79,11 +79,11 @@ def test_root_of_the_inverse_gaussian_draw_is_the_one_of_fp64(dev, maker):
     wl = maker()
     gam = np.sqrt(wl.alpha ** 2 - wl.beta ** 2)
     h = wl.delta / wl.s
-    wrong, near, total = ctypes.c_ulonglong(), ctypes.c_ulonglong(), 0
+    wrong, near, differ, total = ctypes.c_ulonglong(), ctypes.c_ulonglong(), ctypes.c_ulonglong(), 0
     for k in range(4):
         rc = dev.device_roots(wl.dbar * h / gam, (wl.dbar * h) ** 2, wl.beta, -wl.dbar * wl.beta / gam * h, 17, k, 1 << 23, 4e-5,
-                              ctypes.addressof(wrong), ctypes.addressof(near))
+                              ctypes.addressof(wrong), ctypes.addressof(near), ctypes.addressof(differ))
         assert rc == 0
-        assert wrong.value == 0
+        assert wrong.value == 0 and differ.value == 0
         total += near.value
     assert total > 100  # the band in which FP32 and FP64 could differ has been drawn
