@@ -32,9 +32,8 @@ __device__ __forceinline__ void batch_item(const PathArgs &a, unsigned char *sme
     for (int e = tid; e < a.n; e += T) sm.c0[e] = -1.4426950408889634f * a.c0[e];
     for (int e = tid; e < QP; e += T) reinterpret_cast<float *>(sm.cn)[e] = a.cn[e];
     State<NST * R> *st = reinterpret_cast<State<NST * R> *>(state) + tid;
-    bool beyond; // (of swaptions)
     for (uint32_t t = tiles.x; t < tiles.y; ++t)
-        block_tile<SCHEME, QP, B, R, CAPLETS>(a, sm, st, t, acc, comp, t == tiles.x, beyond);
+        block_tile<SCHEME, QP, B, R, CAPLETS>(a, sm, st, t, acc, comp, t == tiles.x);
 }
 
 template <int SCHEME, int QMAX, int R>
@@ -129,7 +128,8 @@ double block_estimate_us(int QP, int n, int s, uint64_t paths)
 int block_kernel_prepare(int scheme, int product, int QP, int R, uint64_t paths, size_t smem, int threads,
                          int *blocks_per_sm)
 {
-    return prepare(pick_kernel(scheme, product, QP, R, paths), smem, kMaxSmem, threads, blocks_per_sm);
+    // less its static shared memory
+    return prepare(pick_kernel(scheme, product, QP, R, paths), smem, kMaxSmem - 1024, threads, blocks_per_sm);
 }
 
 int launch_block_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st, const PathArgs &a)

@@ -46,11 +46,15 @@ __global__ void __launch_bounds__(kMaxThreads, BL) block_kernel(const PathArgs a
     const size_t nout = (size_t)a.n * a.ns * 2;
     double *acc = a.partials + blockIdx.x * nout, *comp = a.partials + (gridDim.x + blockIdx.x) * nout;
     const uint64_t TP = (uint64_t)T * R, ntiles = (a.paths + TP - 1) / TP;
-    bool beyond = false;
+    __shared__ int beyond; // (of the swaptions' kernels only)
+    if (PRICES == SWAPTIONS && tid == 0) beyond = 0; // ordered by the tile's first barrier
     for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-        block_tile<SCHEME, QP, B, R, PRICES>(a, sm, st, tile, acc, comp, tile == blockIdx.x, beyond);
+        block_tile<SCHEME, QP, B, R, PRICES>(a, sm, st, tile, acc, comp, tile == blockIdx.x, &beyond);
     // a mark for wide_kernel, which runs next
-    if (PRICES == SWAPTIONS && __syncthreads_or(beyond) && tid == 0) comp[0] = nan("");
+    if (PRICES == SWAPTIONS) {
+        __syncthreads();
+        if (tid == 0 && beyond) comp[0] = nan("");
+    }
 }
 
 // The full scheme on 20 nodes runs as well in two blocks of 128 threads an SM at

@@ -4,10 +4,12 @@
 // Payoffs are formed in pairs of FP32 numbers (maturity_values): FP64 has a 64th of
 // the FP32 rate.  The pairs have FP32's exponents, so a block that meets a value
 // beyond their range (beyond_pairs) marks its sums, and wide_kernel, launched behind,
-// runs that block's tiles again with FP64 payoffs: 300,007 paths of N = 40, 3.81 ms in
-// pairs, 9.73 ms where every block goes to wide_kernel.  Without a mark wide_kernel
-// ends at once: 9 rates, 8000 paths 131 us a call, 128 without its launch.  (Formed in
-// FP64 within the first kernel instead, the code for it alone cost 2.5 % there.)
+// runs that block's tiles again with FP64 payoffs: 300,007 paths of N = 40, 3.89 ms a
+// call in pairs (3.87 without the check), 9.8 ms where every block goes to wide_kernel.
+// Without a mark wide_kernel ends at once: 9 rates, 8000 paths 131 us a call, 128
+// without its launch.  (Formed in FP64 within the first kernel instead, the code for it
+// alone cost 2.5 % there; the mark kept in a register until the end, N = 120 on 60,000
+// paths took 8.98 ms, 8.62 with the word in shared memory, 8.49 without a check.)
 #include "lll_paths_block.cuh"
 
 namespace lll {
@@ -38,10 +40,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1) wide_kernel(const PathArgs a, 
         double *acc = a.partials + b * nout, *comp = a.partials + (blocks + b) * nout;
         if (!a.wide_strikes && !isnan(comp[0])) continue; // the same for all threads
         __syncthreads();                                  // before the mark is written over
-        bool beyond, first = true;
+        bool first = true;
         for (uint64_t tile = b; tile < ntiles; tile += blocks)
             for (int q = 0; q < R; ++q) {
-                block_tile<SCHEME, QP, B, 1, WIDE_SWAPTIONS>(a, sm, st, tile * R + q, acc, comp, first, beyond);
+                block_tile<SCHEME, QP, B, 1, WIDE_SWAPTIONS>(a, sm, st, tile * R + q, acc, comp, first);
                 first = false;
             }
     }

@@ -185,11 +185,12 @@ enum { CAPLETS = 0, SWAPTIONS = 1, WIDE_SWAPTIONS = 2 };
 // payoffs of every G-th path in double-float pairs (FP64: WIDE_SWAPTIONS), and
 // thread q the G slices.  (Reducing each strike over the warp's lanes instead, by
 // shuffles, took 0.25 of 2.08 ms on the N = 40 workload and three times the
-// latency.)  beyond: set where a swaption of this thread's paths is beyond the pairs.
+// latency.)  beyond (SWAPTIONS): a word in shared memory, set where a swaption of the
+// block's paths is beyond the pairs.
 template <int NST, int R, int PRICES>
 __device__ __forceinline__ void block_maturity(const PathArgs &a, const BlockSmem &sm, const State<NST * R> *st, int T,
                                                int m, const uint64_t (&lp)[R], double *acc, double *comp, bool first,
-                                               bool &beyond)
+                                               int *beyond)
 {
     constexpr bool WIDE = PRICES == WIDE_SWAPTIONS;
     const int n = a.n, ns = a.ns, tid = threadIdx.x;
@@ -211,7 +212,9 @@ __device__ __forceinline__ void block_maturity(const PathArgs &a, const BlockSme
         } else {
             float4 v = maturity_values(a, product, m, z);
             if (lp[u] >= a.paths) v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if constexpr (PRICES == SWAPTIONS) beyond = beyond || beyond_pairs(v);
+            if constexpr (PRICES == SWAPTIONS) {
+                if (beyond_pairs(v)) *beyond = 1;
+            }
             sm.pay[u * T + tid] = v;
         }
         if (a.snap != nullptr && lp[u] < a.paths && lp[u] % a.snap_stride == 0 && lp[u] / a.snap_stride < a.n_snap)
@@ -326,7 +329,7 @@ __device__ __forceinline__ void sweep_chunk(const PathArgs &a, const BlockSmem &
 // hold nothing yet; beyond: see block_maturity.
 template <int SCHEME, int QP, int B, int R, int PRICES>
 __device__ __forceinline__ void block_tile(const PathArgs &a, const BlockSmem &sm, State<(SCHEME == PICARD ? 2 : 1) * R> *st,
-                                           uint64_t tile, double *acc, double *comp, bool first, bool &beyond)
+                                           uint64_t tile, double *acc, double *comp, bool first, int *beyond = nullptr)
 {
     constexpr int NST = (SCHEME == PICARD) ? 2 : 1;
     const int T = blockDim.x, tid = threadIdx.x;
