@@ -594,8 +594,8 @@ namespace {
 // (block) and 2543.  N = 120: 20 nodes 1000 paths 741 and 372, 4096 paths 744 and
 // 902; 8 nodes and 8 steps a period, where the pipeline does not fit shared memory,
 // 2000 paths 4062 (block) and 775.  Over 20 curves (1 to 299 rates, 1 to 500 steps a
-// period, 4 to 32 nodes) and 32 to 130,000 paths the estimates cost 0.7 % against the
-// better choice, a third at worst.
+// period, 4 to 32 nodes) and 32 to 130,000 paths the estimates cost 0.4 % against the
+// better choice, 29 % at worst.
 bool step_as_path(const lll_ctx *ctx, uint64_t paths)
 {
     if (ctx->QR >= ctx->QP || ctx->lpp > 1 || ctx->ppt > 0 || ctx->threads > 0 || ctx->blocks_per_sm > 0 ||

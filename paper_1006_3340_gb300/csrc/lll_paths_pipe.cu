@@ -334,7 +334,7 @@ double pipe_estimate_us(int QP, int shape, size_t smem, int n, int s, uint64_t t
     const double ticks = (double)n * ((s + B - 1) / B) + G - 1, rates = (n + G - 1) / G;
     const uint64_t per_sm = (tiles + sms - 1) / sms;
     const uint64_t at_once = n < 24 ? per_sm : QP <= 8 && B == 4 && 227 * 1024 / smem >= 2 ? 2 : 1;
-    return 10.0 + (double)((per_sm + at_once - 1) / at_once) * ticks * (1.0 + (B == 8 ? 0.32 : 0.16) * rates);
+    return 10.0 + (double)((per_sm + at_once - 1) / at_once) * ticks * (1.0 + rates * (0.08 + 0.003 * (s < B ? s : B) * QP));
 }
 
 int launch_pipe_kernel(int scheme, int QP, int shape, size_t smem, uint64_t paths, cudaStream_t st, const PathArgs &a)

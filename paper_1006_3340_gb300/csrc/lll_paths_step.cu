@@ -285,7 +285,7 @@ size_t step_bytes_per_path(int n, int S) { return 4 * ((size_t)S + 2 * (size_t)S
 double step_estimate_us(int n, int s, uint64_t paths)
 {
     const double S = (double)n * s;
-    return 25.0 + 0.16 * S + 0.6 * n + 7e-6 * (double)paths * s * 0.5 * n * (n + 1.0);
+    return 25.0 + 0.16 * S + 0.6 * n + (7e-6 + 1.2e-8 * n) * (double)paths * s * 0.5 * n * (n + 1.0);
 }
 
 int step_blocks_per_chunk(int Pc) { return (int)blocks_of((size_t)Pc); }
