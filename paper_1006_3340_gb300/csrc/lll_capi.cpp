@@ -250,9 +250,9 @@ int plan_launch(lll_ctx *ctx, int scheme, uint64_t first_path, uint64_t paths, u
         e = (cudaError_t)block_kernel_prepare(scheme, ctx->product, ctx->QR, R, paths, smem, T, &occ);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "block kernel attributes");
     } else {
-        e = (cudaError_t)path_kernel_prepare(scheme, QPk, R, T, smem);
+        e = (cudaError_t)path_kernel_prepare(scheme, QPk, R, paths, T, smem);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
-        e = (cudaError_t)path_kernel_occupancy(scheme, QPk, R, T, smem, &occ);
+        e = (cudaError_t)path_kernel_occupancy(scheme, QPk, R, paths, T, smem, &occ);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy");
     }
     if (occ < 1) return fail(ctx, LLL_EUNSUPPORTED, "launch shape does not fit on an SM");

@@ -90,8 +90,8 @@ struct LaunchPlan {
 // R = paths carried per thread (1, or 2 where compiled: padded Q <= 64).
 int launch_path_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st,
                        const PathArgs &a);
-int path_kernel_occupancy(int scheme, int QP, int R, int threads, size_t smem, int *blocks_per_sm);
-int path_kernel_prepare(int scheme, int QP, int R, int threads, size_t smem);
+int path_kernel_occupancy(int scheme, int QP, int R, uint64_t paths, int threads, size_t smem, int *blocks_per_sm);
+int path_kernel_prepare(int scheme, int QP, int R, uint64_t paths, int threads, size_t smem);
 bool path_kernel_supported(int scheme, int QP, int R);
 size_t path_kernel_smem(int QP, int n, int ns, int threads, int chunk_rows);
 

@@ -330,9 +330,7 @@ struct Bounds {
 // 64 nodes, 200,000 paths of N = 40 12350 / 11500; Brownian full, 2000 paths 834 / 772.
 // The others: full on 64 nodes, 2000 paths 2030 / 2100; Brownian Picard, 200,000 paths
 // 4740 / 4840; 96 nodes 19700 / 20700 (Picard), 15100 / 17300 (full); 32 nodes 785 / 838
-// (Picard); frozen drift, N = 10, 10,000 paths 116 / 122, once its registers are held to
-// seven blocks of 128 threads an SM (else six fit, and N = 40 on 200,000 paths takes
-// 3350, not 2900).
+// (Picard); frozen drift, N = 10, 10,000 paths 116 / 122.
 __host__ __device__ constexpr bool draws_inline(int scheme, int QP, int R)
 {
     return R == 1 && ((scheme == PICARD && QP == 64) || (scheme == FULL && QP == 0));
@@ -421,7 +419,7 @@ KernelFn pick_r(int R, int T)
 {
     if (R == 1) {
         if constexpr (QP <= 32) {
-            if (T <= 128) return path_kernel<SCHEME, QP, 1, SCHEME == FROZEN ? 3 : 2>;
+            if (T <= 128) return path_kernel<SCHEME, QP, 1, 2>;
         }
         if constexpr (QP <= 96) return path_kernel<SCHEME, QP, 1, 1>;
         else return path_kernel<SCHEME, QP, 1, 0>;
@@ -446,12 +444,17 @@ KernelFn pick_qp(int QP, int R, int T)
     }
 }
 
-KernelFn pick(int scheme, int QP, int R, int T)
+// Frozen drift: beyond the paths of six blocks of 128 threads an SM, a kernel whose
+// registers are held to seven (N = 40, 200,000 paths 2.90 ms, 3.35 with six; 299 rates
+// on 2000 paths 9.04 ms, 8.14 without the bound).
+constexpr uint64_t kFrozenWave = 6 * 152 * 128;
+
+KernelFn pick(int scheme, int QP, int R, int T, uint64_t paths)
 {
     switch (scheme) {
     case FULL: return pick_qp<FULL>(QP, R, T);
     case PICARD: return pick_qp<PICARD>(QP, R, T);
-    case FROZEN: return pick_r<FROZEN, 0>(R, T);
+    case FROZEN: return R == 1 && T <= 128 && paths > kFrozenWave ? path_kernel<FROZEN, 0, 1, 3> : pick_r<FROZEN, 0>(R, T);
     default: return nullptr;
     }
 }
@@ -509,23 +512,23 @@ int launch_batch_kernel(int scheme, int QP, int R, int grid, int threads, size_t
     return (int)cudaGetLastError();
 }
 
-bool path_kernel_supported(int scheme, int QP, int R) { return pick(scheme, QP, R, kMaxThreads) != nullptr; }
+bool path_kernel_supported(int scheme, int QP, int R) { return pick(scheme, QP, R, kMaxThreads, 1) != nullptr; }
 
 size_t path_kernel_smem(int QP, int n, int ns, int threads, int chunk_rows)
 {
     return smem_bytes(QP, n, ns, threads, chunk_rows);
 }
 
-int path_kernel_prepare(int scheme, int QP, int R, int threads, size_t smem)
+int path_kernel_prepare(int scheme, int QP, int R, uint64_t paths, int threads, size_t smem)
 {
-    KernelFn f = pick(scheme, QP, R, threads);
+    KernelFn f = pick(scheme, QP, R, threads, paths);
     if (!f) return (int)cudaErrorInvalidValue;
     return (int)allow_smem(f, smem);
 }
 
-int path_kernel_occupancy(int scheme, int QP, int R, int threads, size_t smem, int *blocks_per_sm)
+int path_kernel_occupancy(int scheme, int QP, int R, uint64_t paths, int threads, size_t smem, int *blocks_per_sm)
 {
-    KernelFn f = pick(scheme, QP, R, threads);
+    KernelFn f = pick(scheme, QP, R, threads, paths);
     if (!f) return (int)cudaErrorInvalidValue;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }
@@ -533,7 +536,7 @@ int path_kernel_occupancy(int scheme, int QP, int R, int threads, size_t smem, i
 int launch_path_kernel(int scheme, int QP, int R, int grid, int threads, size_t smem, cudaStream_t st,
                        const PathArgs &a)
 {
-    KernelFn f = pick(scheme, QP, R, threads);
+    KernelFn f = pick(scheme, QP, R, threads, a.paths);
     if (!f) return (int)cudaErrorInvalidValue;
     // The frozen kernel stages no node table; its QP argument is ignored.
     f<<<grid, threads, smem, st>>>(a);

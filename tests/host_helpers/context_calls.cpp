@@ -78,8 +78,8 @@ size_t path_kernel_smem(int QP, int n, int ns, int threads, int rows)
     g_need.push_back({QP, n, ns, threads, rows});
     return 1024;
 }
-int path_kernel_prepare(int, int, int, int, size_t) { return 0; }
-int path_kernel_occupancy(int, int, int, int, size_t, int *b) { return *b = 4, 0; }
+int path_kernel_prepare(int, int, int, uint64_t, int, size_t) { return 0; }
+int path_kernel_occupancy(int, int, int, uint64_t, int, size_t, int *b) { return *b = 4, 0; }
 int launch_path_kernel(int, int, int, int, int, size_t, cudaStream_t, const PathArgs &a) { return ++g_launches, g_path_tab = a.tab, 0; }
 int block_chunk_rates(int, int, int n, int) { return n; }
 size_t block_kernel_smem(int, int, int, int, int) { return 1024; }

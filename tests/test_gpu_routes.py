@@ -145,3 +145,31 @@ def test_volatilities_of_both_signs(lll, scheme, mapping, launch):
     lam = wl.lam[0]
     assert len(lll.lll_sweep_rule(x, W, lam[lam < 0].sum(), lam[lam > 0].sum())[0]) > 0
     _check(lll, wl, x, W, scheme, 500, launch, mapping)
+
+
+@pytest.mark.parametrize("paths", [116736, 116737, 150001])
+@pytest.mark.parametrize("launch", [None, (64, 0, 0, 1, 1)])
+def test_frozen_drift_on_both_sides_of_its_two_kernels(lll, paths, launch):
+    """The last 64 paths of a launch against the oracle, and its sums against those of the
+    same paths in three smaller launches."""
+    wl = _flat(6, 3, 32, 0.15)
+    x, W = quadrature.rule_for(wl)
+    sim = lll.LevyLibor(wl, x, W)
+    try:
+        if launch:
+            sim.set_launch(*launch)
+        sim.simulate("frozen", paths=paths)
+        s1, s2, _ = sim.sums()
+        p1, p2 = np.zeros_like(s1), np.zeros_like(s2)
+        cuts = [0, paths // 3, 2 * (paths // 3), paths - 64, paths]
+        for a, b in zip(cuts, cuts[1:]):
+            sim.simulate("frozen", paths=b - a, first_path=a, snapshots=64)
+            z = sim.paths(0, 64).astype(np.float64)
+            u1, u2, _ = sim.sums()
+            p1, p2 = p1 + u1, p2 + u2
+    finally:
+        sim.close()
+    assert np.allclose(s1, p1, rtol=1e-12, atol=0) and np.allclose(s2, p2, rtol=1e-12, atol=0)
+    ref = ora.simulate(ora.OracleModel(wl, x, W), ora.FROZEN, path0=paths - 64, npaths=64, want_snap=True)
+    mask = ~np.isnan(ref["snap"])
+    assert np.abs(np.expm1(z[mask] - ref["snap"][mask])).max() <= 1e-5
